@@ -366,6 +366,7 @@ extern "C" fe_status fe_set_option(fe_mesh* m, int option, int64_t value) {
           value != FE_PRECOND_JACOBI_PLANES_MODES)
         return fe_fail(FE_EINVAL, "fe_set_option: bad Poisson preconditioner");
       m->poisson_precond = (int)value;
+      m->precond_set = true;
       return FE_OK;
     case FE_OPT_POISSON_ARITH:
       if (value != FE_POISSON_F64 && value != FE_POISSON_MIXED)

@@ -313,3 +313,48 @@ def test_mode_coarse_space(fe, p, ncell, L):
     else:
         assert out[("cef", True)] == out[("cef", False)], out
     assert out[("lcpd", True)] == out[("lcpd", False)], out
+
+
+# n_phi >= 4096 everywhere: chains of 1 to 16 cells, plane sizes off every tile edge, odd planes
+@pytest.mark.parametrize("p,ncell", [(1, (16, 16, 16)), (2, (8, 9, 8)), (3, (5, 6, 6)), (4, (1, 8, 8)),
+                                     (5, (3, 4, 4)), (6, (3, 3, 3))])
+@pytest.mark.parametrize("kind", ["cef", "cpd", "cpd_inside", "lcpd", "lcpd_no_lower_plane"])
+def test_separable_preconditioner(fe, kind, p, ncell):
+    """The default solve (the separable preconditioner in a double CG) reaches the oracle's
+    direct solution, in at most five iterations where whole planes are constrained; a
+    constraint set without a separable form (a patch and no constrained plane) still solves,
+    and so does a second constraint set on the same mesh.  Bound: the 1e-12 relative residual
+    times a condition number below 1e3 relative to the largest value."""
+    L = (2.0 * ncell[0] + 1.0, 2.0 * ncell[1] + 1.0, 2.0 * ncell[2] + 6.0)
+    Lz = L[2]
+    bias = {"cef": W.Bias("cef", field=0.01),
+            "cpd": W.Bias("cpd", dV=0.05, zA=0.0, zB=Lz),
+            "cpd_inside": W.Bias("cpd", dV=0.05, zA=0.23 * Lz, zB=0.81 * Lz),
+            "lcpd": W.Bias("cpd", dV=0.05, zA=0.15 * Lz, zB=0.85 * Lz,
+                           patch=((0.1 * L[0], 0.2 * L[1]), (0.6 * L[0], 0.7 * L[1]))),
+            "lcpd_no_lower_plane": W.Bias("cpd", dV=0.05, zA=-1.0, zB=0.8 * Lz,
+                                          patch=((0.0, 0.2 * L[1]), (0.7 * L[0], 0.9 * L[1])))}[kind]
+    base = W.small_slab(ncell=ncell, p=p, L=L, natoms=3, seed=41)
+    slab = W.Slab(base.name, base.L, base.ncell, base.p, base.R, base.Z, bias)
+    assert slab.n_phi >= 4096
+    om, K, M, X = _oracle(slab)
+    rho, b = potentials.densities(X, M, slab.R, slab.Z, slab.L)
+    vl = potentials.vloc_minus_vsm(X, slab.R, slab.Z, slab.L)
+    f = 4 * math.pi * M * (rho + b)
+    if kind == "cef":
+        ref = poisson.solve_cef_direct(K, f, M)
+    else:
+        mask, vals, _, _ = potentials.cpd_constraints(X, vl, bias, slab.L)
+        ref = poisson.solve_cpd_direct(K, f, mask, vals)
+    m = fe.Mesh.from_slab(slab)
+    m.poisson_solve(W.Bias("cpd", dV=0.1, zA=0.4 * Lz, zB=0.6 * Lz), rtol=1e-8)
+    phi, _, info = m.poisson_solve(bias, rtol=1e-12)
+    assert info.status == 0 and info.rel_residual <= 1e-12
+    assert np.max(np.abs(phi.cpu().numpy() - ref)) <= 1e-9 * np.max(np.abs(ref))
+    if kind in ("cef", "cpd", "cpd_inside"):
+        assert info.iters <= 5, info.iters
+    elif kind == "lcpd":
+        assert info.iters <= 60, info.iters
+    with pytest.raises(fe.FeError) as e:
+        m.poisson_solve(bias, rtol=1e-12, max_iter=1)
+    assert e.value.status == fe._lib.FE_ENOCONV
