@@ -94,19 +94,19 @@ void fill_io(const fe_batch* b, KronInst<T>* inst, const void* const* X, void* c
              const double* alpha, const double* beta, const double* shift) {
   for (size_t i = 0; i < b->meshes.size(); ++i) {
     const fe_mesh* m = b->meshes[i];
-    KronIO<T>& io = inst[i].io;
+    SweepIO<T>& io = inst[i].io;
     io.X = (const T*)X[i];
-    io.ldx = ld[i];
     io.Y = (T*)Y[i];
-    io.ldy = ld[i];
-    io.Z = (Z && beta[i] != 0.0) ? (const T*)Z[i] : nullptr;
-    io.ldz = ld[i];
-    if constexpr (sizeof(T) == 8) io.V = (const T*)m->d_veff;
-    else io.V = (const T*)m->d_veff_f;
+    io.Z = Z ? (const T*)Z[i] : nullptr;
+    io.ld = ld[i];
     io.nvec = nvec[i];
-    io.alpha = (T)alpha[i];
-    io.beta = (T)beta[i];
-    io.shift = (T)shift[i];
+    if constexpr (sizeof(T) == 8) {
+      io.V = (const T*)m->d_veff;
+      fe::sweep_scalars_f64(m->coefH, m->p, alpha[i], beta[i], shift[i], &io);
+    } else {
+      io.V = (const T*)m->d_veff_f;
+      fe::sweep_scalars_f32(m->coefH, m->p, alpha[i], beta[i], shift[i], &io);
+    }
   }
 }
 
@@ -114,8 +114,8 @@ template <typename T>
 int64_t plan_with(const fe_batch* b, KronInst<T>* inst, int zseg) {
   const int n = (int)b->meshes.size();
   for (int i = 0; i < n; ++i) inst[i].g = fe_geom(b->meshes[i], true);
-  if constexpr (sizeof(T) == 8) return fe::kron_batch_plan_f64(b->p, inst, n, zseg);
-  else return fe::kron_batch_plan_f32(b->p, inst, n, zseg);
+  if constexpr (sizeof(T) == 8) return fe::sweep_batch_plan_f64(b->p, inst, n, zseg);
+  else return fe::sweep_batch_plan_f32(b->p, inst, n, zseg);
 }
 
 template <typename T>
@@ -134,7 +134,7 @@ fe_status ensure_counter(fe_batch* b) {
 }
 
 template <typename T>
-fe_status launch_with(fe_batch* b, const KronInst<T>* d_inst, int64_t total, bool use_z,
+fe_status launch_with(fe_batch* b, const KronInst<T>* d_inst, int64_t total, int64_t widest,
                       bool full, int persistent) {
   const int n = (int)b->meshes.size();
   unsigned long long* counter = nullptr;
@@ -143,16 +143,15 @@ fe_status launch_with(fe_batch* b, const KronInst<T>* d_inst, int64_t total, boo
     counter = b->d_counter;
   }
   if constexpr (sizeof(T) == 8)
-    return fe::kron_batch_f64(b->meshes[0]->coefH, b->p, d_inst, n, total, use_z, full, b->stream,
-                              counter);
+    return fe::sweep_batch_f64(b->meshes[0]->coefH, b->p, widest, full, d_inst, n, total, b->stream, counter);
   else
-    return fe::kron_batch_f32(b->meshes[0]->coefH, b->p, d_inst, n, total, use_z, full, b->stream,
-                              counter);
+    return fe::sweep_batch_f32(b->meshes[0]->coefH, b->p, widest, full, d_inst, n, total, b->stream, counter);
 }
 
 template <typename T>
-fe_status launch(fe_batch* b, const KronInst<T>* d_inst, int64_t total, bool use_z, bool full) {
-  return launch_with(b, d_inst, total, use_z, full, b->persistent);
+fe_status launch(fe_batch* b, const KronInst<T>* d_inst, int64_t total, int64_t widest,
+                 bool full) {
+  return launch_with(b, d_inst, total, widest, full, b->persistent);
 }
 
 template <typename T>
@@ -201,6 +200,7 @@ fe_status tune(fe_batch* b, const void* const* X, void* const* W, const int64_t*
   cudaEvent_t e0, e1;
   FE_CUDA(cudaEventCreate(&e0));
   FE_CUDA(cudaEventCreate(&e1));
+  const int64_t widest = *std::max_element(nvec, nvec + n);
   double best = 1e300;
   int best_z = 0, best_p = 0, tried = 0;
   std::vector<int> resolved;
@@ -223,10 +223,10 @@ fe_status tune(fe_batch* b, const void* const* X, void* const* W, const int64_t*
     const bool full = all_full(inst.data(), n);
     for (int pers = 0; pers <= 1 && st == FE_OK; ++pers) {
       const KronInst<T>* d = (const KronInst<T>*)b->d_desc;
-      st = launch_with(b, d, total, false, full, pers);   // warm-up
+      st = launch_with(b, d, total, widest, full, pers);   // warm-up
       if (st != FE_OK) break;
       cudaEventRecord(e0, b->stream);
-      for (int r = 0; r < 2 && st == FE_OK; ++r) st = launch_with(b, d, total, false, full, pers);
+      for (int r = 0; r < 2 && st == FE_OK; ++r) st = launch_with(b, d, total, widest, full, pers);
       cudaEventRecord(e1, b->stream);
       if (st != FE_OK) break;
       if (cudaEventSynchronize(e1) != cudaSuccess) {
@@ -271,7 +271,8 @@ fe_status batch_apply(fe_batch* b, const void* const* X, void* const* Y, const i
   FE_TRY(grow_desc(b, n * sizeof(KronInst<T>)));
   FE_CUDA(cudaMemcpyAsync(b->d_desc, inst.data(), n * sizeof(KronInst<T>),
                           cudaMemcpyHostToDevice, b->stream));
-  return launch(b, (const KronInst<T>*)b->d_desc, total, false, all_full(inst.data(), n));
+  return launch(b, (const KronInst<T>*)b->d_desc, total, *std::max_element(nvec, nvec + n),
+                all_full(inst.data(), n));
 }
 
 // The recurrence of fe_cheb_filter, per instance, with every step one batched launch.  All
@@ -321,8 +322,9 @@ fe_status batch_filter(fe_batch* b, void* const* X, const int64_t* nvec, const i
   FE_TRY(grow_desc(b, bytes));
   FE_CUDA(cudaMemcpyAsync(b->d_desc, inst.data(), bytes, cudaMemcpyHostToDevice, b->stream));
   const KronInst<T>* d = (const KronInst<T>*)b->d_desc;
+  const int64_t widest = *std::max_element(nvec, nvec + n);
   const bool full = all_full(inst.data(), n);
-  for (int s = 0; s < degree; ++s) FE_TRY(launch(b, d + s * n, total, s > 0, full));
+  for (int s = 0; s < degree; ++s) FE_TRY(launch(b, d + s * n, total, widest, full));
   for (size_t i = 0; i < n; ++i)
     if (cur[i] != X[i])
       FE_CUDA(cudaMemcpy2DAsync(X[i], ld[i] * eb, cur[i], ld[i] * eb, nvec[i] * eb,

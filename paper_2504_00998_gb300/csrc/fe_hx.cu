@@ -43,12 +43,29 @@ fe_status fe_tc_apply(fe_mesh* m, const float* X, float* Y, const float* Z, int6
 fe_status fe_ktc_apply(fe_mesh* m, const float* X, float* Y, const float* Z, int64_t nvec,
                        int64_t ld, float alpha, float beta, float shift);
 
+namespace {
+
+// the sum-factorised operator in double or float; gx, gy: the Bloch term's scales
+fe_status sweep_step(fe_mesh* m, const void* X, void* Y, const void* Z, int64_t nvec, int64_t ld,
+                     double alpha, double beta, double shift, double gx, double gy, bool dbl) {
+  const KronGeom g = fe_geom(m, true);
+  if (dbl) {
+    SweepIO<double> io{(const double*)X, (double*)Y, (const double*)Z, m->d_veff, ld, nvec};
+    fe::sweep_scalars_f64(m->coefH, m->p, alpha, beta, shift, &io);
+    return fe::sweep_f64(m->coefH, gx, gy, g, io, m->stream);
+  }
+  SweepIO<float> io{(const float*)X, (float*)Y, (const float*)Z, m->d_veff_f, ld, nvec};
+  fe::sweep_scalars_f32(m->coefH, m->p, alpha, beta, shift, &io);
+  return fe::sweep_f32(m->coefH, gx, gy, g, io, m->stream);
+}
+
+}  // namespace
+
 // Y = alpha (Ht - shift) X + beta Z in the requested arithmetic.
 // (plus alpha Ht_nloc X when the mesh carries the nonlocal term)
 // With a Bloch wave vector (Section 2.1, H^k_loc), Ht_k = Ht_0 + |k|^2 / 2 - i A on complex
-// blocks stored as interleaved (re, im) lanes; nvec and ld count real lanes here.  The first
-// launch applies Ht_0 + |k|^2 / 2 to every lane with the Chebyshev combination, the second
-// accumulates alpha (-i A X) into Y (A = M^-1/2 (kx Gx + ky Gy) M^-1/2, real antisymmetric).
+// blocks stored as interleaved (re, im) lanes; nvec and ld count real lanes here
+// (A = M^-1/2 (kx Gx + ky Gy) M^-1/2, real antisymmetric).
 fe_status fe_hx_step(fe_mesh* m, const void* X, void* Y, const void* Z, int64_t nvec, int64_t ld,
                      double alpha, double beta, double shift, fe_precision prec) {
   if (m->has_k) {
@@ -57,33 +74,13 @@ fe_status fe_hx_step(fe_mesh* m, const void* X, void* Y, const void* Z, int64_t 
     if (m->nl.natoms > 0)
       return fe_fail(FE_EUNSUPPORTED, "Bloch operator: the nonlocal term is Gamma-point only");
     const double sh = shift - 0.5 * (m->kx * m->kx + m->ky * m->ky);
-    const KronGeom g = fe_geom(m, true);
-    if (prec == FE_F64) {
-      KronIO<double> io{(const double*)X, ld, (double*)Y, ld, (const double*)Z, ld, m->d_veff,
-                        nvec, alpha, beta, sh};
-      FE_TRY(fe::kron_f64(m->coefH, g, io, m->stream));
-      KronIO<double> ia{(const double*)X, ld, (double*)Y, ld, (const double*)Y, ld, nullptr,
-                        nvec, alpha, 1.0, 0.0};
-      FE_TRY(fe::kron_f64(m->coefA, g, ia, m->stream));
-    } else {
-      KronIO<float> io{(const float*)X, ld, (float*)Y, ld, (const float*)Z, ld, m->d_veff_f,
-                       nvec, (float)alpha, (float)beta, (float)sh};
-      FE_TRY(fe::kron_f32(m->coefH, g, io, m->stream));
-      KronIO<float> ia{(const float*)X, ld, (float*)Y, ld, (const float*)Y, ld, nullptr, nvec,
-                       (float)alpha, 1.0f, 0.0f};
-      FE_TRY(fe::kron_f32(m->coefA, g, ia, m->stream));
-    }
+    const double gx = m->kx * m->h[1] * m->h[2] / 4.0, gy = m->ky * m->h[0] * m->h[2] / 4.0;
+    FE_TRY(sweep_step(m, X, Y, Z, nvec, ld, alpha, beta, sh, gx, gy, prec == FE_F64));
     // the real symmetric quadrature potential acts on the (re, im) lanes alike
     return fe_quad_apply(m, X, Y, nvec, ld, alpha, prec == FE_F64);
   }
-  if (prec == FE_F64) {
-    KronIO<double> io{(const double*)X, ld, (double*)Y, ld, (const double*)Z, ld, m->d_veff,
-                      nvec, alpha, beta, shift};
-    FE_TRY(fe::kron_f64(m->coefH, fe_geom(m, true), io, m->stream));
-  } else if (prec == FE_F32) {
-    KronIO<float> io{(const float*)X, ld, (float*)Y, ld, (const float*)Z, ld, m->d_veff_f,
-                     nvec, (float)alpha, (float)beta, (float)shift};
-    FE_TRY(fe::kron_f32(m->coefH, fe_geom(m, true), io, m->stream));
+  if (prec == FE_F64 || prec == FE_F32) {
+    FE_TRY(sweep_step(m, X, Y, Z, nvec, ld, alpha, beta, shift, 0.0, 0.0, prec == FE_F64));
   } else if (prec == FE_F32_F32ACC) {
     FE_TRY(fe_ktc_apply(m, (const float*)X, (float*)Y, (const float*)Z, nvec, ld, (float)alpha,
                         (float)beta, (float)shift));

@@ -125,10 +125,8 @@ struct KronCoef {
   double wz[FE_MAXN1];    // GLL weights (for the z mass factor of a plane)
   double zin;             // J^-1/2 (or 1 for the Poisson operator)
   double zout;            // 1/2 J^-1/2 (or 1)
-  double ax, ay;          // the in-plane stiffness scales hy hz / (2 hx), hx hz / (2 hy)
+  double ax, ay, az;      // the stiffness scales hy hz / (2 hx), hx hz / (2 hy), hx hy / (2 hz)
   int mass_scale;         // 1: Hamiltonian (mass-scaled), 0: plain K
-  int cplx;               // 1: the Bloch first-derivative operator A; the launch writes -i A X
-                          //    on interleaved (re, im) lanes
 };
 
 struct KronGeom {
@@ -148,41 +146,59 @@ struct KronIO {
   T alpha, beta, shift;      // Y = alpha (H - shift) X + beta Z
 };
 
+// Arguments of a sweep launch: Y = alpha (Ht - shift) X + beta Z with the scalars in the form
+// the kernel uses (fe::sweep_scalars), one leading dimension for the three blocks.
+template <typename T>
+struct SweepIO {
+  const T* X;
+  T* Y;
+  const T* Z;                // nullptr: no Z term
+  const T* V;
+  int64_t ld, nvec;
+  T al, zs, vs, shift, v0;   // Y = al (K/cz X + (vs (V - shift) + v0) X + zs Z)
+};
+
 // One instance of a batched operator launch (device-resident array, ascending cta0).
 template <typename T>
 struct KronInst {
   KronGeom g;
-  KronIO<T> io;
+  SweepIO<T> io;
   int64_t cta0;              // first CTA of this instance in the batched 1D grid
   int64_t nvt;               // vector tiles of this instance
   int full;                  // complete xy blocks and vector tiles (set by the plan)
 };
 
 
-// operator launchers: double with 16-byte chunks, float with 16-byte chunks, and double
-// with one element per node (single-vector Poisson operator)
-// (the tile fields of g are chosen by the launcher)
+// Operator launchers.  sweep_f32 / sweep_f64: the mass-scaled Hamiltonian (fe_sweep.cuh) on
+// blocks of vectors; bgx, bgy != 0 (kx hy hz / 4, ky hx hz / 4) add the Bloch term -i A on
+// interleaved (re, im) lanes.  kron_k1: the plain stiffness on one double
+// vector (fe_kron.cuh).
 namespace fe {
-fe_status kron_f64(const KronCoef& cf, const KronGeom& g, const KronIO<double>& io,
-                   cudaStream_t st);
-fe_status kron_f32(const KronCoef& cf, const KronGeom& g, const KronIO<float>& io,
-                   cudaStream_t st);
+fe_status sweep_f64(const KronCoef& cf, double bgx, double bgy, const KronGeom& g,
+                    const SweepIO<double>& io, cudaStream_t st);
+fe_status sweep_f32(const KronCoef& cf, double bgx, double bgy, const KronGeom& g,
+                    const SweepIO<float>& io, cudaStream_t st);
+// the scalars of io for alpha, beta and shift (al, zs, vs, shift, v0; Z is dropped for beta = 0)
+void sweep_scalars_f64(const KronCoef& cf, int p, double alpha, double beta, double shift,
+                       SweepIO<double>* io);
+void sweep_scalars_f32(const KronCoef& cf, int p, double alpha, double beta, double shift,
+                       SweepIO<float>* io);
 fe_status kron_k1(const KronCoef& cf, const KronGeom& g, const KronIO<double>& io,
                   cudaStream_t st);
 // Batched launches: plan fills the tile fields, z segmentation, nvt and cta0 of n host
 // instances (g from fe_geom, io.nvec set) and returns the total CTA count; launch runs one
-// operator application over the device copy of those instances.
+// operator application over the device copy of those instances (widest: their largest nvec).
 // zseg_req > 0 asks for that z-segment length (cells per CTA along z); counter != nullptr
 // launches the persistent, dynamically scheduled form (counter: one device word, reset by
 // the launch).
-int64_t kron_batch_plan_f64(int p, KronInst<double>* inst, int n, int zseg_req);
-int64_t kron_batch_plan_f32(int p, KronInst<float>* inst, int n, int zseg_req);
-fe_status kron_batch_f64(const KronCoef& cf, int p, const KronInst<double>* d_inst, int n,
-                         int64_t total_ctas, bool use_z, bool full, cudaStream_t st,
-                         unsigned long long* counter);
-fe_status kron_batch_f32(const KronCoef& cf, int p, const KronInst<float>* d_inst, int n,
-                         int64_t total_ctas, bool use_z, bool full, cudaStream_t st,
-                         unsigned long long* counter);
+int64_t sweep_batch_plan_f64(int p, KronInst<double>* inst, int n, int zseg_req);
+int64_t sweep_batch_plan_f32(int p, KronInst<float>* inst, int n, int zseg_req);
+fe_status sweep_batch_f64(const KronCoef& cf, int p, int64_t widest, bool full,
+                          const KronInst<double>* d_inst, int n, int64_t total_ctas, cudaStream_t st,
+                          unsigned long long* counter);
+fe_status sweep_batch_f32(const KronCoef& cf, int p, int64_t widest, bool full,
+                          const KronInst<float>* d_inst, int n, int64_t total_ctas, cudaStream_t st,
+                          unsigned long long* counter);
 }  // namespace fe
 
 // ---- nonlocal projector tables (fe_nonlocal.cu) --------------------------------------------
@@ -210,7 +226,6 @@ struct fe_mesh {
   double h[3], J;
   double xi[FE_MAXN1], w[FE_MAXN1];
   double K1[FE_MAXN1][FE_MAXN1], M1[FE_MAXN1][FE_MAXN1];
-  double G1[FE_MAXN1][FE_MAXN1];   // int l_i l_j' on the reference interval
   cudaStream_t stream;
   int device;
   cudaStream_t aux_stream = nullptr;   // library-owned, non-blocking: graph capture
@@ -218,10 +233,8 @@ struct fe_mesh {
 
   KronCoef coefH;          // Hamiltonian (mass-scaled, 1/2 factor)
   KronCoef coefK;          // plain stiffness
-  // Bloch wave vector (x, y) and the antisymmetric operator M^-1/2 (kx Gx + ky Gy) M^-1/2
-  double kx = 0.0, ky = 0.0;
+  double kx = 0.0, ky = 0.0;   // Bloch wave vector
   bool has_k = false;
-  KronCoef coefA;
 
   double* d_veff = nullptr;   // [n_psi]
   float* d_veff_f = nullptr;  // [n_psi]

@@ -1,5 +1,6 @@
-// Matrix-free application of the finite-element operators of Section 2.3 on the uniform
-// tensor-product slab mesh.
+// Matrix-free application of the finite-element stiffness of Section 2.3 on the uniform
+// tensor-product slab mesh, without scratch memory (the double product of one vector where the
+// cell-by-cell form's scratch cannot be had; blocks of vectors run in fe_sweep.cuh).
 //
 // For a uniform hexahedral mesh the assembled stiffness K_IJ = int grad N_I . grad N_J is a
 // sum of Kronecker products of the exactly integrated 1D element matrices,
@@ -7,9 +8,7 @@
 // (ax = hy hz / (2 hx), ...) and the GLL-lumped overlap is M = J mx (x) my (x) mz.  The
 // kernel evaluates, output-stationary,
 //   Y = alpha * ( oscale * K (S X) + (V - shift) X ) + beta * Z
-// which is the Hamiltonian Ht = 1/2 M^-1/2 K M^-1/2 + V (Eq. Veff and Hloc) with the
-// three-term Chebyshev update fused (S = M^-1/2, oscale = 1/2 M^-1/2), or the Poisson
-// operator K (S = I, oscale = 1, no potential).
+// with S = 1 and oscale = 1 for the Poisson operator (no potential), or the mass-scaled form.
 //
 // Work decomposition: one CTA owns the nodes of an xy block of BX x BY cells (half-open),
 // a tile of NCH vector chunks, and a range of z layers.  It sweeps the z planes in order.
@@ -31,7 +30,6 @@
 #include <cmath>
 #include <type_traits>
 
-#include "fe_gll_tables.h"
 #include "fe_internal.h"
 
 namespace fe {
@@ -57,9 +55,7 @@ struct KronCoefT {
   T rsq[FE_MAXN1], sq[FE_MAXN1];
   T rsq_face, sq_face, face_fix;
   T zout, izout;
-  T ax, ay;   // in-plane stiffness scales (used with the compile-time shape tables)
   int mass_scale;
-  int cplx;   // write -i (operator X) on interleaved (re, im) lanes
 };
 
 template <typename T>
@@ -93,10 +89,7 @@ inline KronCoefT<T> convert_coef(const KronCoef& c) {
   o.face_fix = c.mass_scale ? (T)std::sqrt(2.0) : T(1);
   o.zout = (T)c.zout;
   o.izout = (T)(1.0 / c.zout);
-  o.ax = (T)c.ax;
-  o.ay = (T)c.ay;
   o.mass_scale = c.mass_scale;
-  o.cplx = c.cplx;
   return o;
 }
 
@@ -119,34 +112,9 @@ struct alignas(sizeof(T) * CH) Chunk {
 };
 
 template <>
-__device__ __forceinline__ float Chunk<float, 4>::fma_t(float a, float b, float c) {
-  return __fmaf_rn(a, b, c);
-}
-// d0,d1 += c * (b0,b1): one paired FP32 FMA (the same correctly rounded fma in each lane)
-__device__ __forceinline__ void ffma2(float& d0, float& d1, float c, float b0, float b1) {
-  asm("{\n\t.reg .b64 ra, rb, rd;\n\tmov.b64 ra, {%2, %2};\n\tmov.b64 rb, {%3, %4};\n\t"
-      "mov.b64 rd, {%0, %1};\n\tfma.rn.f32x2 rd, ra, rb, rd;\n\tmov.b64 {%0, %1}, rd;\n\t}"
-      : "+f"(d0), "+f"(d1) : "f"(c), "f"(b0), "f"(b1));
-}
-// float chunks accumulate two lanes per instruction
-template <>
-__device__ __forceinline__ void Chunk<float, 4>::fma(float a, const Chunk& x) {
-  ffma2(v[0], v[1], a, x.v[0], x.v[1]);
-  ffma2(v[2], v[3], a, x.v[2], x.v[3]);
-}
-template <>
-__device__ __forceinline__ double Chunk<double, 2>::fma_t(double a, double b, double c) {
-  return __fma_rn(a, b, c);
-}
-template <>
 __device__ __forceinline__ double Chunk<double, 1>::fma_t(double a, double b, double c) {
   return __fma_rn(a, b, c);
 }
-template <>
-__device__ __forceinline__ float Chunk<float, 1>::fma_t(float a, float b, float c) {
-  return __fmaf_rn(a, b, c);
-}
-
 template <int BYTES>
 __device__ __forceinline__ void cp_async(void* smem, const void* gmem, int nbytes_valid) {
   unsigned s = (unsigned)__cvta_generic_to_shared(smem);
@@ -197,10 +165,7 @@ struct KronTileT {
 // One CTA's work: xy block bxy (x fastest), vector tile vti, z segment zsi.
 // FULL: every xy block is complete and every vector tile full, so no ownership, edge or
 // ragged-vector test is needed anywhere in the sweep.
-// CT (float Hamiltonian): the in-plane contractions take the shape-only tables M1 sig and
-// K1 sig as compile-time constants (FFMA immediates instead of constant-bank loads) and apply
-// the mesh scales ay, ax as one multiply per y output and one FMA per x output.
-template <typename T, int CH, class TL, bool FULL, bool CT>
+template <typename T, int CH, class TL, bool FULL>
 __device__ __forceinline__ void kron_body(const KronCoefT<T>& cf, const KronGeom& g,
                                           const KronIO<T>& io, int bxy, int vti, int zsi) {
   using C = Chunk<T, CH>;
@@ -216,8 +181,7 @@ __device__ __forceinline__ void kron_body(const KronCoefT<T>& cf, const KronGeom
   C* W1 = B + BYn * ARS * NCH;                                 // [BYn][WRS][NCH]
   C* W2 = W1 + BYn * WRS * NCH;
   C* Zr = W2 + BYn * WRS * NCH;                                // [ZR][BYn][BXn][NCH]
-  // the shape-table variants are launched for the mass-scaled Hamiltonian only
-  const bool mass_scale = CT || cf.mass_scale;
+  const bool mass_scale = cf.mass_scale;
   const bool use_z = io.Z != nullptr;                          // (beta != 0 by launch)
   const bool use_v = io.V != nullptr;
   T* Vs = reinterpret_cast<T*>(Zr + (use_z ? TL::ZR * NZI : 0));   // [NSB][BYn][BXn]
@@ -376,19 +340,8 @@ __device__ __forceinline__ void kron_body(const KronCoefT<T>& cf, const KronGeom
       const int64_t v0 = vt0 + (int64_t)it_ch[i] * CH;
       const T sc = io.alpha * ps * it_sxy[i];
       C out;
-      // (the shape-table variants are launched for the real operator only)
-      if (!CT && cf.cplx) {
-        // -i (a + i b) = b - i a on each (re, im) lane pair (even chunk widths only)
-        out.zero();
 #pragma unroll
-        for (int e = 0; e + 1 < CH; e += 2) {
-          out.v[e] = sc * acc[i][j].v[e + 1];
-          out.v[e + 1] = -sc * acc[i][j].v[e];
-        }
-      } else {
-#pragma unroll
-        for (int e = 0; e < CH; ++e) out.v[e] = sc * acc[i][j].v[e];
-      }
+      for (int e = 0; e < CH; ++e) out.v[e] = sc * acc[i][j].v[e];
       if (use_z) {
         const C zc = zsrc[tid + i * NTHR];
 #pragma unroll
@@ -455,19 +408,11 @@ __device__ __forceinline__ void kron_body(const KronCoefT<T>& cf, const KronGeom
     }
   };
 
-  // in-plane 1D coefficients: the mesh's tables, or (CT) the compile-time shape tables
-  auto cYM = [&](int j, int k) -> T {
-    if constexpr (CT) return (T)gll_ms<P>(j, k); else return cf.AyM[j][k];
-  };
-  auto cYK = [&](int j, int k) -> T {
-    if constexpr (CT) return (T)gll_ks<P>(j, k); else return cf.AyK[j][k];
-  };
-  auto cXM = [&](int j, int k) -> T {
-    if constexpr (CT) return (T)gll_ms<P>(j, k); else return cf.AxM[j][k];
-  };
-  auto cXK = [&](int j, int k) -> T {
-    if constexpr (CT) return (T)gll_ks<P>(j, k); else return cf.AxK[j][k];
-  };
+  // in-plane 1D coefficients
+  auto cYM = [&](int j, int k) -> T { return cf.AyM[j][k]; };
+  auto cYK = [&](int j, int k) -> T { return cf.AyK[j][k]; };
+  auto cXM = [&](int j, int k) -> T { return cf.AxM[j][k]; };
+  auto cXK = [&](int j, int k) -> T { return cf.AxK[j][k]; };
 
   // scalar-lane items of the in-plane phases (used when each thread has at most one)
   constexpr int NL = NCH * CH;
@@ -534,7 +479,6 @@ __device__ __forceinline__ void kron_body(const KronCoefT<T>& cf, const KronGeom
             a.fma(cYM(P, P), own[0]);
             b.fma(cYK(P, P), own[0]);
           }
-          if constexpr (CT) b.v[0] *= cf.ay;
           As[obase + j * ARS * NL] = a;
           Bs[obase + j * ARS * NL] = b;
         }
@@ -566,15 +510,13 @@ __device__ __forceinline__ void kron_body(const KronCoefT<T>& cf, const KronGeom
           }
 #pragma unroll
           for (int j = 0; j < P; ++j) {
-            S1 u, v, vk;   // (CT: v gathers M1 sig b, vk gathers K1 sig a, scaled by ax)
+            S1 u, v;
             u.zero();
             v.zero();
-            vk.zero();
-            S1& vka = CT ? vk : v;
 #pragma unroll
             for (int kk = 0; kk <= P; ++kk) {
               u.fma(cXM(j, kk), ao[kk]);
-              vka.fma(cXK(j, kk), ao[kk]);
+              v.fma(cXK(j, kk), ao[kk]);
               v.fma(cXM(j, kk), bo[kk]);
             }
             if (j == 0) {
@@ -583,14 +525,13 @@ __device__ __forceinline__ void kron_body(const KronCoefT<T>& cf, const KronGeom
                 const S1 ap = arow[kk * NL];
                 const S1 bp = brow[kk * NL];
                 u.fma(cXM(P, kk), ap);
-                vka.fma(cXK(P, kk), ap);
+                v.fma(cXK(P, kk), ap);
                 v.fma(cXM(P, kk), bp);
               }
               u.fma(cXM(P, P), ao[0]);
-              vka.fma(cXK(P, P), ao[0]);
+              v.fma(cXK(P, P), ao[0]);
               v.fma(cXM(P, P), bo[0]);
             }
-            if constexpr (CT) v.fma(cf.ax, vk);
             W1s[obase + j * NL] = u;
             W2s[obase + j * NL] = v;
           }
@@ -650,77 +591,13 @@ __device__ __forceinline__ void kron_body(const KronCoefT<T>& cf, const KronGeom
 // 1D grid, vector tile fastest: the CTAs that read the other halves of a node's DRAM
 // bursts (neighbouring vector tiles of the same xy block) run side by side, so a burst is
 // fetched once; neighbouring xy blocks (halo sharing) follow within the resident window.
-// the float block operator (four-lane chunks) takes the compile-time shape tables
-template <typename T, int CH>
-struct KronShapeTables {
-  static constexpr bool value = std::is_same<T, float>::value && CH == 4;
-};
-
-// Residency bound: the float operator's tiles of up to 256 threads are held to three CTAs per
-// SM (at most 85 registers), where the per-plane barriers of one CTA overlap two others' work.
-template <typename T, int CH, class TL>
-struct KronMinBlocks {
-  static constexpr int value = (std::is_same<T, float>::value && CH == 4 && TL::NTHR <= 256) ? 3 : 1;
-};
-
-template <typename T, int CH, class TL, bool FULL, bool CT>
-__global__ void __launch_bounds__(TL::NTHR, (KronMinBlocks<T, CH, TL>::value))
+template <typename T, int CH, class TL, bool FULL>
+__global__ void __launch_bounds__(TL::NTHR)
 kron_kernel(const KronCoefT<T> cf, const KronGeom g, const KronIO<T> io, int nvt) {
   const int b = blockIdx.x;
   const int nxy = g.nbx * g.nby;
   const int r = b / nvt;
-  kron_body<T, CH, TL, FULL, CT>(cf, g, io, r % nxy, b % nvt, r / nxy);
-}
-
-// Batched form: many independent meshes that share p and the cell size (so one coefficient
-// table) in one launch.  The 1D grid concatenates the instances' CTA grids; a CTA finds its
-// instance by binary search over the ascending first-CTA offsets.
-template <typename T, int CH, class TL, bool FULL, bool CT>
-__global__ void __launch_bounds__(TL::NTHR, (KronMinBlocks<T, CH, TL>::value))
-kron_batch_kernel(const KronCoefT<T> cf, const KronInst<T>* __restrict__ inst, int ninst) {
-  const int64_t b = blockIdx.x;
-  int lo = 0, hi = ninst - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (inst[mid].cta0 <= b) lo = mid; else hi = mid - 1;
-  }
-  const KronGeom g = inst[lo].g;
-  const KronIO<T> io = inst[lo].io;
-  const int64_t local = b - inst[lo].cta0;
-  const int nxy = g.nbx * g.nby;
-  const int64_t nvt = inst[lo].nvt;
-  const int64_t r = local / nvt;
-  kron_body<T, CH, TL, FULL, CT>(cf, g, io, (int)(r % nxy), (int)(local % nvt), (int)(r / nxy));
-}
-
-// Persistent batched form: a grid of resident CTAs takes the batch's work items (the CTAs of
-// the one-CTA-per-item grid above) from a device counter, so that the items of tall and
-// short instances spread over the SMs as they finish (dynamic load balance for uneven slab
-// heights).  The counter starts at zero for each launch.
-template <typename T, int CH, class TL, bool FULL, bool CT>
-__global__ void __launch_bounds__(TL::NTHR, (KronMinBlocks<T, CH, TL>::value))
-kron_batch_persist_kernel(const KronCoefT<T> cf, const KronInst<T>* __restrict__ inst, int ninst,
-                          int64_t total, unsigned long long* __restrict__ counter) {
-  __shared__ long long s_item;
-  for (;;) {
-    __syncthreads();   // every thread is done with the previous item's shared memory
-    if (threadIdx.x == 0) s_item = (long long)atomicAdd(counter, 1ull);
-    __syncthreads();
-    const int64_t b = s_item;
-    if (b >= total) break;
-    int lo = 0, hi = ninst - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (inst[mid].cta0 <= b) lo = mid; else hi = mid - 1;
-    }
-    const KronGeom g = inst[lo].g;
-    const KronIO<T> io = inst[lo].io;
-    const int64_t local = b - inst[lo].cta0;
-    const int nxy = g.nbx * g.nby;
-    const int64_t nvt = inst[lo].nvt;
-    const int64_t r = local / nvt;
-    kron_body<T, CH, TL, FULL, CT>(cf, g, io, (int)(r % nxy), (int)(local % nvt), (int)(r / nxy));
-  }
+  kron_body<T, CH, TL, FULL>(cf, g, io, r % nxy, b % nvt, r / nxy);
 }
 
 // Dynamic shared memory limit, and the largest shared-memory carveout so that the residency
@@ -760,13 +637,7 @@ fe_status kron_launch_t(const KronCoef& cf, const KronGeom& g, const KronIO<T>& 
   if (smem > 227 * 1024) return fe_fail(FE_EINVAL, "tile needs %zu bytes of shared memory", smem);
   const int64_t vtile = (int64_t)TL::NCH * CH;
   const bool full = g.NX % TL::BXn == 0 && g.NY % TL::BYn == 0 && io.nvec % vtile == 0;
-  auto kern = full ? kron_kernel<T, CH, TL, true, false> : kron_kernel<T, CH, TL, false, false>;
-  if constexpr (KronShapeTables<T, CH>::value) {
-    if (cf.mass_scale && !cf.cplx)
-      kern = full ? kron_kernel<T, CH, TL, true, true> : kron_kernel<T, CH, TL, false, true>;
-  }
-  if (cf.cplx && (CH % 2 != 0 || io.nvec % 2 != 0))
-    return fe_fail(FE_EINVAL, "complex operator needs interleaved (re, im) lane pairs");
+  auto kern = full ? kron_kernel<T, CH, TL, true> : kron_kernel<T, CH, TL, false>;
   FE_TRY(kron_func_setup(kern, smem));
   const int64_t nvt = (io.nvec + vtile - 1) / vtile;
   const int64_t total = (int64_t)g.nbx * g.nby * nvt * ((g.nz + g.zseg - 1) / g.zseg);
@@ -825,116 +696,6 @@ fe_status kron_go(const KronCoef& cf, KronGeom g, const KronIO<T>& io, cudaStrea
   while (zseg > 2 && base * ((g.nz + zseg - 1) / zseg) < want) zseg = (zseg + 1) / 2;
   g.zseg = zseg;
   return kron_launch_t<T, CH, TL>(cf, g, io, st);
-}
-
-// batched plan: every instance gets tile TL; z segments are split (uniformly) only while the
-// whole batch has fewer than four CTAs per SM, or have the requested length zseg_req > 0
-template <typename T, int CH, class TL>
-int64_t kron_batch_plan_t(KronInst<T>* inst, int n, int zseg_req) {
-  int nzmax = 1;
-  for (int i = 0; i < n; ++i) {
-    KronGeom& g = inst[i].g;
-    g.bx = TL::BX;
-    g.by = TL::BY;
-    g.nbx = (g.NX / g.p + TL::BX - 1) / TL::BX;
-    g.nby = (g.NY / g.p + TL::BY - 1) / TL::BY;
-    inst[i].nvt = (inst[i].io.nvec + (int64_t)TL::NCH * CH - 1) / ((int64_t)TL::NCH * CH);
-    inst[i].full = g.NX % TL::BXn == 0 && g.NY % TL::BYn == 0 &&
-                   inst[i].io.nvec % ((int64_t)TL::NCH * CH) == 0;
-    nzmax = g.nz > nzmax ? g.nz : nzmax;
-  }
-  const int64_t want = 4 * (int64_t)device_sms();
-  auto total_for = [&](int zseg) {
-    int64_t t = 0;
-    for (int i = 0; i < n; ++i) {
-      const KronGeom& g = inst[i].g;
-      t += (int64_t)g.nbx * g.nby * inst[i].nvt * ((g.nz + zseg - 1) / zseg);
-    }
-    return t;
-  };
-  int zseg = nzmax;
-  if (zseg_req > 0) zseg = zseg_req < nzmax ? zseg_req : nzmax;
-  else
-    while (zseg > 2 && total_for(zseg) < want) zseg = (zseg + 1) / 2;
-  int64_t cta = 0;
-  for (int i = 0; i < n; ++i) {
-    KronGeom& g = inst[i].g;
-    g.zseg = zseg;
-    inst[i].cta0 = cta;
-    cta += (int64_t)g.nbx * g.nby * inst[i].nvt * ((g.nz + zseg - 1) / zseg);
-  }
-  return cta;
-}
-
-template <typename T, int CH, class TL>
-fe_status kron_batch_launch_t(const KronCoef& cf, const KronInst<T>* d_inst, int n,
-                              int64_t total, bool use_z, bool full, cudaStream_t st,
-                              unsigned long long* counter) {
-  const size_t smem = kron_smem<T, CH, TL>(use_z, true);
-  if (smem > 227 * 1024) return fe_fail(FE_EINVAL, "tile needs %zu bytes of shared memory", smem);
-  if (total < 1 || total > 0x7fffffffLL) return fe_fail(FE_EINVAL, "batched grid of %lld CTAs", (long long)total);
-  const bool ct = KronShapeTables<T, CH>::value && cf.mass_scale && !cf.cplx;
-  KronCoefT<T> cft = convert_coef<T>(cf);
-  if (counter) {
-    // persistent grid: as many CTAs as stay resident, each taking items from the counter
-    auto kern = full ? kron_batch_persist_kernel<T, CH, TL, true, false>
-                     : kron_batch_persist_kernel<T, CH, TL, false, false>;
-    if constexpr (KronShapeTables<T, CH>::value) {
-      if (ct) kern = full ? kron_batch_persist_kernel<T, CH, TL, true, true>
-                          : kron_batch_persist_kernel<T, CH, TL, false, true>;
-    }
-    FE_TRY(kron_func_setup(kern, smem));
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, TL::NTHR, smem) != cudaSuccess ||
-        per_sm < 1) {
-      cudaGetLastError();
-      per_sm = 1;
-    }
-    const int64_t grid = std::min<int64_t>(total, (int64_t)per_sm * device_sms());
-    if (cudaMemsetAsync(counter, 0, sizeof(unsigned long long), st) != cudaSuccess) {
-      cudaGetLastError();
-      return fe_fail(FE_ECUDA, "batched kron: counter reset failed");
-    }
-    kern<<<(unsigned)grid, TL::NTHR, smem, st>>>(cft, d_inst, n, total, counter); fe_count_launch();
-  } else {
-    auto kern = full ? kron_batch_kernel<T, CH, TL, true, false> : kron_batch_kernel<T, CH, TL, false, false>;
-    if constexpr (KronShapeTables<T, CH>::value) {
-      if (ct) kern = full ? kron_batch_kernel<T, CH, TL, true, true> : kron_batch_kernel<T, CH, TL, false, true>;
-    }
-    FE_TRY(kron_func_setup(kern, smem));
-    kern<<<(unsigned)total, TL::NTHR, smem, st>>>(cft, d_inst, n); fe_count_launch();
-  }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return fe_fail(FE_ECUDA, "batched kron launch: %s", cudaGetErrorString(e));
-  return FE_OK;
-}
-
-template <typename T, int CH, int NCH>
-int64_t kron_batch_plan_dispatch(int p, KronInst<T>* inst, int n, int zseg_req) {
-  switch (p) {
-    case 1: return kron_batch_plan_t<T, CH, typename KronTileFor<1, NCH, CH>::type>(inst, n, zseg_req);
-    case 2: return kron_batch_plan_t<T, CH, typename KronTileFor<2, NCH, CH>::type>(inst, n, zseg_req);
-    case 3: return kron_batch_plan_t<T, CH, typename KronTileFor<3, NCH, CH>::type>(inst, n, zseg_req);
-    case 4: return kron_batch_plan_t<T, CH, typename KronTileFor<4, NCH, CH>::type>(inst, n, zseg_req);
-    case 5: return kron_batch_plan_t<T, CH, typename KronTileFor<5, NCH, CH>::type>(inst, n, zseg_req);
-    case 6: return kron_batch_plan_t<T, CH, typename KronTileFor<6, NCH, CH>::type>(inst, n, zseg_req);
-    default: return -1;
-  }
-}
-
-template <typename T, int CH, int NCH>
-fe_status kron_batch_dispatch(const KronCoef& cf, int p, const KronInst<T>* d_inst, int n,
-                              int64_t total, bool use_z, bool full, cudaStream_t st,
-                              unsigned long long* counter) {
-  switch (p) {
-#define FE_BCASE(pp)                                                                      \
-  case pp:                                                                                \
-    return kron_batch_launch_t<T, CH, typename KronTileFor<pp, NCH, CH>::type>(cf, d_inst, n, \
-                                                                          total, use_z, full, st, counter);
-    FE_BCASE(1) FE_BCASE(2) FE_BCASE(3) FE_BCASE(4) FE_BCASE(5) FE_BCASE(6)
-#undef FE_BCASE
-    default: return fe_fail(FE_EUNSUPPORTED, "p = %d", p);
-  }
 }
 
 template <typename T, int CH, int NCH>

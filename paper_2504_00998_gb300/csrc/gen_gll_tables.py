@@ -1,13 +1,19 @@
-"""Writes fe_gll_tables.h: the shape-only 1D tables of the float Hamiltonian operator kernel
-and of the float Gauss-quadrature potential kernel.
+"""Writes fe_gll_tables.h: the shape-only 1D tables of the Hamiltonian sweep kernel and of the
+float Gauss-quadrature potential kernel.
 
-For degree p the in-plane contractions of the mass-scaled operator use
-  MS[j][k] = M1[j][k] sig_k,   KS[j][k] = K1[j][k] sig_k,
-with M1, K1 the exactly integrated 1D mass and stiffness matrices of the Lagrange basis on the
-p + 1 Gauss-Lobatto-Legendre nodes of [-1, 1] and sig_k = 1 / sqrt(m_k) (m_k = w_k, or 2 w_0 at
-a node shared by two cells).  They depend on p only; the mesh enters through the scalars
-ax, ay at run time.  GB[q][i] = l_i(g_q) interpolates from the GLL nodes to the p + 1
-Gauss-Legendre points g_q of [-1, 1] (the potential integrated by Gauss quadrature).  The rules are computed the way the library's mesh set-up computes them
+They depend on the degree p only; the mesh enters through scalars at run time.  K1, M1 are the
+exactly integrated 1D stiffness and mass matrices of the Lagrange basis on the p + 1
+Gauss-Lobatto-Legendre nodes of [-1, 1], sig_k = 1 / sqrt(m_k) (m_k = w_k, or 2 w_0 at a node
+shared by two cells).  GB[q][i] = l_i(g_q) interpolates from the GLL nodes to the p + 1
+Gauss-Legendre points g_q of [-1, 1] (the potential integrated by Gauss quadrature).
+
+The sweep kernel (fe_sweep.cuh) takes the symmetrically scaled tables, in double:
+  KH[j][k] = sig_j K1[j][k] sig_k,  GH[j][k] = sig_j G1[j][k] sig_k  (G1 = int l_j l_k'),
+  TH[j] = sqrt(p (p + 1) / (2 (2 p + 1))) sig_j w_j P_p(x_j):
+the exact mass differs from the GLL-lumped one only in the L_p . L_p product (the rule is exact
+to degree 2 p - 1; <L_p, L_p> is 2 / (2 p + 1) exactly and 2 / p by the rule), so
+M1 = diag(w) - g (w P_p)(w P_p)^T with g = (p / 2)^2 (2 / p - 2 / (2 p + 1)).
+NH[j] = 1 / sig_j is the constant function in the scaled variables (KH NH = 0).  The rules are computed the way the library's mesh set-up computes them
 (three-term Legendre recurrence, Newton from the same starting points, (p+1)-point Gauss
 quadrature of the products) and rounded to float.
 
@@ -71,22 +77,24 @@ def lagrange(xn, i, t):
     return v, d
 
 
-def tables(p):
+def hat_tables(p):
     n1 = p + 1
     xi, w = gll_rule(p)
     gq, gw = gauss_rule(n1)
     K1 = [[0.0] * n1 for _ in range(n1)]
-    M1 = [[0.0] * n1 for _ in range(n1)]
+    G1 = [[0.0] * n1 for _ in range(n1)]
     for a in range(n1):
         ld = [lagrange(xi, i, gq[a]) for i in range(n1)]
         for i in range(n1):
             for j in range(n1):
                 K1[i][j] += gw[a] * ld[i][1] * ld[j][1]
-                M1[i][j] += gw[a] * ld[i][0] * ld[j][0]
+                G1[i][j] += gw[a] * ld[i][0] * ld[j][1]
     sig = [1.0 / math.sqrt(2.0 * w[0] if k in (0, p) else w[k]) for k in range(n1)]
-    MS = [[M1[j][k] * sig[k] for k in range(n1)] for j in range(n1)]
-    KS = [[K1[j][k] * sig[k] for k in range(n1)] for j in range(n1)]
-    return MS, KS
+    KH = [[sig[j] * K1[j][k] * sig[k] for k in range(n1)] for j in range(n1)]
+    GH = [[sig[j] * G1[j][k] * sig[k] for k in range(n1)] for j in range(n1)]
+    c = math.sqrt(p * (p + 1.0) / (2.0 * (2.0 * p + 1.0)))
+    TH = [c * sig[j] * w[j] * legendre(p, xi[j])[0] for j in range(n1)]
+    return KH, GH, TH, [1.0 / v for v in sig]
 
 
 def gauss_interp(p):
@@ -105,36 +113,24 @@ def emit(name, A):
     return f"__device__ constexpr float {name}[{len(A)}][{len(A)}] = {{\n    {rows}}};\n"
 
 
+def emit_double(name, A):
+    rows = ",\n    ".join("{" + ", ".join(repr(v) for v in r) + "}" for r in A)
+    return f"__device__ constexpr double {name}[{len(A)}][{len(A[0])}] = {{\n    {rows}}};\n"
+
+
 def main():
-    out = ["// Generated by gen_gll_tables.py (do not edit): shape-only 1D tables M1 sig and K1 sig",
-           "// of the float Hamiltonian operator and the GLL-to-Gauss interpolation GB for",
-           "// p = 1..6 (see the script for their definition).",
+    out = ["// Generated by gen_gll_tables.py (do not edit): the GLL-to-Gauss interpolation GB and the",
+           "// tables KH, GH, TH, NH of the sweep kernel for p = 1..6 (see the script for their",
+           "// definition).",
            "#pragma once", "", "namespace fe {", ""]
     for p in range(1, 7):
-        MS, KS = tables(p)
-        out.append(emit(f"kGllMS{p}", MS))
-        out.append(emit(f"kGllKS{p}", KS))
         out.append(emit(f"kGaussB{p}", gauss_interp(p)))
-    out.append("""// MS[j][k] and KS[j][k] of degree P (compile-time indices fold to immediates)
-template <int P>
-__device__ __forceinline__ constexpr float gll_ms(int j, int k) {
-  if constexpr (P == 1) return kGllMS1[j][k];
-  else if constexpr (P == 2) return kGllMS2[j][k];
-  else if constexpr (P == 3) return kGllMS3[j][k];
-  else if constexpr (P == 4) return kGllMS4[j][k];
-  else if constexpr (P == 5) return kGllMS5[j][k];
-  else return kGllMS6[j][k];
-}
-template <int P>
-__device__ __forceinline__ constexpr float gll_ks(int j, int k) {
-  if constexpr (P == 1) return kGllKS1[j][k];
-  else if constexpr (P == 2) return kGllKS2[j][k];
-  else if constexpr (P == 3) return kGllKS3[j][k];
-  else if constexpr (P == 4) return kGllKS4[j][k];
-  else if constexpr (P == 5) return kGllKS5[j][k];
-  else return kGllKS6[j][k];
-}
-// GB[q][i] of degree P
+        KH, GH, TH, NH = hat_tables(p)
+        out.append(emit_double(f"kHatK{p}", KH))
+        out.append(emit_double(f"kHatG{p}", GH))
+        out.append(emit_double(f"kHatT{p}", [TH]))
+        out.append(emit_double(f"kHatN{p}", [NH]))
+    out.append("""// GB[q][i] of degree P
 template <int P>
 __device__ __forceinline__ constexpr float gauss_b(int q, int i) {
   if constexpr (P == 1) return kGaussB1[q][i];
@@ -143,6 +139,43 @@ __device__ __forceinline__ constexpr float gauss_b(int q, int i) {
   else if constexpr (P == 4) return kGaussB4[q][i];
   else if constexpr (P == 5) return kGaussB5[q][i];
   else return kGaussB6[q][i];
+}
+// KH[j][k], GH[j][k], TH[j] and NH[j] of degree P
+template <int P>
+__device__ __forceinline__ constexpr double hat_k(int j, int k) {
+  if constexpr (P == 1) return kHatK1[j][k];
+  else if constexpr (P == 2) return kHatK2[j][k];
+  else if constexpr (P == 3) return kHatK3[j][k];
+  else if constexpr (P == 4) return kHatK4[j][k];
+  else if constexpr (P == 5) return kHatK5[j][k];
+  else return kHatK6[j][k];
+}
+template <int P>
+__device__ __forceinline__ constexpr double hat_g(int j, int k) {
+  if constexpr (P == 1) return kHatG1[j][k];
+  else if constexpr (P == 2) return kHatG2[j][k];
+  else if constexpr (P == 3) return kHatG3[j][k];
+  else if constexpr (P == 4) return kHatG4[j][k];
+  else if constexpr (P == 5) return kHatG5[j][k];
+  else return kHatG6[j][k];
+}
+template <int P>
+__device__ __forceinline__ constexpr double hat_t(int j) {
+  if constexpr (P == 1) return kHatT1[0][j];
+  else if constexpr (P == 2) return kHatT2[0][j];
+  else if constexpr (P == 3) return kHatT3[0][j];
+  else if constexpr (P == 4) return kHatT4[0][j];
+  else if constexpr (P == 5) return kHatT5[0][j];
+  else return kHatT6[0][j];
+}
+template <int P>
+__device__ __forceinline__ constexpr double hat_n(int j) {
+  if constexpr (P == 1) return kHatN1[0][j];
+  else if constexpr (P == 2) return kHatN2[0][j];
+  else if constexpr (P == 3) return kHatN3[0][j];
+  else if constexpr (P == 4) return kHatN4[0][j];
+  else if constexpr (P == 5) return kHatN5[0][j];
+  else return kHatN6[0][j];
 }
 
 }  // namespace fe""")

@@ -264,3 +264,31 @@ def test_rayleigh_ritz_jacobi_eigensolver_matches_oracle(fe, prec):
     assert np.max(np.abs(Q.T @ Q - np.eye(40))) <= (1e-10 if prec == "f64" else 1e-5)
     if prec == "f64":
         assert np.max(np.abs(Q.T @ (H @ Q) - np.diag(lam))) <= 1e-9
+
+
+# one cell more and one less than the sweep kernel's tiles, one vector around its vector tiles
+# (8 and 16 float, 4 and 8 double), z segments of one layer and of several
+@pytest.mark.parametrize("p,ncell", [(1, (9, 8, 5)), (2, (4, 5, 4)), (3, (4, 3, 7)), (4, (3, 4, 5)),
+                                     (5, (2, 3, 4)), (6, (3, 2, 3))])
+@pytest.mark.parametrize("nvec", [7, 9, 16, 17, 33])
+def test_sweep_tile_edges(fe, p, ncell, nvec):
+    """Ragged tiles in x, y and the vectors, float and double, on cells of three different
+    lengths; entry-by-entry bounds as above, and the alpha, beta, shift combination of a filter
+    step through a degree-two filter (column bounds as above)."""
+    L = (1.7 * ncell[0], 2.0 * ncell[1], 2.4 * ncell[2])
+    om, H, m, rng = _setup(fe, L, ncell, p, (True, False), seed=p)
+    X = rng.standard_normal((om.n_psi, nvec))
+    lo, hi = -2.0, 1.1 * float(abs(H).sum(axis=1).max())
+    a = lo + 0.1 * (hi - lo)
+    for prec, tol, ftol in ((fe.FE_F64, 1e-13, 1e-11), (fe.FE_F32, 1e-6, 1e-5)):
+        ld = -(-nvec // 4) * 4
+        buf, Xg = _block(X, prec, fe, ld)
+        x = Xg.double().cpu().numpy()
+        ybuf = torch.full_like(buf, 7.0)
+        fe._lib.call("fe_apply_H", m.handle, fe._ptr(buf), fe._ptr(ybuf), nvec, ld, int(prec))
+        assert_operator_entries(ybuf[:, :nvec].double().cpu().numpy(), H @ x, magnitude(H, x), tol,
+                                f"H X p={p}")
+        assert torch.all(ybuf[:, nvec:] == 7.0)
+        ref = chefsi.cheb_filter(lambda Z: H @ Z, x, 2, a, hi, lo)
+        m.cheb_filter(Xg, 2, a, hi, lo, prec=prec)
+        assert_column_maxabs(Xg.double().cpu().numpy(), ref, ftol, "filter")
