@@ -21,54 +21,123 @@
 namespace {
 
 constexpr int NCHAN = 4;
-constexpr int PROJ_THREADS = 128;
 
-// C[a][beta][v] for one atom and a tile of PROJ_THREADS vectors
+// 16-byte groups of vectors (rows are 16-byte aligned and a multiple of 16 bytes long, so a
+// group that holds a vector lies inside its row)
 template <typename T>
-__global__ void k_nl_project(const T* __restrict__ X, int64_t ld, int64_t nvec,
-                             const int* __restrict__ atom_ptr, const int* __restrict__ ent_node,
-                             const T* __restrict__ ent_val, T* __restrict__ C) {
-  const int a = blockIdx.x;
-  const int64_t v = (int64_t)blockIdx.y * PROJ_THREADS + threadIdx.x;
-  if (v >= nvec) return;
-  T c0 = T(0), c1 = T(0), c2 = T(0), c3 = T(0);
-  for (int e = atom_ptr[a]; e < atom_ptr[a + 1]; ++e) {
-    const T x = X[(int64_t)ent_node[e] * ld + v];
-    c0 += ent_val[4 * e + 0] * x;
-    c1 += ent_val[4 * e + 1] * x;
-    c2 += ent_val[4 * e + 2] * x;
-    c3 += ent_val[4 * e + 3] * x;
+struct NlGroup;
+template <>
+struct NlGroup<float> {
+  using V = float4;
+  static constexpr int W = 4;
+  static __device__ __forceinline__ float4 zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
+  static __device__ __forceinline__ float4 fma(float a, const float4& x, const float4& y) {
+    return make_float4(fmaf(a, x.x, y.x), fmaf(a, x.y, y.y), fmaf(a, x.z, y.z), fmaf(a, x.w, y.w));
   }
-  T* Ca = C + (int64_t)a * NCHAN * nvec;
-  Ca[v] = c0;
-  Ca[nvec + v] = c1;
-  Ca[2 * nvec + v] = c2;
-  Ca[3 * nvec + v] = c3;
+  static __device__ __forceinline__ float4 add_xor(float4 x, int o) {
+    x.x += __shfl_xor_sync(0xffffffffu, x.x, o);
+    x.y += __shfl_xor_sync(0xffffffffu, x.y, o);
+    x.z += __shfl_xor_sync(0xffffffffu, x.z, o);
+    x.w += __shfl_xor_sync(0xffffffffu, x.w, o);
+    return x;
+  }
+};
+template <>
+struct NlGroup<double> {
+  using V = double2;
+  static constexpr int W = 2;
+  static __device__ __forceinline__ double2 zero() { return make_double2(0.0, 0.0); }
+  static __device__ __forceinline__ double2 fma(double a, const double2& x, const double2& y) {
+    return make_double2(::fma(a, x.x, y.x), ::fma(a, x.y, y.y));
+  }
+  static __device__ __forceinline__ double2 add_xor(double2 x, int o) {
+    x.x += __shfl_xor_sync(0xffffffffu, x.x, o);
+    x.y += __shfl_xor_sync(0xffffffffu, x.y, o);
+    return x;
+  }
+};
+
+constexpr int PROJ_GROUPS = 8, PROJ_SLOTS = 32;   // vector groups and entry slots of a block
+constexpr int PROJ_THREADS = PROJ_GROUPS * PROJ_SLOTS;
+
+// C[a][beta][v] = D[a][beta] sum_e Pt[e][beta] X[node_e][v] for one atom and a tile of vector
+// groups (rows of C are ldc long, a multiple of a group).  An atom has a thousand entries
+// and there are few atoms, so its entries are spread over 32 slots of a block, four loads in
+// flight each, and the slots summed in a fixed order: with one thread walking all entries of
+// a vector the launch took 300 us (64 atoms, 128 float vectors, 190,400 nodes, p = 5), bound by
+// the latency of its loads; now 24 us.  (The coefficients D are applied here, once an atom,
+// instead of at every node.)
+template <typename T>
+__global__ void __launch_bounds__(PROJ_THREADS)
+k_nl_project(const T* __restrict__ X, int64_t ld, int64_t nvec, const int* __restrict__ atom_ptr,
+             const int* __restrict__ ent_node, const T* __restrict__ ent_val,
+             const T* __restrict__ Dv, T* __restrict__ C, int64_t ldc) {
+  using G = NlGroup<T>;
+  using V = typename G::V;
+  __shared__ V red[PROJ_THREADS / 32][PROJ_GROUPS][NCHAN];
+  const int a = blockIdx.x, g = threadIdx.x % PROJ_GROUPS, slot = threadIdx.x / PROJ_GROUPS;
+  const int64_t v = ((int64_t)blockIdx.y * PROJ_GROUPS + g) * G::W;
+  const bool in = v < nvec;
+  const int e1 = atom_ptr[a + 1];
+  V c[NCHAN];
+#pragma unroll
+  for (int b = 0; b < NCHAN; ++b) c[b] = G::zero();
+#pragma unroll 4
+  for (int e = atom_ptr[a] + slot; e < e1; e += PROJ_SLOTS) {
+    V x = G::zero();
+    if (in) x = *reinterpret_cast<const V*>(X + (int64_t)ent_node[e] * ld + v);
+#pragma unroll
+    for (int b = 0; b < NCHAN; ++b) c[b] = G::fma(ent_val[(int64_t)NCHAN * e + b], x, c[b]);
+  }
+#pragma unroll
+  for (int b = 0; b < NCHAN; ++b) {
+    c[b] = G::add_xor(c[b], 8);
+    c[b] = G::add_xor(c[b], 16);
+    if ((threadIdx.x & 31) < PROJ_GROUPS) red[threadIdx.x / 32][g][b] = c[b];
+  }
+  __syncthreads();
+  if (threadIdx.x < PROJ_GROUPS * NCHAN) {
+    const int b = threadIdx.x / PROJ_GROUPS;
+    V t = red[0][g][b];
+#pragma unroll
+    for (int w = 1; w < PROJ_THREADS / 32; ++w) t = G::fma(T(1), red[w][g][b], t);
+    // (a group past the last vector lies in the padding of C's row, or beyond it)
+    if (in)
+      *reinterpret_cast<V*>(C + ((int64_t)a * NCHAN + b) * ldc + v) =
+          G::fma(Dv[NCHAN * a + b], t, G::zero());
+  }
 }
 
-// Y[node][v] += alpha sum_e sum_beta Pt[e][beta] D[a_e][beta] C[a_e][beta][v]; one warp per
-// touched node, lanes over the vectors
+// Y[node][v] += alpha sum_e sum_beta Pt[e][beta] C[a_e][beta][v]: one thread per touched node
+// and vector group (35 us with a warp per node and scalar lanes, 21 us so, on the same slab:
+// half of it the update of Y itself)
 template <typename T>
-__global__ void k_nl_apply(T* __restrict__ Y, int64_t ld, int64_t nvec, int ntouched,
-                           const int* __restrict__ tn_node, const int* __restrict__ tn_ptr,
-                           const int* __restrict__ tn_ent, const int* __restrict__ ent_atom,
-                           const T* __restrict__ ent_val, const T* __restrict__ Dv,
-                           const T* __restrict__ C, T alpha) {
-  const int lane = threadIdx.x & 31;
-  const int warps = gridDim.x * (blockDim.x >> 5);
-  for (int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < ntouched; t += warps) {
-    T* yrow = Y + (int64_t)tn_node[t] * ld;
-    const int e0 = tn_ptr[t], e1 = tn_ptr[t + 1];
-    for (int64_t v = lane; v < nvec; v += 32) {
-      T acc = T(0);
-      for (int k = e0; k < e1; ++k) {
-        const int e = tn_ent[k];
-        const int a = ent_atom[e];
-        const T* Ca = C + (int64_t)a * NCHAN * nvec;
+__global__ void __launch_bounds__(256)
+k_nl_apply(T* __restrict__ Y, int64_t ld, int64_t nvec, int64_t ntouched,
+           const int* __restrict__ tn_node, const int* __restrict__ tn_ptr,
+           const int* __restrict__ tn_ent, const int* __restrict__ ent_atom,
+           const T* __restrict__ ent_val, const T* __restrict__ C, int64_t ldc, T alpha) {
+  using G = NlGroup<T>;
+  using V = typename G::V;
+  const uint32_t ng = (uint32_t)(ldc / G::W);
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ntouched * ng;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t t = i / ng, v = (i - t * ng) * G::W;
+    T* yp = Y + (int64_t)tn_node[t] * ld + v;
+    V y = *reinterpret_cast<const V*>(yp), acc = G::zero();
+    for (int k = tn_ptr[t]; k < tn_ptr[t + 1]; ++k) {
+      const int e = tn_ent[k];
+      const T* Ca = C + (int64_t)ent_atom[e] * NCHAN * ldc + v;
 #pragma unroll
-        for (int b = 0; b < NCHAN; ++b) acc += ent_val[4 * e + b] * Dv[4 * a + b] * Ca[b * nvec + v];
-      }
-      yrow[v] += alpha * acc;
+      for (int b = 0; b < NCHAN; ++b)
+        acc = G::fma(ent_val[(int64_t)NCHAN * e + b], *reinterpret_cast<const V*>(Ca + b * ldc), acc);
+    }
+    y = G::fma(alpha, acc, y);
+    if (v + G::W <= nvec) {
+      *reinterpret_cast<V*>(yp) = y;
+    } else {
+      const T* o = reinterpret_cast<const T*>(&y);
+      for (int64_t j = 0; v + j < nvec; ++j) yp[j] = o[j];
     }
   }
 }
@@ -210,28 +279,24 @@ fe_status fe_nonlocal_apply(fe_mesh* m, const void* X, void* Y, int64_t nvec, in
   if (nl.natoms == 0 || nl.nnz == 0) return FE_OK;
   cudaStream_t st = m->stream;
   const size_t eb = dbl ? 8 : 4;
+  const int64_t w = dbl ? 2 : 4, ldc = (nvec + w - 1) / w * w, ng = ldc / w;
   void* c;
-  FE_TRY(fe_ws(m, WS_NL, eb * NCHAN * (size_t)nl.natoms * nvec + 64, &c));
-  dim3 pg(nl.natoms, (unsigned)((nvec + PROJ_THREADS - 1) / PROJ_THREADS));
-  int ab = (nl.ntouched + 7) / 8;
-  if (ab > 152 * 32) ab = 152 * 32;
-  if (dbl) {
-    k_nl_project<double><<<pg, PROJ_THREADS, 0, st>>>((const double*)X, ld, nvec, nl.atom_ptr,
-                                                      nl.ent_node, nl.ent_val, (double*)c);
+  FE_TRY(fe_ws(m, WS_NL, eb * NCHAN * (size_t)nl.natoms * ldc + 64, &c));
+  const int64_t tiles = (ng + PROJ_GROUPS - 1) / PROJ_GROUPS;
+  if (tiles > 65535) return fe_fail(FE_EINVAL, "nonlocal term: too many vectors");
+  const dim3 pg(nl.natoms, (unsigned)tiles);
+  const int ab = (int)std::min<int64_t>(((int64_t)nl.ntouched * ng + 255) / 256, 152 * 32);
+  auto run = [&](auto zero, const auto* val, const auto* D) {
+    using T = decltype(zero);
+    k_nl_project<T><<<pg, PROJ_THREADS, 0, st>>>((const T*)X, ld, nvec, nl.atom_ptr, nl.ent_node, val,
+                                                 D, (T*)c, ldc);
     fe_count_launch();
-    k_nl_apply<double><<<ab, 256, 0, st>>>((double*)Y, ld, nvec, nl.ntouched, nl.tn_node, nl.tn_ptr,
-                                           nl.tn_ent, nl.ent_atom, nl.ent_val, nl.D,
-                                           (const double*)c, alpha);
+    k_nl_apply<T><<<ab, 256, 0, st>>>((T*)Y, ld, nvec, nl.ntouched, nl.tn_node, nl.tn_ptr, nl.tn_ent,
+                                      nl.ent_atom, val, (const T*)c, ldc, (T)alpha);
     fe_count_launch();
-  } else {
-    k_nl_project<float><<<pg, PROJ_THREADS, 0, st>>>((const float*)X, ld, nvec, nl.atom_ptr,
-                                                     nl.ent_node, nl.ent_val_f, (float*)c);
-    fe_count_launch();
-    k_nl_apply<float><<<ab, 256, 0, st>>>((float*)Y, ld, nvec, nl.ntouched, nl.tn_node, nl.tn_ptr,
-                                          nl.tn_ent, nl.ent_atom, nl.ent_val_f, nl.D_f,
-                                          (const float*)c, (float)alpha);
-    fe_count_launch();
-  }
+  };
+  if (dbl) run(0.0, (const double*)nl.ent_val, (const double*)nl.D);
+  else run(0.f, (const float*)nl.ent_val_f, (const float*)nl.D_f);
   FE_CUDA(cudaGetLastError());
   return FE_OK;
 }

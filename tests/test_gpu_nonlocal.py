@@ -99,3 +99,21 @@ def test_batch_and_static_filter_refuse_the_term(fe):
         fe._lib.call("fe_cheb_filter_static", m.handle, fe._ptr(X), 4, 4, 4, 1.0, 2.0, 0.0,
                      fe.FE_F64)
     assert e.value.status == 7
+
+
+@pytest.mark.parametrize("nvec", [1, 3, 31, 33, 70])
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+def test_nonlocal_vector_tiles(fe, prec, nvec):
+    """Vector counts around the projection's tiles (16 and 32 vectors) and its 16-byte groups,
+    in padded rows whose padding stays untouched; same bounds as above."""
+    P = fe.FE_F64 if prec == "f64" else fe.FE_F32
+    om, H, m = _setup(fe, (True, False), p=2)
+    ld = -(-nvec // 4) * 4 + 4
+    buf = torch.full((om.n_psi, ld), 3.0, dtype=fe.storage_dtype(P), device="cuda")
+    buf[:, :nvec] = torch.tensor(np.random.default_rng(nvec).standard_normal((om.n_psi, nvec)))
+    out = torch.full_like(buf, 7.0)
+    fe._lib.call("fe_apply_H", m.handle, fe._ptr(buf), fe._ptr(out), nvec, ld, int(P))
+    ref = H @ buf[:, :nvec].double().cpu().numpy()
+    err = np.linalg.norm(out[:, :nvec].double().cpu().numpy() - ref) / np.linalg.norm(ref)
+    assert err <= (1e-10 if prec == "f64" else 2e-5), err
+    assert torch.all(out[:, nvec:] == 7.0)
