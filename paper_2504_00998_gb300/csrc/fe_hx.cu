@@ -149,6 +149,9 @@ extern "C" fe_status fe_poisson_apply_K(fe_mesh* m, const double* x, double* y) 
     return fe_fail(FE_EINVAL, "fe_poisson_apply_K: arrays must be 8-byte aligned");
   if (x == y) return fe_fail(FE_EINVAL, "fe_poisson_apply_K: x and y must differ");
   FE_TRY(fe_activate(m));
+  bool done = false;
+  FE_TRY(fe_kcell_apply_f64(m, x, y, &done));
+  if (done) return FE_OK;
   KronIO<double> io{x, 1, y, 1, nullptr, 1, nullptr, 1, 1.0, 0.0, 0.0};
   return fe::kron_k1(m->coefK, fe_geom(m, false), io, m->stream);
 }

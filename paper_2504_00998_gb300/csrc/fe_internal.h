@@ -316,6 +316,8 @@ fe_status fe_rr_complex(fe_mesh* m, void* X, int64_t nvec, int64_t ld, double* e
 // scratch (WS_KCELL) is fe_kcell_scratch_bytes
 size_t fe_kcell_scratch_bytes(const fe_mesh* m);
 fe_status fe_kcell_apply_f32(fe_mesh* m, const float* x, float* y);
+// the same in double (fe_kcell64.cu), where its scratch can be had (*done)
+fe_status fe_kcell_apply_f64(fe_mesh* m, const double* x, double* y, bool* done);
 fe_status fe_activate(const fe_mesh* m);
 KronGeom fe_geom(const fe_mesh* m, bool psi);
 // Y = alpha (Ht - shift) X + beta Z (plus alpha Ht_nloc X and the quadrature potential when

@@ -46,10 +46,12 @@ struct PGeom {
   double ax, ay, az;
 };
 
+// (32-bit: a mesh has fewer than 2^31 nodes)
 __device__ __forceinline__ void pnode(const PGeom& g, int64_t id, int* gx, int* gy, int* gz) {
-  *gx = (int)(id % g.NX);
-  *gy = (int)((id / g.NX) % g.NY);
-  *gz = (int)(id / ((int64_t)g.NX * g.NY));
+  const uint32_t row = (uint32_t)id / (uint32_t)g.NX;
+  *gx = (int)((uint32_t)id - row * (uint32_t)g.NX);
+  *gz = (int)(row / (uint32_t)g.NY);
+  *gy = (int)(row - (uint32_t)*gz * (uint32_t)g.NY);
 }
 
 __device__ __forceinline__ double zcoord(const PGeom& g, int gz) {
@@ -73,7 +75,25 @@ __device__ __forceinline__ double vapp(double z, double E, double Lz) {
   return -E * (z - 0.5 * Lz);
 }
 
-// f = 4 pi M (rho + b); Jacobi inverse; constraint mask and values; phi initialisation
+// 1 / K_II of the assembled stiffness
+__device__ __forceinline__ double jacobi_inverse(const PGeom& g, int gx, int gy, int gz) {
+  const int nz = g.NZ - 1;
+  double kx = diag1(g.K1diag, g.p, gx, true, 0), mx = diag1(g.M1diag, g.p, gx, true, 0);
+  double ky = diag1(g.K1diag, g.p, gy, true, 0), my = diag1(g.M1diag, g.p, gy, true, 0);
+  double kz = diag1(g.K1diag, g.p, gz, false, nz), mz = diag1(g.M1diag, g.p, gz, false, nz);
+  double d = g.ax * kx * my * mz + g.ay * mx * ky * mz + g.az * mx * my * kz;
+  return 1.0 / d;
+}
+__global__ void k_dinv(PGeom g, double* __restrict__ dinv, int64_t n) {
+  for (int64_t id = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; id < n;
+       id += (int64_t)gridDim.x * blockDim.x) {
+    int gx, gy, gz;
+    pnode(g, id, &gx, &gy, &gz);
+    dinv[id] = jacobi_inverse(g, gx, gy, gz);
+  }
+}
+
+// f = 4 pi M (rho + b); Jacobi inverse (dinv may be null); constraint mask and values; phi initialisation
 // (f_ext: a given load instead of 4 pi M (rho + b); phic_ext: given constrained values)
 __global__ void k_setup(PGeom g, fe_poisson_bc bc, const double* __restrict__ mass,
                         const double* __restrict__ rho, const double* __restrict__ b,
@@ -86,12 +106,7 @@ __global__ void k_setup(PGeom g, fe_poisson_bc bc, const double* __restrict__ ma
     int gx, gy, gz;
     pnode(g, id, &gx, &gy, &gz);
     f[id] = f_ext ? f_ext[id] : FOUR_PI * mass[id] * (rho[id] + b[id]);
-    int nz = g.NZ - 1;
-    double kx = diag1(g.K1diag, g.p, gx, true, 0), mx = diag1(g.M1diag, g.p, gx, true, 0);
-    double ky = diag1(g.K1diag, g.p, gy, true, 0), my = diag1(g.M1diag, g.p, gy, true, 0);
-    double kz = diag1(g.K1diag, g.p, gz, false, nz), mz = diag1(g.M1diag, g.p, gz, false, nz);
-    double d = g.ax * kx * my * mz + g.ay * mx * ky * mz + g.az * mx * my * kz;
-    dinv[id] = 1.0 / d;
+    if (dinv) dinv[id] = jacobi_inverse(g, gx, gy, gz);
     unsigned char c = 0;
     double val = 0.0;
     if (bc.kind == FE_BIAS_CPD) {
@@ -364,7 +379,7 @@ __global__ void k_vbare(PGeom g, const double* __restrict__ phi, const double* _
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < npsi;
        i += (int64_t)gridDim.x * blockDim.x) {
     int64_t id = i + off;
-    int gz = (int)(id / ((int64_t)g.NX * g.NY));
+    int gz = (int)((uint32_t)id / ((uint32_t)g.NX * (uint32_t)g.NY));
     double v = phi[id] + vlms[id];
     if (cef) v += vapp(zcoord(g, gz), field, g.Lz);
     out[i] = v;
@@ -1513,8 +1528,12 @@ static fe_status poisson_solve_on(fe_mesh* m, const double* rho, const fe_poisso
   const int gb = fe::grid_for(n);
   PGeom g = make_geom(m);
 
-  k_setup<<<gb, 256, 0, st>>>(g, *bc, m->d_mass, rh, m->d_b, m->d_vlms, f_ext, phic_ext, f, dinv,
-                              mask, phi, n); fe_count_launch();
+  // (the separable preconditioner does not use the Jacobi inverse: forty FP64 operations a node)
+  const bool separable = mixed && use_graph && n >= SEP_MIN_NODES && !m->precond_set &&
+                         m->poisson_iter == FE_POISSON_ITER_PERSISTENT && m->cg_stall < 0 &&
+                         fe_sep::supported(m);
+  k_setup<<<gb, 256, 0, st>>>(g, *bc, m->d_mass, rh, m->d_b, m->d_vlms, f_ext, phic_ext, f,
+                              separable ? nullptr : dinv, mask, phi, n); fe_count_launch();
   if (project) {
     k_psum<double><<<fe::RED_BLOCKS, fe::RED_THREADS, 0, st>>>(f, nullptr, n, pa); fe_count_launch();
     k_psum<double><<<fe::RED_BLOCKS, fe::RED_THREADS, 0, st>>>(m->d_mass, nullptr, n, pb); fe_count_launch();
@@ -1523,8 +1542,10 @@ static fe_status poisson_solve_on(fe_mesh* m, const double* rho, const fe_poisso
   }
 
   // double residual r = f - K phi (masked; CEF: minus its mean) and |r|^2 on the host
-  auto residual = [&](double* rr) -> fe_status {
-    FE_TRY(fe_poisson_apply_K(m, phi, q));
+  // (at_zero: phi is zero everywhere, as the CEF solve starts, so K phi needs no product)
+  auto residual = [&](double* rr, bool at_zero = false) -> fe_status {
+    if (at_zero) FE_CUDA(cudaMemsetAsync(q, 0, sizeof(double) * n, st));
+    else FE_TRY(fe_poisson_apply_K(m, phi, q));
     k_resid0<<<gb, 256, 0, st>>>(f, q, mask, r, n); fe_count_launch();
     if (project) {
       k_psum<double><<<fe::RED_BLOCKS, fe::RED_THREADS, 0, st>>>(r, nullptr, n, pa); fe_count_launch();
@@ -1540,7 +1561,7 @@ static fe_status poisson_solve_on(fe_mesh* m, const double* rho, const fe_poisso
     return FE_OK;
   };
   double rr = 0.0;
-  FE_TRY(residual(&rr));
+  FE_TRY(residual(&rr, project));
   if (!std::isfinite(rr)) {
     // a NaN or infinity in rho, the atoms or the constraint values: no iteration can mean
     // anything, so report it instead of running to the iteration cap
@@ -1556,8 +1577,7 @@ static fe_status poisson_solve_on(fe_mesh* m, const double* rho, const fe_poisso
   int64_t gk_f = 0, gk_d = 0;
 
   // Separable preconditioner: default options, meshes of SEP_MIN_NODES nodes or more
-  if (mixed && rr > tol2 && use_graph && n >= SEP_MIN_NODES && !m->precond_set &&
-      m->poisson_iter == FE_POISSON_ITER_PERSISTENT && m->cg_stall < 0 && fe_sep::supported(m)) {
+  if (separable && rr > tol2) {
     if (m->sep_state == 0 || !same_constraints(m->sep_key, *bc)) {
       std::vector<double> hcnt(nzp);
       k_plane_sum<double><<<nzp, fe::RED_THREADS, 0, st>>>(nullptr, mask, plane_n, z); fe_count_launch();
@@ -1582,6 +1602,9 @@ static fe_status poisson_solve_on(fe_mesh* m, const double* rho, const fe_poisso
   const double* ccnt = nullptr;
   const float* Amodes = nullptr;
   const float* mtab = nullptr;
+  if (separable && rr > tol2 && used < bc->max_iter) {
+    k_dinv<<<gb, 256, 0, st>>>(g, dinv, n); fe_count_launch();
+  }
   if (rr > tol2 && used < bc->max_iter)
     FE_TRY(coarse_setup(m, bc, mask, z, q, &Ainv, &ccnt, &Amodes, &mtab));
   double* csum = Ainv ? (double*)(ccnt + nzp) : nullptr;
@@ -1662,7 +1685,8 @@ static fe_status poisson_solve_on(fe_mesh* m, const double* rho, const fe_poisso
   if (project) {
     k_psum<double><<<fe::RED_BLOCKS, fe::RED_THREADS, 0, st>>>(m->d_mass, phi, n, pa); fe_count_launch();
     k_psum<double><<<fe::RED_BLOCKS, fe::RED_THREADS, 0, st>>>(m->d_mass, nullptr, n, pb); fe_count_launch();
-    k_shift_mean<<<gb, fe::RED_BLOCKS, 0, st>>>(phi, pa, pb, n); fe_count_launch();
+    // (few blocks: each one sums the partials)
+    k_shift_mean<<<std::min(gb, 304), fe::RED_BLOCKS, 0, st>>>(phi, pa, pb, n); fe_count_launch();
   }
   if (vbare) {
     k_vbare<<<fe::grid_for(m->n_psi), 256, 0, st>>>(g, phi, m->d_vlms, bc->field, project,

@@ -425,6 +425,10 @@ __device__ __forceinline__ double sum_partials(const double* part, int n) {
   return block_total(v);
 }
 
+// blocks of the vector steps (six an SM: the loads of a few entries a thread in flight, and few
+// enough partials for every block of the next step to sum them itself)
+constexpr int VEC_BLOCKS = 912;
+
 // scalars of iteration `it` in slots it % 2 (an iteration reads the previous one's while it
 // writes its own)
 struct Scalars {
@@ -443,15 +447,23 @@ k_sep_direction(double* __restrict__ p, const double* __restrict__ z, int64_t n,
     beta = old != 0.0 ? -s->alpha[(it + 1) % 2] * qz / old : 0.0;
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) s->rz[it % 2] = rz;
+  if (it == 0) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x)
+      p[i] = z[i];
+    return;
+  }
+#pragma unroll 4
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
-    p[i] = it > 0 ? fma(beta, p[i], z[i]) : z[i];
+    p[i] = fma(beta, p[i], z[i]);
 }
 
 __global__ void __launch_bounds__(fe::RED_THREADS)
 k_sep_dot(const double* __restrict__ p, const double* __restrict__ q, int64_t n,
           double* __restrict__ part) {
   double v = 0.0;
+#pragma unroll 4
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
     v = fma(p[i], q[i], v);
@@ -466,10 +478,11 @@ k_sep_update(double* __restrict__ phi, double* __restrict__ r, const double* __r
              const double* __restrict__ q, const unsigned char* __restrict__ mask, int64_t n,
              const double* __restrict__ part_pq, Scalars* s, int it,
              double* __restrict__ part_rr) {
-  const double pq = sum_partials(part_pq, fe::RED_BLOCKS);
+  const double pq = sum_partials(part_pq, gridDim.x);
   const double alpha = pq != 0.0 ? s->rz[it % 2] / pq : 0.0;
   if (blockIdx.x == 0 && threadIdx.x == 0) s->alpha[it % 2] = alpha;
   double v = 0.0;
+#pragma unroll 4
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     phi[i] = fma(alpha, p[i], phi[i]);
@@ -500,7 +513,7 @@ bool supported(const fe_mesh* m) {
 }
 
 size_t part_doubles(const fe_mesh* m) {
-  return 2 * (size_t)out_blocks(m->NZ * m->NY, m->NX) + 2 * fe::RED_BLOCKS + 16;
+  return 2 * (size_t)out_blocks(m->NZ * m->NY, m->NX) + 2 * VEC_BLOCKS + 16;
 }
 
 fe_status plan(fe_mesh* m, const double* cnt, bool constant_null) {
@@ -575,8 +588,8 @@ fe_status solve(fe_mesh* m, const Buf& b, double tol2, int maxit, double* rr, in
   const int rows = nz * NY, np = out_blocks(rows, NX);
   double* part_z = b.part;
   double* part_a = part_z + 2 * (size_t)np;
-  double* part_b = part_a + fe::RED_BLOCKS;
-  Scalars* s = reinterpret_cast<Scalars*>(part_b + fe::RED_BLOCKS);
+  double* part_b = part_a + VEC_BLOCKS;
+  Scalars* s = reinterpret_cast<Scalars*>(part_b + VEC_BLOCKS);
   double* total = reinterpret_cast<double*>(s + 1);
   // the constrained planes' entries of z and p stay zero
   FE_CUDA(cudaMemsetAsync(b.z, 0, sizeof(double) * n, st));
@@ -609,15 +622,15 @@ fe_status solve(fe_mesh* m, const Buf& b, double tol2, int maxit, double* rr, in
     g.W = t.VxT; g.in = b.ta; g.out_d = b.z + off; g.M = rows; g.N = NX; g.K = NX;
     g.mask = b.mask + off; g.r = b.r + off; g.q = it > 0 ? b.q + off : nullptr; g.part = part_z;
     FE_TRY(gemm<RIGHT_OUT>(g, 1, st));
-    k_sep_direction<<<fe::RED_BLOCKS, fe::RED_THREADS, 0, st>>>(b.p, b.z, n, part_z, np, s, it);
+    k_sep_direction<<<VEC_BLOCKS, fe::RED_THREADS, 0, st>>>(b.p, b.z, n, part_z, np, s, it);
     fe_count_launch();
     FE_TRY(fe_poisson_apply_K(m, b.p, b.q));
-    k_sep_dot<<<fe::RED_BLOCKS, fe::RED_THREADS, 0, st>>>(b.p, b.q, n, part_a);
+    k_sep_dot<<<VEC_BLOCKS, fe::RED_THREADS, 0, st>>>(b.p, b.q, n, part_a);
     fe_count_launch();
-    k_sep_update<<<fe::RED_BLOCKS, fe::RED_THREADS, 0, st>>>(b.phi, b.r, b.p, b.q, b.mask, n, part_a,
+    k_sep_update<<<VEC_BLOCKS, fe::RED_THREADS, 0, st>>>(b.phi, b.r, b.p, b.q, b.mask, n, part_a,
                                                              s, it, part_b);
     fe_count_launch();
-    k_sep_total<<<1, fe::RED_THREADS, 0, st>>>(part_b, fe::RED_BLOCKS, total);
+    k_sep_total<<<1, fe::RED_THREADS, 0, st>>>(part_b, VEC_BLOCKS, total);
     fe_count_launch();
     FE_CUDA(cudaGetLastError());
     FE_CUDA(cudaMemcpyAsync(rr, total, sizeof(double), cudaMemcpyDeviceToHost, st));

@@ -358,3 +358,22 @@ def test_separable_preconditioner(fe, kind, p, ncell):
     with pytest.raises(fe.FeError) as e:
         m.poisson_solve(bias, rtol=1e-12, max_iter=1)
     assert e.value.status == fe._lib.FE_ENOCONV
+
+
+@pytest.mark.parametrize("ncell,p", [((33, 1, 2), 1), ((17, 2, 1), 2), ((16, 3, 2), 3), ((9, 2, 3), 4),
+                                     ((8, 1, 2), 5), ((5, 3, 2), 6)])
+def test_apply_K_cell_strips(fe, ncell, p):
+    """The double stiffness product at full, partial and single strips of cells, with three
+    different cell lengths: 1e-12 relative as above, entry by entry 1e-13 of |K| |x|, and two
+    calls agree bit for bit."""
+    L = (1.3 * ncell[0], 1.9 * ncell[1], 2.6 * ncell[2])
+    om = OMesh(L, ncell, p)
+    K = assembly.assemble_stiffness(om)
+    m = fe.Mesh(L, ncell, p)
+    x = np.random.default_rng(p).standard_normal(om.n_phi)
+    xt = torch.tensor(x, device="cuda")
+    y = m.poisson_apply_K(xt)
+    assert torch.equal(y, m.poisson_apply_K(xt))
+    y, ref = y.cpu().numpy(), K @ x
+    assert np.linalg.norm(y - ref) / np.linalg.norm(ref) <= 1e-12
+    assert np.all(np.abs(y - ref) <= 1e-13 * (abs(K) @ np.abs(x)))
