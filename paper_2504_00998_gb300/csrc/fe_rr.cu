@@ -84,6 +84,78 @@ __global__ void k_symmetrize(double* __restrict__ S, int n) {
   }
 }
 
+// S = X^T X and (HX non-null) Hs = X^T HX of narrow double blocks (n <= 64 vectors, node-major):
+// block partials over a share of the rows, then their sums in block order (bitwise
+// repeatable).  Both products read X once.  FP64 issue bounds it (2 n^2 N FMAs, about 50 us for
+// 15,228 x 32); cuBLAS's SYRK takes one CTA for such an n (4.4 ms) and its split-K GEMM 107 us
+// for the second product.
+constexpr int GRAM_MAX = 64, GRAM_BLOCKS = 152, GRAM_ROWS = 16, GRAM_THREADS = 256;
+
+// MB x MB entries of S and of Hs a thread: entry (ti + 16 a, tj + 16 b)
+template <int MB>
+__global__ void __launch_bounds__(GRAM_THREADS)
+k_gram_partial(const double* __restrict__ X, int64_t ld, const double* __restrict__ HX, int64_t ldh,
+               int n, int64_t N, double* __restrict__ part) {
+  constexpr int W = 16 * MB;
+  __shared__ double xs[GRAM_ROWS][W], hs[GRAM_ROWS][W];
+  const int tid = threadIdx.x, ti = tid / 16, tj = tid % 16;
+  const int64_t r0 = N * blockIdx.x / gridDim.x, r1 = N * (blockIdx.x + 1) / gridDim.x;
+  double s[MB][MB], h[MB][MB];
+#pragma unroll
+  for (int a = 0; a < MB; ++a)
+#pragma unroll
+    for (int b = 0; b < MB; ++b) s[a][b] = h[a][b] = 0.0;
+  for (int64_t r = r0; r < r1; r += GRAM_ROWS) {
+    for (int e = tid; e < GRAM_ROWS * W; e += GRAM_THREADS) {
+      const int row = e / W, c = e - row * W;
+      const bool in = r + row < r1 && c < n;
+      xs[row][c] = in ? X[(r + row) * ld + c] : 0.0;
+      hs[row][c] = in && HX ? HX[(r + row) * ldh + c] : 0.0;
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int row = 0; row < GRAM_ROWS; ++row) {
+      double xi[MB], xj[MB], hj[MB];
+#pragma unroll
+      for (int a = 0; a < MB; ++a) {
+        xi[a] = xs[row][ti + 16 * a];
+        xj[a] = xs[row][tj + 16 * a];
+        hj[a] = hs[row][tj + 16 * a];
+      }
+#pragma unroll
+      for (int a = 0; a < MB; ++a)
+#pragma unroll
+        for (int b = 0; b < MB; ++b) {
+          s[a][b] = fma(xi[a], xj[b], s[a][b]);
+          if (HX) h[a][b] = fma(xi[a], hj[b], h[a][b]);
+        }
+    }
+    __syncthreads();
+  }
+  double* ps = part + (int64_t)blockIdx.x * 2 * n * n;
+#pragma unroll
+  for (int a = 0; a < MB; ++a)
+#pragma unroll
+    for (int b = 0; b < MB; ++b) {
+      const int i = ti + 16 * a, j = tj + 16 * b;
+      if (i >= n || j >= n) continue;
+      ps[(int64_t)j * n + i] = s[a][b];
+      if (HX) ps[(int64_t)n * n + (int64_t)j * n + i] = h[a][b];
+    }
+}
+
+// entry e of the two matrices: its block partials in order, four chains
+__global__ void k_gram_sum(const double* __restrict__ part, int blocks, int64_t nn, int two,
+                           double* __restrict__ S, double* __restrict__ Hs) {
+  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (e >= nn * (two ? 2 : 1)) return;
+  double t[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int b = 0; b < blocks; ++b) t[b & 3] += part[(int64_t)b * 2 * nn + e];
+  const double v = (t[0] + t[1]) + (t[2] + t[3]);
+  if (e < nn) S[e] = v;
+  else Hs[e - nn] = v;
+}
+
 struct RrWs {
   double *S, *Q, *d, *eig, *work;
   int* info;
@@ -96,6 +168,37 @@ fe_status gram(fe_mesh* m, const double* A, int64_t lda, const double* B, int64_
   // S = A B^T with A, B = nvec x N column-major
   FE_CUBLAS(cublasDgemm(m->cublas, CUBLAS_OP_N, CUBLAS_OP_T, (int)nvec, (int)nvec,
                         (int)m->n_psi, &one, A, (int)lda, B, (int)ldb, &zero, S, (int)nvec));
+  return FE_OK;
+}
+
+// S = X^T X (its upper triangle at least) and, where Hs is given, Hs = X^T HX
+fe_status gram_pair(fe_mesh* m, const double* X, int64_t ld, const double* HX, int64_t ldh,
+                    int64_t nvec, double* S, double* Hs) {
+  const int n = (int)nvec;
+  void* part = nullptr;
+  fe_status st = FE_ENOMEM;
+  if (n <= GRAM_MAX) st = fe_ws(m, WS_RR_TC32, sizeof(double) * 2 * (size_t)n * n * GRAM_BLOCKS, &part);
+  if (st != FE_OK && st != FE_ENOMEM) return st;
+  if (st == FE_OK) {   // (without room for the partials: the library products)
+    double* p = (double*)part;
+    const double* hx = Hs ? HX : nullptr;
+    if (n <= 16)
+      k_gram_partial<1><<<GRAM_BLOCKS, GRAM_THREADS, 0, m->stream>>>(X, ld, hx, ldh, n, m->n_psi, p);
+    else if (n <= 32)
+      k_gram_partial<2><<<GRAM_BLOCKS, GRAM_THREADS, 0, m->stream>>>(X, ld, hx, ldh, n, m->n_psi, p);
+    else
+      k_gram_partial<4><<<GRAM_BLOCKS, GRAM_THREADS, 0, m->stream>>>(X, ld, hx, ldh, n, m->n_psi, p);
+    fe_count_launch();
+    const int64_t nn = (int64_t)n * n;
+    k_gram_sum<<<(unsigned)((2 * nn + 127) / 128), 128, 0, m->stream>>>(p, GRAM_BLOCKS, nn, Hs != nullptr, S, Hs);
+    fe_count_launch();
+    FE_CUDA(cudaGetLastError());
+    return FE_OK;
+  }
+  const double one = 1.0, zero = 0.0;
+  FE_CUBLAS(cublasDsyrk(m->cublas, CUBLAS_FILL_MODE_UPPER, CUBLAS_OP_N, n, (int)m->n_psi, &one, X,
+                        (int)ld, &zero, S, n));
+  if (Hs) FE_TRY(gram(m, X, ld, HX, ldh, nvec, Hs));
   return FE_OK;
 }
 
@@ -118,9 +221,7 @@ fe_status sym_eig(fe_mesh* m, int n, RrWs& w) {
 fe_status cholqr_pass(fe_mesh* m, double* X, int64_t ld, int64_t nvec, RrWs& w, double shift,
                       int* broke) {
   const int n = (int)nvec;
-  const double one_ = 1.0, zero_ = 0.0;
-  FE_CUBLAS(cublasDsyrk(m->cublas, CUBLAS_FILL_MODE_UPPER, CUBLAS_OP_N, n, (int)m->n_psi, &one_,
-                        X, (int)ld, &zero_, w.S, n));
+  FE_TRY(gram_pair(m, X, ld, nullptr, 0, nvec, w.S, nullptr));
   k_fill_lower<<<fe::grid_for((int64_t)n * n), 256, 0, m->stream>>>(w.S, n); fe_count_launch();
   k_scale_gram<<<1, 256, 0, m->stream>>>(w.S, n, w.d, shift); fe_count_launch();
   k_scale_cols<<<fe::grid_for(m->n_psi * nvec), 256, 0, m->stream>>>(X, ld, nvec, m->n_psi, w.d); fe_count_launch();
@@ -232,9 +333,7 @@ fe_status rr_gram_path(fe_mesh* m, const double* X, int64_t ld, const double* HX
   const int n = (int)nvec;
   const double one = 1.0, zero = 0.0;
   // S = A A^T (upper), Hs = A B^T
-  FE_CUBLAS(cublasDsyrk(m->cublas, CUBLAS_FILL_MODE_UPPER, CUBLAS_OP_N, n, (int)m->n_psi, &one,
-                        X, (int)ld, &zero, w.S, n));
-  FE_TRY(gram(m, X, ld, HX, ldh, nvec, w.Q));
+  FE_TRY(gram_pair(m, X, ld, HX, ldh, nvec, w.S, w.Q));
   FE_TRY(rr_small(m, nvec, w, eig, ill, kGramCondF64));
   if (*ill) return FE_OK;
   // Xout^T = C^T A

@@ -292,3 +292,21 @@ def test_sweep_tile_edges(fe, p, ncell, nvec):
         ref = chefsi.cheb_filter(lambda Z: H @ Z, x, 2, a, hi, lo)
         m.cheb_filter(Xg, 2, a, hi, lo, prec=prec)
         assert_column_maxabs(Xg.double().cpu().numpy(), ref, ftol, "filter")
+
+
+@pytest.mark.parametrize("n", [1, 15, 16, 17, 32, 33, 64, 65])
+def test_rayleigh_ritz_gram_sizes(fe, n):
+    """Double Rayleigh-Ritz at the edges of the narrow Gram kernel (tiles of 16, 32 and 64
+    vectors, library products above), rows padded past the block; bounds as above."""
+    om, H, m, rng = _setup(fe, (4.0, 4.0, 9.0), (2, 2, 4), 3, (True, True), seed=n)
+    X = rng.standard_normal((om.n_psi, n))
+    lam_ref, _ = chefsi.rayleigh_ritz(lambda Z: H @ Z, X)
+    buf, Xg = _block(X, fe.FE_F64, fe, -(-n // 2) * 2 + 2)
+    lam = torch.empty(n, dtype=torch.float64, device="cuda")
+    fe._lib.call("fe_rayleigh_ritz", m.handle, fe._ptr(buf), n, buf.stride(0), fe._ptr(lam), fe.FE_F64)
+    lam = lam.cpu().numpy()
+    assert np.max(np.abs(lam - lam_ref)) <= 1e-8
+    Q = Xg.cpu().numpy()
+    assert np.max(np.abs(Q.T @ Q - np.eye(n))) <= 1e-10
+    assert np.max(np.abs(Q.T @ (H @ Q) - np.diag(lam))) <= 1e-9
+    assert torch.all(buf[:, n:] == 0.0)
