@@ -68,11 +68,21 @@ __device__ __forceinline__ double diag1(const double* d, int p, int gi, bool per
   return d[0] + d[p];
 }
 
-__device__ __forceinline__ double vapp(double z, double E, double Lz) {
-  const double z1 = 0.1 * Lz, z2 = 0.9 * Lz;
-  if (z < z1) return -E * (z1 - 0.5 * Lz) * z / z1;
-  if (z > z2) return -E * (z2 - 0.5 * Lz) * (Lz - z) / (Lz - z2);
-  return -E * (z - 0.5 * Lz);
+// the sawtooth V_app: slope -E on [z1, z2], the ramps' slopes taken on the host (a division is
+// some twenty FP64 operations)
+struct VApp {
+  double E, Lz, z1, z2, s1, s2;
+};
+VApp make_vapp(double E, double Lz) {
+  VApp v{E, Lz, 0.1 * Lz, 0.9 * Lz, 0.0, 0.0};
+  v.s1 = -E * (v.z1 - 0.5 * Lz) / v.z1;
+  v.s2 = -E * (v.z2 - 0.5 * Lz) / (Lz - v.z2);
+  return v;
+}
+__device__ __forceinline__ double vapp(const VApp& v, double z) {
+  if (z < v.z1) return v.s1 * z;
+  if (z > v.z2) return v.s2 * (v.Lz - z);
+  return -v.E * (z - 0.5 * v.Lz);
 }
 
 // 1 / K_II of the assembled stiffness
@@ -374,14 +384,14 @@ __global__ void k_shift_mean(double* __restrict__ phi, const double* part_mphi,
 
 // V_eff at psi nodes: phi + (V_loc - V_sm) + V_app
 __global__ void k_vbare(PGeom g, const double* __restrict__ phi, const double* __restrict__ vlms,
-                        double field, int cef, int gz_lo, double* __restrict__ out, int64_t npsi) {
+                        VApp va, int cef, int gz_lo, double* __restrict__ out, int64_t npsi) {
   int64_t off = (int64_t)gz_lo * g.NX * g.NY;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < npsi;
        i += (int64_t)gridDim.x * blockDim.x) {
     int64_t id = i + off;
     int gz = (int)((uint32_t)id / ((uint32_t)g.NX * (uint32_t)g.NY));
     double v = phi[id] + vlms[id];
-    if (cef) v += vapp(zcoord(g, gz), field, g.Lz);
+    if (cef) v += vapp(va, zcoord(g, gz));
     out[i] = v;
   }
 }
@@ -1178,7 +1188,8 @@ extern "C" fe_status fe_vbare_phi(fe_mesh* m, const double* phi, const fe_poisso
   if (!m || !phi || !bc || !out) return fe_fail(FE_EINVAL, "fe_vbare_phi: null argument");
   if (!m->d_vlms) return fe_fail(FE_EINVAL, "fe_vbare_phi: call fe_set_atoms first");
   FE_TRY(fe_activate(m));
-  k_vbare<<<fe::grid_for(m->n_phi), 256, 0, m->stream>>>(make_geom(m), phi, m->d_vlms, bc->field,
+  k_vbare<<<fe::grid_for(m->n_phi), 256, 0, m->stream>>>(make_geom(m), phi, m->d_vlms,
+                                                           make_vapp(bc->field, m->desc.L[2]),
                                                            bc->kind == FE_BIAS_CEF, 0, out,
                                                            m->n_phi); fe_count_launch();
   FE_CUDA(cudaGetLastError());
@@ -1689,7 +1700,7 @@ static fe_status poisson_solve_on(fe_mesh* m, const double* rho, const fe_poisso
     k_shift_mean<<<std::min(gb, 304), fe::RED_BLOCKS, 0, st>>>(phi, pa, pb, n); fe_count_launch();
   }
   if (vbare) {
-    k_vbare<<<fe::grid_for(m->n_psi), 256, 0, st>>>(g, phi, m->d_vlms, bc->field, project,
+    k_vbare<<<fe::grid_for(m->n_psi), 256, 0, st>>>(g, phi, m->d_vlms, make_vapp(bc->field, g.Lz), project,
                                                       m->gz_lo, vbare, m->n_psi); fe_count_launch();
   }
   FE_CUDA(cudaGetLastError());

@@ -230,6 +230,52 @@ bool chain_eigen(const fe_mesh* m, int nc, bool periodic, int lo, int hi,
   return true;
 }
 
+// ---- reductions -----------------------------------------------------------------------------------
+// FP64 adds are slow here (sixteen cycles a warp and SM), so a block's sum is one warp's work:
+// each lane adds its share of the threads' terms in order, then a shuffle tree.  The total is
+// valid in thread 0.  blockDim.x is 256.
+__device__ __forceinline__ double block_total(double v) {
+  __shared__ double s[256];
+  s[threadIdx.x] = v;
+  __syncthreads();
+  double t = 0.0;
+  if (threadIdx.x < 32) {
+#pragma unroll
+    for (int w = 0; w < 8; ++w) t += s[threadIdx.x + 32 * w];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+  }
+  __syncthreads();
+  return t;
+}
+// Whether this block is the last of `blocks` to get here (every block's partials are then
+// visible); it finishes the sum, and the ticket is ready for the next launch.
+__device__ __forceinline__ bool last_block(unsigned int* ticket, unsigned int blocks) {
+  __shared__ bool last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(ticket, 1u) == blocks - 1;
+    if (last) {
+      *ticket = 0;
+      __threadfence();
+    }
+  }
+  __syncthreads();
+  return last;
+}
+__device__ __forceinline__ double sum_partials(const double* part, int n) {
+  double v = 0.0;
+  for (int i = threadIdx.x; i < n; i += 256) v += __ldcg(part + i);
+  return block_total(v);
+}
+
+// scalars of the iteration: r.z, alpha, beta, |r|^2, and the tickets of the three reductions
+struct Scalars {
+  double rz, alpha, beta, rr;
+  unsigned int ticket[3];
+};
+
 // ---- transforms -----------------------------------------------------------------------------
 // Device tables of the plan (floats): V [node][mode] and its transpose for every direction
 // and the eigenvalues with their mesh scale.
@@ -254,9 +300,11 @@ struct Gemm {
   const unsigned char* mask;
   const double *r, *q;   // dot products r.z (and q.z unless null) of the written values
   double* part;          // [2][blocks]
+  Scalars* s;
+  int first;             // the first iteration: no direction to keep
 };
 
-enum { LEFT = 0, LEFT_SCALE = 1, RIGHT_IN = 2, RIGHT_OUT = 3 };
+enum { LEFT = 0, LEFT_SCALE = 1, RIGHT_IN = 2, RIGHT_OUT = 3 };   // (LEFT_SCALE: z products only)
 
 constexpr int GT = 256, BK = 16;
 
@@ -343,28 +391,100 @@ __global__ void __launch_bounds__(GT) k_sep_gemm(const Gemm g) {
         g.out_d[at] = z;
         rz += g.r[at] * z;
         if (g.q) qz += g.q[at] * z;
-      } else if constexpr (MODE == LEFT_SCALE) {
-        const int bb = nn / g.NX, aa = nn - bb * g.NX;
-        const float l = g.lz[mm] + (g.ly[bb] + g.lx[aa]);
-        g.out[at] = l > g.null_below ? acc[i][j] / l : 0.f;
       } else {
         g.out[(RIGHT ? 0 : (int64_t)blockIdx.z * g.out_batch) + at] = acc[i][j];
       }
     }
   }
   if constexpr (MODE == RIGHT_OUT) {
-    __shared__ double s[2][GT / 32];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      rz += __shfl_down_sync(0xffffffffu, rz, o);
-      qz += __shfl_down_sync(0xffffffffu, qz, o);
+    // r.z and q.z; the last block takes the direction's beta = -alpha_old (q.z) / (r.z)_old
+    // (the flexible form: the float preconditioner is symmetric to rounding only)
+    const int nb = gridDim.x * gridDim.y, at = blockIdx.y * gridDim.x + blockIdx.x;
+    rz = block_total(rz);
+    qz = block_total(qz);
+    if (t == 0) {
+      g.part[at] = rz;
+      g.part[nb + at] = qz;
     }
-    if (t % 32 == 0) { s[0][t / 32] = rz; s[1][t / 32] = qz; }
+    if (last_block(&g.s->ticket[0], nb)) {
+      rz = sum_partials(g.part, nb);
+      qz = g.first ? 0.0 : sum_partials(g.part + nb, nb);
+      if (t == 0) {
+        Scalars* s = g.s;
+        const double old = s->rz;
+        s->beta = g.first || old == 0.0 ? 0.0 : -s->alpha * qz / old;
+        s->rz = rz;
+      }
+    }
+  }
+}
+
+// The z products (LEFT, LEFT_SCALE) at a larger tile: 64 x 128 a block, 4 x 8 results a thread
+// read as three 16-byte words for 32 FMAs (nine words for 20 in k_sep_gemm).  M is the length
+// of the z chain and N a whole plane: on the benchmark slab 237 to 241 x 6400, 200 blocks,
+// 37 us a product against 43 (means of the two; the 5 x 4 tile of k_sep_gemm).
+template <int MODE>
+__global__ void __launch_bounds__(GT) k_sep_gemm_z(const Gemm g) {
+  constexpr int BM = 64, BN = 128;
+  __shared__ __align__(16) float As[BK][BM];
+  __shared__ __align__(16) float Bs[BK][BN];
+  const int t = threadIdx.x, tx = t % 16, ty = t / 16;
+  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+  float acc[4][8];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+  float ra[4], rb[8];
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int k = k0 + t / 64 + 4 * i, m = m0 + t % 64;
+      ra[i] = (k < g.K && m < g.M) ? g.W[(int64_t)k * g.M + m] : 0.f;
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int k = k0 + t / 128 + 2 * i, n = n0 + t % 128;
+      rb[i] = (k < g.K && n < g.N) ? g.in[(int64_t)k * g.N + n] : 0.f;
+    }
+  };
+  fetch(0);
+  for (int k0 = 0; k0 < g.K; k0 += BK) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) As[t / 64 + 4 * i][t % 64] = ra[i];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) Bs[t / 128 + 2 * i][t % 128] = rb[i];
     __syncthreads();
-    if (t < 2) {
-      double v = 0.0;
-      for (int w = 0; w < GT / 32; ++w) v += s[t][w];
-      g.part[(int64_t)t * gridDim.x * gridDim.y + (int64_t)blockIdx.y * gridDim.x + blockIdx.x] = v;
+    if (k0 + BK < g.K) fetch(k0 + BK);
+#pragma unroll
+    for (int k = 0; k < BK; ++k) {
+      const float4 a = *reinterpret_cast<const float4*>(&As[k][4 * ty]);
+      const float4 b0 = *reinterpret_cast<const float4*>(&Bs[k][4 * tx]);
+      const float4 b1 = *reinterpret_cast<const float4*>(&Bs[k][64 + 4 * tx]);
+      const float av[4] = {a.x, a.y, a.z, a.w};
+      const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[i][j] = __fmaf_rn(av[i], bv[j], acc[i][j]);
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int mm = m0 + 4 * ty + i;
+    if (mm >= g.M) continue;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int nn = n0 + (j < 4 ? 4 * tx + j : 60 + 4 * tx + j);
+      if (nn >= g.N) continue;
+      float v = acc[i][j];
+      if constexpr (MODE == LEFT_SCALE) {
+        const int bb = nn / g.NX, aa = nn - bb * g.NX;
+        const float l = g.lz[mm] + (g.ly[bb] + g.lx[aa]);
+        v = l > g.null_below ? v / l : 0.f;
+      }
+      g.out[(int64_t)mm * g.N + nn] = v;
     }
   }
 }
@@ -401,103 +521,75 @@ fe_status gemm(const Gemm& g, int batch, cudaStream_t st) {
   return FE_OK;
 }
 
-// blocks of the last x product, whose dot-product partials the direction update sums
+template <int MODE>
+fe_status gemm_z(const Gemm& g, cudaStream_t st) {
+  k_sep_gemm_z<MODE><<<dim3((g.N + 127) / 128, (g.M + 63) / 64), GT, 0, st>>>(g);
+  fe_count_launch();
+  FE_CUDA(cudaGetLastError());
+  return FE_OK;
+}
+
+// blocks of the last x product (its dot-product partials)
 int out_blocks(int rows, int NX) {
   const int tm = tile_for(rows), tn = tile_for(NX);
   return ((rows + 16 * tm - 1) / (16 * tm)) * ((NX + 16 * tn - 1) / (16 * tn));
 }
 
 // ---- vector steps ------------------------------------------------------------------------------
-__device__ __forceinline__ double block_total(double v) {
-  __shared__ double s[32];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  if (threadIdx.x % 32 == 0) s[threadIdx.x / 32] = v;
-  __syncthreads();
-  double t = 0.0;
-  for (int w = 0; w < (int)blockDim.x / 32; ++w) t += s[w];
-  __syncthreads();
-  return t;
-}
-__device__ __forceinline__ double sum_partials(const double* part, int n) {
-  double v = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) v += part[i];
-  return block_total(v);
-}
+// blocks of the vector steps (four an SM)
+constexpr int VEC_BLOCKS = 608;
 
-// blocks of the vector steps (six an SM: the loads of a few entries a thread in flight, and few
-// enough partials for every block of the next step to sum them itself)
-constexpr int VEC_BLOCKS = 912;
-
-// scalars of iteration `it` in slots it % 2 (an iteration reads the previous one's while it
-// writes its own)
-struct Scalars {
-  double rz[2], alpha[2];
-};
-
-// p = z + beta p, beta = -alpha_old (q.z) / (r.z)_old (the flexible form: the float
-// preconditioner is symmetric to rounding only); block 0 keeps r.z
-__global__ void __launch_bounds__(fe::RED_THREADS)
-k_sep_direction(double* __restrict__ p, const double* __restrict__ z, int64_t n,
-                const double* __restrict__ part, int np, Scalars* s, int it) {
-  const double rz = sum_partials(part, np);
-  double beta = 0.0;
-  if (it > 0) {
-    const double qz = sum_partials(part + np, np), old = s->rz[(it + 1) % 2];
-    beta = old != 0.0 ? -s->alpha[(it + 1) % 2] * qz / old : 0.0;
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0) s->rz[it % 2] = rz;
-  if (it == 0) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-      p[i] = z[i];
+// p = z + beta p (p = z in the first iteration)
+__global__ void __launch_bounds__(256)
+k_sep_direction(double* __restrict__ p, const double* __restrict__ z, int64_t n, const Scalars* s,
+                int first) {
+  const int64_t step = (int64_t)gridDim.x * 256;
+  if (first) {
+    for (int64_t i = blockIdx.x * (int64_t)256 + threadIdx.x; i < n; i += step) p[i] = z[i];
     return;
   }
+  const double beta = s->beta;
 #pragma unroll 4
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
+  for (int64_t i = blockIdx.x * (int64_t)256 + threadIdx.x; i < n; i += step)
     p[i] = fma(beta, p[i], z[i]);
 }
 
-__global__ void __launch_bounds__(fe::RED_THREADS)
+// p.q; the last block takes alpha = r.z / p.q
+__global__ void __launch_bounds__(256)
 k_sep_dot(const double* __restrict__ p, const double* __restrict__ q, int64_t n,
-          double* __restrict__ part) {
+          double* __restrict__ part, Scalars* s) {
   double v = 0.0;
 #pragma unroll 4
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
+  for (int64_t i = blockIdx.x * (int64_t)256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256)
     v = fma(p[i], q[i], v);
   v = block_total(v);
   if (threadIdx.x == 0) part[blockIdx.x] = v;
+  if (last_block(&s->ticket[1], gridDim.x)) {
+    const double pq = sum_partials(part, gridDim.x);
+    if (threadIdx.x == 0) s->alpha = pq != 0.0 ? s->rz / pq : 0.0;
+  }
 }
 
-// alpha = r.z / p.q; phi += alpha p, r -= alpha q on free nodes (p is zero elsewhere);
-// partials of r.r
-__global__ void __launch_bounds__(fe::RED_THREADS)
+// phi += alpha p, r -= alpha q on free nodes (p is zero elsewhere); |r|^2
+__global__ void __launch_bounds__(256)
 k_sep_update(double* __restrict__ phi, double* __restrict__ r, const double* __restrict__ p,
              const double* __restrict__ q, const unsigned char* __restrict__ mask, int64_t n,
-             const double* __restrict__ part_pq, Scalars* s, int it,
-             double* __restrict__ part_rr) {
-  const double pq = sum_partials(part_pq, gridDim.x);
-  const double alpha = pq != 0.0 ? s->rz[it % 2] / pq : 0.0;
-  if (blockIdx.x == 0 && threadIdx.x == 0) s->alpha[it % 2] = alpha;
+             double* __restrict__ part, Scalars* s) {
+  const double alpha = s->alpha;
   double v = 0.0;
 #pragma unroll 4
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
+  for (int64_t i = blockIdx.x * (int64_t)256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
     phi[i] = fma(alpha, p[i], phi[i]);
     const double x = mask[i] ? 0.0 : fma(-alpha, q[i], r[i]);
     r[i] = x;
     v = fma(x, x, v);
   }
   v = block_total(v);
-  if (threadIdx.x == 0) part_rr[blockIdx.x] = v;
-}
-
-__global__ void __launch_bounds__(fe::RED_THREADS)
-k_sep_total(const double* __restrict__ part, int np, double* out) {
-  const double v = sum_partials(part, np);
-  if (threadIdx.x == 0) *out = v;
+  if (threadIdx.x == 0) part[blockIdx.x] = v;
+  if (last_block(&s->ticket[2], gridDim.x)) {
+    const double rr = sum_partials(part, gridDim.x);
+    if (threadIdx.x == 0) s->rr = rr;
+  }
 }
 
 // the largest chain the host eigensolver takes: about 9 n^3 flops after the mirror split
@@ -513,7 +605,7 @@ bool supported(const fe_mesh* m) {
 }
 
 size_t part_doubles(const fe_mesh* m) {
-  return 2 * (size_t)out_blocks(m->NZ * m->NY, m->NX) + 2 * VEC_BLOCKS + 16;
+  return 2 * (size_t)out_blocks(m->NZ * m->NY, m->NX) + VEC_BLOCKS + 16;
 }
 
 fe_status plan(fe_mesh* m, const double* cnt, bool constant_null) {
@@ -587,10 +679,9 @@ fe_status solve(fe_mesh* m, const Buf& b, double tol2, int maxit, double* rr, in
   t.lz = t.ly + NY;
   const int rows = nz * NY, np = out_blocks(rows, NX);
   double* part_z = b.part;
-  double* part_a = part_z + 2 * (size_t)np;
-  double* part_b = part_a + VEC_BLOCKS;
-  Scalars* s = reinterpret_cast<Scalars*>(part_b + VEC_BLOCKS);
-  double* total = reinterpret_cast<double*>(s + 1);
+  double* part = part_z + 2 * (size_t)np;
+  Scalars* s = reinterpret_cast<Scalars*>(part + VEC_BLOCKS);
+  FE_CUDA(cudaMemsetAsync(s, 0, sizeof(Scalars), st));
   // the constrained planes' entries of z and p stay zero
   FE_CUDA(cudaMemsetAsync(b.z, 0, sizeof(double) * n, st));
   const double rr0 = *rr;
@@ -610,10 +701,10 @@ fe_status solve(fe_mesh* m, const Buf& b, double tol2, int maxit, double* rr, in
     g = {};
     g.W = t.Vz; g.in = b.tb; g.out = b.ta; g.M = nz; g.N = (int)plane; g.K = nz;
     g.lx = t.lx; g.ly = t.ly; g.lz = t.lz; g.NX = NX; g.null_below = m->sep_null;
-    FE_TRY(gemm<LEFT_SCALE>(g, 1, st));
+    FE_TRY(gemm_z<LEFT_SCALE>(g, st));
     g = {};
     g.W = t.VzT; g.in = b.ta; g.out = b.tb; g.M = nz; g.N = (int)plane; g.K = nz;
-    FE_TRY(gemm<LEFT>(g, 1, st));
+    FE_TRY(gemm_z<LEFT>(g, st));
     g = {};
     g.W = t.VyT; g.in = b.tb; g.out = b.ta; g.M = NY; g.N = NX; g.K = NY;
     g.in_batch = g.out_batch = plane;
@@ -621,19 +712,17 @@ fe_status solve(fe_mesh* m, const Buf& b, double tol2, int maxit, double* rr, in
     g = {};
     g.W = t.VxT; g.in = b.ta; g.out_d = b.z + off; g.M = rows; g.N = NX; g.K = NX;
     g.mask = b.mask + off; g.r = b.r + off; g.q = it > 0 ? b.q + off : nullptr; g.part = part_z;
+    g.s = s; g.first = it == 0;
     FE_TRY(gemm<RIGHT_OUT>(g, 1, st));
-    k_sep_direction<<<VEC_BLOCKS, fe::RED_THREADS, 0, st>>>(b.p, b.z, n, part_z, np, s, it);
+    k_sep_direction<<<VEC_BLOCKS, 256, 0, st>>>(b.p, b.z, n, s, it == 0);
     fe_count_launch();
     FE_TRY(fe_poisson_apply_K(m, b.p, b.q));
-    k_sep_dot<<<VEC_BLOCKS, fe::RED_THREADS, 0, st>>>(b.p, b.q, n, part_a);
+    k_sep_dot<<<VEC_BLOCKS, 256, 0, st>>>(b.p, b.q, n, part, s);
     fe_count_launch();
-    k_sep_update<<<VEC_BLOCKS, fe::RED_THREADS, 0, st>>>(b.phi, b.r, b.p, b.q, b.mask, n, part_a,
-                                                             s, it, part_b);
-    fe_count_launch();
-    k_sep_total<<<1, fe::RED_THREADS, 0, st>>>(part_b, VEC_BLOCKS, total);
+    k_sep_update<<<VEC_BLOCKS, 256, 0, st>>>(b.phi, b.r, b.p, b.q, b.mask, n, part, s);
     fe_count_launch();
     FE_CUDA(cudaGetLastError());
-    FE_CUDA(cudaMemcpyAsync(rr, total, sizeof(double), cudaMemcpyDeviceToHost, st));
+    FE_CUDA(cudaMemcpyAsync(rr, &s->rr, sizeof(double), cudaMemcpyDeviceToHost, st));
     FE_CUDA(cudaStreamSynchronize(st));
     *iters = it + 1;
     // no progress over thirty iterations, or a breakdown: hand the solve back

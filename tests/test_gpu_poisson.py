@@ -360,6 +360,29 @@ def test_separable_preconditioner(fe, kind, p, ncell):
     assert e.value.status == fe._lib.FE_ENOCONV
 
 
+# z chains of 65 to 129 nodes on planes of 36 to 225 (tiles of 64 and 128 in the z products)
+@pytest.mark.parametrize("p,ncell", [(6, (1, 1, 11)), (4, (3, 3, 16)), (1, (11, 12, 64)), (5, (3, 3, 26))])
+@pytest.mark.parametrize("kind", ["cef", "cpd"])
+def test_separable_long_chains(fe, kind, p, ncell):
+    """The default solve on long cells against the oracle's direct one (bounds as above)."""
+    L = (2.0 * ncell[0], 2.0 * ncell[1], 1.5 * ncell[2])
+    bias = {"cef": W.Bias("cef", field=0.01), "cpd": W.Bias("cpd", dV=0.05, zA=0.0, zB=L[2])}[kind]
+    base = W.small_slab(ncell=ncell, p=p, L=L, natoms=3, seed=43)
+    slab = W.Slab(base.name, base.L, base.ncell, base.p, base.R, base.Z, bias)
+    om, K, M, X = _oracle(slab)
+    rho, b = potentials.densities(X, M, slab.R, slab.Z, slab.L)
+    vl = potentials.vloc_minus_vsm(X, slab.R, slab.Z, slab.L)
+    f = 4 * math.pi * M * (rho + b)
+    if kind == "cef":
+        ref = poisson.solve_cef_direct(K, f, M)
+    else:
+        mask, vals, _, _ = potentials.cpd_constraints(X, vl, bias, slab.L)
+        ref = poisson.solve_cpd_direct(K, f, mask, vals)
+    phi, _, info = fe.Mesh.from_slab(slab).poisson_solve(bias, rtol=1e-12)
+    assert info.status == 0 and info.rel_residual <= 1e-12 and info.iters <= 5
+    assert np.max(np.abs(phi.cpu().numpy() - ref)) <= 1e-9 * np.max(np.abs(ref))
+
+
 @pytest.mark.parametrize("ncell,p", [((33, 1, 2), 1), ((17, 2, 1), 2), ((16, 3, 2), 3), ((9, 2, 3), 4),
                                      ((8, 1, 2), 5), ((5, 3, 2), 6)])
 def test_apply_K_cell_strips(fe, ncell, p):
