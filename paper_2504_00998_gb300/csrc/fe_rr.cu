@@ -84,33 +84,50 @@ __global__ void k_symmetrize(double* __restrict__ S, int n) {
   }
 }
 
-// S = X^T X and (HX non-null) Hs = X^T HX of narrow double blocks (n <= 64 vectors, node-major):
-// block partials over a share of the rows, then their sums in block order (bitwise
-// repeatable).  Both products read X once.  FP64 issue bounds it (2 n^2 N FMAs, about 50 us for
-// 15,228 x 32); cuBLAS's SYRK takes one CTA for such an n (4.4 ms) and its split-K GEMM 107 us
-// for the second product.
-constexpr int GRAM_MAX = 64, GRAM_BLOCKS = 152, GRAM_ROWS = 16, GRAM_THREADS = 256;
+// S = X^T X (its upper triangle) and, where HX is given, Hs = X^T HX of double blocks
+// (node-major): a block takes one tile pair (I, J) of columns and a share of the rows, then the
+// partials are summed in a fixed order (bitwise repeatable).  FP64 issue bounds it: 15,228 x 32
+// 69 + 13 us for both products, where cuBLAS takes 4.4 ms for the SYRK (one block for such an
+// n) and 107 us for the GEMM.  A whole Rayleigh-Ritz of 389,120 nodes, with library Gram
+// products and with these: 32 vectors 116 and 4.4 ms, 64 124 and 12.5, 128 148 and 40, 256 227
+// and 140, 512 638 and 522, 1024 2464 and 1994; 15,228 nodes: 128 11.9 and 7.7, 1024 141 and 122.
+constexpr int GRAM_BLOCKS = 608, GRAM_ROWS = 16, GRAM_THREADS = 256;
 
-// MB x MB entries of S and of Hs a thread: entry (ti + 16 a, tj + 16 b)
-template <int MB>
-__global__ void __launch_bounds__(GRAM_THREADS)
-k_gram_partial(const double* __restrict__ X, int64_t ld, const double* __restrict__ HX, int64_t ldh,
-               int n, int64_t N, double* __restrict__ part) {
+// Tile width / 16: the narrowest tile that holds n, else 48 or 64 columns, whichever pads less.
+int gram_mb(int n) {
+  if (n <= 64) return (n + 15) / 16;
+  return (n + 47) / 48 * 48 < (n + 63) / 64 * 64 ? 3 : 4;
+}
+// row shares of a tile pair: about GRAM_BLOCKS blocks in all, at least 32 rows a share
+int gram_shares(int tiles, int64_t N) {
+  const int64_t most = std::max<int64_t>(1, N / 32), want = (GRAM_BLOCKS + tiles * tiles - 1) / (tiles * tiles);
+  return (int)std::min(most, want);
+}
+
+// MB x MB entries of S and of Hs a thread: entry (ti + 16 a, tj + 16 b) of the tile pair.  A
+// diagonal tile skips the entries a > b, which are below the diagonal.
+template <int MB, bool S, bool H, bool DIAG>
+__device__ __forceinline__ void gram_share(const double* __restrict__ X, int64_t ld,
+                                           const double* __restrict__ HX, int64_t ldh, int n, int i0,
+                                           int j0, int64_t r0, int64_t r1,
+                                           double (*__restrict__ xs)[16 * MB],
+                                           double (*__restrict__ ys)[16 * MB],
+                                           double (*__restrict__ hs)[16 * MB], double* __restrict__ ps) {
   constexpr int W = 16 * MB;
-  __shared__ double xs[GRAM_ROWS][W], hs[GRAM_ROWS][W];
   const int tid = threadIdx.x, ti = tid / 16, tj = tid % 16;
-  const int64_t r0 = N * blockIdx.x / gridDim.x, r1 = N * (blockIdx.x + 1) / gridDim.x;
   double s[MB][MB], h[MB][MB];
 #pragma unroll
   for (int a = 0; a < MB; ++a)
 #pragma unroll
     for (int b = 0; b < MB; ++b) s[a][b] = h[a][b] = 0.0;
   for (int64_t r = r0; r < r1; r += GRAM_ROWS) {
-    for (int e = tid; e < GRAM_ROWS * W; e += GRAM_THREADS) {
-      const int row = e / W, c = e - row * W;
-      const bool in = r + row < r1 && c < n;
-      xs[row][c] = in ? X[(r + row) * ld + c] : 0.0;
-      hs[row][c] = in && HX ? HX[(r + row) * ldh + c] : 0.0;
+#pragma unroll
+    for (int k = 0; k < MB; ++k) {   // (16 x W entries: MB a thread)
+      const int e = tid + k * GRAM_THREADS, row = e / W, c = e - row * W;
+      const bool in = r + row < r1;
+      xs[row][c] = in && i0 + c < n ? X[(r + row) * ld + i0 + c] : 0.0;
+      if constexpr (S && !DIAG) ys[row][c] = in && j0 + c < n ? X[(r + row) * ld + j0 + c] : 0.0;
+      if constexpr (H) hs[row][c] = in && j0 + c < n ? HX[(r + row) * ldh + j0 + c] : 0.0;
     }
     __syncthreads();
 #pragma unroll 4
@@ -119,41 +136,72 @@ k_gram_partial(const double* __restrict__ X, int64_t ld, const double* __restric
 #pragma unroll
       for (int a = 0; a < MB; ++a) {
         xi[a] = xs[row][ti + 16 * a];
-        xj[a] = xs[row][tj + 16 * a];
-        hj[a] = hs[row][tj + 16 * a];
+        if constexpr (S) xj[a] = DIAG ? xs[row][tj + 16 * a] : ys[row][tj + 16 * a];
+        if constexpr (H) hj[a] = hs[row][tj + 16 * a];
       }
 #pragma unroll
       for (int a = 0; a < MB; ++a)
 #pragma unroll
         for (int b = 0; b < MB; ++b) {
-          s[a][b] = fma(xi[a], xj[b], s[a][b]);
-          if (HX) h[a][b] = fma(xi[a], hj[b], h[a][b]);
+          if (S && !(DIAG && a > b)) s[a][b] = fma(xi[a], xj[b], s[a][b]);
+          if constexpr (H) h[a][b] = fma(xi[a], hj[b], h[a][b]);
         }
     }
     __syncthreads();
   }
-  double* ps = part + (int64_t)blockIdx.x * 2 * n * n;
 #pragma unroll
   for (int a = 0; a < MB; ++a)
 #pragma unroll
     for (int b = 0; b < MB; ++b) {
-      const int i = ti + 16 * a, j = tj + 16 * b;
+      const int i = i0 + ti + 16 * a, j = j0 + tj + 16 * b;
       if (i >= n || j >= n) continue;
-      ps[(int64_t)j * n + i] = s[a][b];
-      if (HX) ps[(int64_t)n * n + (int64_t)j * n + i] = h[a][b];
+      if (S && !(DIAG && a > b)) ps[(int64_t)j * n + i] = s[a][b];
+      if constexpr (H) ps[(int64_t)n * n + (int64_t)j * n + i] = h[a][b];
     }
 }
 
-// entry e of the two matrices: its block partials in order, four chains
-__global__ void k_gram_sum(const double* __restrict__ part, int blocks, int64_t nn, int two,
-                           double* __restrict__ S, double* __restrict__ Hs) {
-  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (e >= nn * (two ? 2 : 1)) return;
-  double t[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int b = 0; b < blocks; ++b) t[b & 3] += part[(int64_t)b * 2 * nn + e];
-  const double v = (t[0] + t[1]) + (t[2] + t[3]);
+template <int MB, bool H>
+__global__ void __launch_bounds__(GRAM_THREADS, 2)
+k_gram_partial(const double* __restrict__ X, int64_t ld, const double* __restrict__ HX, int64_t ldh,
+               int n, int tiles, int64_t N, double* __restrict__ part) {
+  __shared__ double xs[GRAM_ROWS][16 * MB], ys[GRAM_ROWS][16 * MB], hs[H ? GRAM_ROWS : 1][16 * MB];
+  const int I = blockIdx.y % tiles, J = blockIdx.y / tiles;
+  const int i0 = I * 16 * MB, j0 = J * 16 * MB;
+  const int64_t r0 = N * blockIdx.x / gridDim.x, r1 = N * (blockIdx.x + 1) / gridDim.x;
+  double* ps = part + (int64_t)blockIdx.x * (H ? 2 : 1) * n * n;
+  if (I == J) gram_share<MB, true, H, true>(X, ld, HX, ldh, n, i0, j0, r0, r1, xs, ys, hs, ps);
+  else if (I < J) gram_share<MB, true, H, false>(X, ld, HX, ldh, n, i0, j0, r0, r1, xs, ys, hs, ps);
+  else if constexpr (H) gram_share<MB, false, true, false>(X, ld, HX, ldh, n, i0, j0, r0, r1, xs, ys, hs, ps);
+}
+
+// entry e of the two matrices: its partials in eight interleaved chains, added in order (the
+// part of S below the diagonal is not formed)
+__global__ void __launch_bounds__(256)
+k_gram_sum(const double* __restrict__ part, int shares, int n, int64_t entries,
+           double* __restrict__ S, double* __restrict__ Hs) {
+  __shared__ double t[8][32];
+  const int lane = threadIdx.x % 32, chain = threadIdx.x / 32;
+  const int64_t nn = (int64_t)n * n, e = blockIdx.x * (int64_t)32 + lane;
+  const bool on = e < entries && (e >= nn || e % n <= e / n);
+  double v = 0.0;
+  if (on)
+    for (int b = chain; b < shares; b += 8) v += part[(int64_t)b * entries + e];
+  t[chain][lane] = v;
+  __syncthreads();
+  if (chain || !on) return;
+#pragma unroll
+  for (int k = 1; k < 8; ++k) v += t[k][lane];
   if (e < nn) S[e] = v;
   else Hs[e - nn] = v;
+}
+
+template <int MB>
+void gram_launch(const double* X, int64_t ld, const double* HX, int64_t ldh, int n, int64_t N,
+                 int shares, double* part, cudaStream_t st) {
+  const int tiles = (n + 16 * MB - 1) / (16 * MB);
+  const dim3 grid(shares, tiles * tiles);
+  if (HX) k_gram_partial<MB, true><<<grid, GRAM_THREADS, 0, st>>>(X, ld, HX, ldh, n, tiles, N, part);
+  else k_gram_partial<MB, false><<<grid, GRAM_THREADS, 0, st>>>(X, ld, nullptr, 0, n, tiles, N, part);
 }
 
 struct RrWs {
@@ -175,22 +223,20 @@ fe_status gram(fe_mesh* m, const double* A, int64_t lda, const double* B, int64_
 fe_status gram_pair(fe_mesh* m, const double* X, int64_t ld, const double* HX, int64_t ldh,
                     int64_t nvec, double* S, double* Hs) {
   const int n = (int)nvec;
+  const int mb = gram_mb(n), shares = gram_shares((n + 16 * mb - 1) / (16 * mb), m->n_psi);
+  const int64_t entries = (Hs ? 2 : 1) * nvec * nvec;
   void* part = nullptr;
-  fe_status st = FE_ENOMEM;
-  if (n <= GRAM_MAX) st = fe_ws(m, WS_RR_TC32, sizeof(double) * 2 * (size_t)n * n * GRAM_BLOCKS, &part);
+  const fe_status st = fe_ws(m, WS_RR_TC32, sizeof(double) * (size_t)entries * shares, &part);
   if (st != FE_OK && st != FE_ENOMEM) return st;
   if (st == FE_OK) {   // (without room for the partials: the library products)
     double* p = (double*)part;
     const double* hx = Hs ? HX : nullptr;
-    if (n <= 16)
-      k_gram_partial<1><<<GRAM_BLOCKS, GRAM_THREADS, 0, m->stream>>>(X, ld, hx, ldh, n, m->n_psi, p);
-    else if (n <= 32)
-      k_gram_partial<2><<<GRAM_BLOCKS, GRAM_THREADS, 0, m->stream>>>(X, ld, hx, ldh, n, m->n_psi, p);
-    else
-      k_gram_partial<4><<<GRAM_BLOCKS, GRAM_THREADS, 0, m->stream>>>(X, ld, hx, ldh, n, m->n_psi, p);
+    if (mb == 1) gram_launch<1>(X, ld, hx, ldh, n, m->n_psi, shares, p, m->stream);
+    else if (mb == 2) gram_launch<2>(X, ld, hx, ldh, n, m->n_psi, shares, p, m->stream);
+    else if (mb == 3) gram_launch<3>(X, ld, hx, ldh, n, m->n_psi, shares, p, m->stream);
+    else gram_launch<4>(X, ld, hx, ldh, n, m->n_psi, shares, p, m->stream);
     fe_count_launch();
-    const int64_t nn = (int64_t)n * n;
-    k_gram_sum<<<(unsigned)((2 * nn + 127) / 128), 128, 0, m->stream>>>(p, GRAM_BLOCKS, nn, Hs != nullptr, S, Hs);
+    k_gram_sum<<<(unsigned)((entries + 31) / 32), 256, 0, m->stream>>>(p, shares, n, entries, S, Hs);
     fe_count_launch();
     FE_CUDA(cudaGetLastError());
     return FE_OK;

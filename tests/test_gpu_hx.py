@@ -294,10 +294,10 @@ def test_sweep_tile_edges(fe, p, ncell, nvec):
         assert_column_maxabs(Xg.double().cpu().numpy(), ref, ftol, "filter")
 
 
-@pytest.mark.parametrize("n", [1, 15, 16, 17, 32, 33, 64, 65])
+@pytest.mark.parametrize("n", [1, 15, 16, 17, 32, 33, 48, 49, 64, 65, 96, 97, 130, 200])
 def test_rayleigh_ritz_gram_sizes(fe, n):
-    """Double Rayleigh-Ritz at the edges of the narrow Gram kernel (tiles of 16, 32 and 64
-    vectors, library products above), rows padded past the block; bounds as above."""
+    """Double Rayleigh-Ritz at the edges of the Gram kernel's tiles (16, 32, 48 and 64 columns,
+    pairs of tiles above), rows padded past the block; bounds as above."""
     om, H, m, rng = _setup(fe, (4.0, 4.0, 9.0), (2, 2, 4), 3, (True, True), seed=n)
     X = rng.standard_normal((om.n_psi, n))
     lam_ref, _ = chefsi.rayleigh_ritz(lambda Z: H @ Z, X)
