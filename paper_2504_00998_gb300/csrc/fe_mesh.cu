@@ -395,9 +395,15 @@ extern "C" fe_status fe_lumped_mass(const fe_mesh* m, double* out) {
   return FE_OK;
 }
 
-__global__ void k_d2f(const double* __restrict__ a, float* __restrict__ b, int64_t n) {
+// both copies of the potential in one launch
+__global__ void k_set_potential(const double* __restrict__ v, double* __restrict__ d,
+                                float* __restrict__ f, int64_t n) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < n) b[i] = (float)a[i];
+  if (i < n) {
+    const double x = v[i];
+    d[i] = x;
+    f[i] = (float)x;
+  }
 }
 
 extern "C" fe_status fe_set_potential(fe_mesh* m, const double* veff) {
@@ -410,10 +416,8 @@ extern "C" fe_status fe_set_potential(fe_mesh* m, const double* veff) {
       return fe_fail(FE_ENOMEM, "potential allocation failed");
     }
   }
-  FE_CUDA(cudaMemcpyAsync(m->d_veff, veff, m->n_psi * sizeof(double), cudaMemcpyDeviceToDevice,
-                          m->stream));
   int nb = (int)((m->n_psi + 255) / 256);
-  k_d2f<<<nb, 256, 0, m->stream>>>(m->d_veff, m->d_veff_f, m->n_psi); fe_count_launch();
+  k_set_potential<<<nb, 256, 0, m->stream>>>(veff, m->d_veff, m->d_veff_f, m->n_psi); fe_count_launch();
   FE_CUDA(cudaGetLastError());
   m->has_potential = true;
   m->has_quad = false;   // back to the collocated potential

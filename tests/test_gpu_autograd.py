@@ -213,6 +213,32 @@ def test_hamiltonian_autograd(fe, ag, prec):
                 assert abs(fd_x - an_x) <= 1e-6 * abs(an_x)
 
 
+@pytest.mark.parametrize("nvec", [1, 3, 4, 7, 127, 128, 131])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_potential_vjp_aligned_and_unaligned(fe, nvec, offset):
+    """The float row sums on rows with and without 16-byte alignment, with zeros, subnormals and
+    non-finite entries.  Products of floats are exact in double, so the bound is nvec roundings
+    of the sum of magnitudes."""
+    m = fe.Mesh((4.0, 4.0, 9.0), (2, 2, 4), 3)
+    rng = np.random.default_rng(53)
+    ld = -(-(nvec + 1) // 4) * 4
+
+    def block():
+        a = (rng.standard_normal((m.n_psi, ld)) * 10.0 ** rng.uniform(-30, 8, (m.n_psi, ld))).astype(np.float32)
+        a[3::7, :] = 0.0
+        a[4::7, :] *= np.float32(1e-14)
+        return torch.tensor(a, device="cuda")[:, offset:offset + nvec]
+    X, Y = block(), block()
+    g = m.potential_vjp(X, Y, prec=fe.FE_F32).cpu()
+    prod = X.double().cpu() * Y.double().cpu()
+    bound = nvec * 2.0 ** -52 * prod.abs().sum(1)
+    assert torch.all((g - prod.sum(1)).abs() <= bound)
+    X[5, 0], X[6, nvec - 1], Y[6, nvec - 1] = math.inf, math.nan, 1.0
+    Y[5, 0] = -2.0
+    g = m.potential_vjp(X, Y, prec=fe.FE_F32).cpu()
+    assert g[5] == -math.inf and torch.isnan(g[6])
+
+
 def test_hamiltonian_autograd_bloch(fe, ag):
     """Complex blocks at a Bloch wave vector: dL/dX = Ht_k Ybar (Hermitian) and
     dL/dV = Re sum_v Ybar conj(X), checked by central differences along real V and complex
