@@ -7,11 +7,11 @@
 // the arithmetic is kept short.  With the GLL weights W taken out, K1 = W K', and the exact
 // mass is M1 = W P with P = 1 - s q^T: it differs from the GLL rule in the L_p . L_p product
 // only (q_k = w_k P_p(x_k), s_j = p (p + 1) / (2 (2 p + 1)) P_p(x_j)), so a mass line costs a dot
-// product and an update.  A cell product is then 168 double operations a line triple (at p = 5)
-// where dense mass lines take 252, and it has no halo: 160 + 16 us a product on the
-// 16 x 16 x 48-cell p = 5 slab (1.54 M nodes, 48 operations a node, 0.87 of the FP64 rate that a
-// DGEMM reaches), where the sweep kernel, with its halo columns, segment overlap and idle
-// lanes, takes 377 us.
+// product and an update, and it has no halo.  Even p: 168 double operations a line triple where
+// dense mass lines take 252 (at p = 5).  Odd p: the mirror parts below, 120 operations.  A product
+// on the 16 x 16 x 48-cell p = 5 slab (1.54 M nodes) takes 129 + 16 us (160 + 16 without the
+// mirror parts; 377 in the sweep kernel, with its halo columns, segment overlap and idle
+// lanes).
 #include <cstdint>
 
 #include "fe_internal.h"
@@ -140,6 +140,194 @@ k_cell64_apply(const Cell64 cf, const double* __restrict__ x, double* __restrict
   }
 }
 
+// ---- odd p: mirror parts ------------------------------------------------------------------------
+// K' commutes with the mirror image of a cell and q, s are odd, so a line of p + 1 values is
+// kept as its (p + 1) / 2 even parts u_k + u_{p-k} (at k) and its odd ones u_k - u_{p-k} (at p - k):
+// a stiffness line then takes half the operations and a mass line too.  In the three directions
+// the parts are taken and put back once: a thread of the y and the z pass has the four mirror
+// images of a line.  (Even p has a middle line without an image, which would leave those threads
+// a third idle: 5 x 5 lines are 9 quadruples.)
+template <int P>
+struct Mirror {
+  static constexpr int N1 = P + 1, H = N1 / 2;
+  static constexpr int CX = P == 1 ? 64 : P == 3 ? 16 : 7;   // cells a block: two whole warps
+  static constexpr int QUADS = CX * H * H, NTHR = (QUADS + 31) / 32 * 32;
+  static constexpr int NODES = CX * N1 * N1 * N1, ROWS = CX * N1 * N1;
+  static_assert(P % 2 == 1, "no middle node");
+};
+
+constexpr int MAXH = FE_MAXN1 / 2;
+struct Mirror64 {
+  double Kx[2][MAXH][MAXH], Ky[2][MAXH][MAXH], Kz[2][MAXH][MAXH];   // even, odd parts
+  double q[MAXH], s[MAXH], w[MAXH];
+};
+
+Mirror64 mirror64(const Cell64& c, int p) {
+  Mirror64 t = {};
+  for (int j = 0; j < (p + 1) / 2; ++j) {
+    t.q[j] = 2.0 * c.q[j];
+    t.s[j] = c.s[j];
+    t.w[j] = c.w[j];
+    for (int k = 0; k < (p + 1) / 2; ++k)
+      for (int o = 0; o < 2; ++o) {
+        t.Kx[o][j][k] = o ? c.Kx[j][k] - c.Kx[j][p - k] : c.Kx[j][k] + c.Kx[j][p - k];
+        t.Ky[o][j][k] = o ? c.Ky[j][k] - c.Ky[j][p - k] : c.Ky[j][k] + c.Ky[j][p - k];
+        t.Kz[o][j][k] = o ? c.Kz[j][k] - c.Kz[j][p - k] : c.Kz[j][k] + c.Kz[j][p - k];
+      }
+  }
+  return t;
+}
+
+// out += K in
+template <int P>
+__device__ __forceinline__ void mirror_k(const double (&K)[2][MAXH][MAXH], const double (&in)[P + 1],
+                                         double (&out)[P + 1]) {
+#pragma unroll
+  for (int j = 0; j < (P + 1) / 2; ++j)
+#pragma unroll
+    for (int k = 0; k < (P + 1) / 2; ++k) {
+      out[j] = fma(K[0][j][k], in[k], out[j]);
+      out[P - j] = fma(K[1][j][k], in[P - k], out[P - j]);
+    }
+}
+// the mass of in, in place: the odd parts only
+template <int P>
+__device__ __forceinline__ void mirror_mass(const Mirror64& cf, double (&in)[P + 1]) {
+  double d = 0.0;
+#pragma unroll
+  for (int k = 0; k < (P + 1) / 2; ++k) d = fma(cf.q[k], in[P - k], d);
+#pragma unroll
+  for (int k = 0; k < (P + 1) / 2; ++k) in[P - k] = fma(-cf.s[k], d, in[P - k]);
+}
+
+template <int P>
+__global__ void __launch_bounds__(Mirror<P>::NTHR)
+k_cell64_mirror(const Mirror64 cf, const double* __restrict__ x, double* __restrict__ ycell, int nx,
+                int ny, int cells, int NX, int NY) {
+  using M = Mirror<P>;
+  constexpr int N1 = M::N1, CX = M::CX, H = M::H, NT = M::NTHR;
+  __shared__ double A[M::NODES];   // [lz][ly][cell][lx]: the nodes, then A
+  __shared__ double B[M::NODES];
+  __shared__ int at[3][CX];        // the cells' indices (the last cell again past the end)
+  const int tid = threadIdx.x, first = blockIdx.x * CX;
+  for (int c = tid; c < CX; c += NT) {
+    const int id = min(first + c, cells - 1), row = id / nx;
+    at[0][c] = id - row * nx;
+    at[2][c] = row / ny;
+    at[1][c] = row - at[2][c] * ny;
+  }
+  __syncthreads();
+#pragma unroll 8
+  for (int e = tid; e < M::NODES; e += NT) {
+    const int lx = e % N1, c = (e / N1) % CX, ly = (e / (N1 * CX)) % N1, lz = e / (N1 * CX * N1);
+    int gx = at[0][c] * P + lx, gy = at[1][c] * P + ly;
+    gx -= gx >= NX ? NX : 0;
+    gy -= gy >= NY ? NY : 0;
+    A[e] = x[((int64_t)(at[2][c] * P + lz) * NY + gy) * NX + gx];
+  }
+  __syncthreads();
+  const int k0 = tid % H, cell = (tid / H) % CX, k1 = tid / (H * CX);
+  // y lines, the mirror images in x and z: to parts in three directions (eight times the
+  // parts), then A = P u, B = Ky u
+  if (tid < M::QUADS) {
+    double* a = A + cell * N1;
+    double* b = B + cell * N1;
+    double in[4][N1];   // 2 (odd in z) + (odd in x)
+#pragma unroll
+    for (int k = 0; k < N1; ++k) {
+      const double* lo = a + (k1 * N1 + k) * CX * N1;
+      const double* hi = a + ((P - k1) * N1 + k) * CX * N1;
+      const double e0 = lo[k0] + lo[P - k0], o0 = lo[k0] - lo[P - k0];
+      const double e1 = hi[k0] + hi[P - k0], o1 = hi[k0] - hi[P - k0];
+      in[0][k] = e0 + e1;
+      in[1][k] = o0 + o1;
+      in[2][k] = e0 - e1;
+      in[3][k] = o0 - o1;
+    }
+#pragma unroll
+    for (int l = 0; l < 4; ++l) {
+      const int o = (l & 2 ? P - k1 : k1) * N1 * CX * N1 + (l & 1 ? P - k0 : k0);
+      double u[N1], v[N1];
+#pragma unroll
+      for (int k = 0; k < H; ++k) {
+        u[k] = in[l][k] + in[l][P - k];
+        u[P - k] = in[l][k] - in[l][P - k];
+        v[k] = v[P - k] = 0.0;
+      }
+      mirror_k<P>(cf.Ky, u, v);
+      mirror_mass<P>(cf, u);
+#pragma unroll
+      for (int j = 0; j < N1; ++j) {
+        a[o + j * CX * N1] = u[j];
+        b[o + j * CX * N1] = v[j];
+      }
+    }
+  }
+  __syncthreads();
+  // x lines, in place: A <- P a, B <- Kx a + P b
+  for (int r = tid; r < M::ROWS; r += NT) {
+    double a[N1], b[N1];
+#pragma unroll
+    for (int k = 0; k < N1; ++k) {
+      a[k] = A[r * N1 + k];
+      b[k] = B[r * N1 + k];
+    }
+    mirror_mass<P>(cf, b);
+    mirror_k<P>(cf.Kx, a, b);
+    mirror_mass<P>(cf, a);
+#pragma unroll
+    for (int k = 0; k < N1; ++k) {
+      A[r * N1 + k] = a[k];
+      B[r * N1 + k] = b[k];
+    }
+  }
+  __syncthreads();
+  // z lines, the mirror images in x and y: y_e = W (x) W (x) W (Kz A + P B), back to nodal
+  // values, to the discontinuous grid
+  if (tid < M::QUADS && first + cell < cells) {
+    double r[4][N1];   // 2 (odd in y) + (odd in x)
+#pragma unroll
+    for (int l = 0; l < 4; ++l) {
+      const int o = ((l & 2 ? P - k1 : k1) * CX + cell) * N1 + (l & 1 ? P - k0 : k0);
+      double u[N1], v[N1];
+#pragma unroll
+      for (int k = 0; k < N1; ++k) {
+        u[k] = A[o + k * N1 * CX * N1];
+        v[k] = B[o + k * N1 * CX * N1];
+      }
+      mirror_mass<P>(cf, v);
+      mirror_k<P>(cf.Kz, u, v);
+#pragma unroll
+      for (int k = 0; k < H; ++k) {
+        r[l][k] = v[k] + v[P - k];
+        r[l][P - k] = v[k] - v[P - k];
+      }
+    }
+    double w0 = 0.0, w1 = 0.0;
+#pragma unroll
+    for (int k = 0; k < H; ++k) {
+      w0 = k == k0 ? cf.w[k] : w0;
+      w1 = k == k1 ? cf.w[k] : w1;
+    }
+    const double wxy = 0.125 * (w0 * w1);
+    const int64_t dnx = (int64_t)nx * N1, dny = (int64_t)ny * N1;
+    double* out = ycell + ((int64_t)at[2][cell] * N1 * dny + (int64_t)at[1][cell] * N1) * dnx +
+                  (int64_t)at[0][cell] * N1;
+#pragma unroll
+    for (int j = 0; j < N1; ++j) {
+      const double w = wxy * cf.w[j < H ? j : P - j];
+      const double e0 = r[0][j] + r[1][j], e1 = r[0][j] - r[1][j];
+      const double o0 = r[2][j] + r[3][j], o1 = r[2][j] - r[3][j];
+      double* lo = out + (j * dny + k1) * dnx;
+      double* hi = out + (j * dny + P - k1) * dnx;
+      lo[k0] = w * (e0 + o0);
+      lo[P - k0] = w * (e1 + o1);
+      hi[k0] = w * (e0 - o0);
+      hi[P - k0] = w * (e1 - o1);
+    }
+  }
+}
+
 // y at node (gx, gy, gz): the sum of its one to eight copies, lower cells first
 template <int P>
 __global__ void __launch_bounds__(256)
@@ -178,8 +366,15 @@ template <int P>
 fe_status run(fe_mesh* m, const double* x, double* y, double* yc) {
   using S = CellStrip<P>;
   const Cell64 cf = cell64(m);
-  k_cell64_apply<P><<<dim3((m->nx + S::CX - 1) / S::CX, m->ny, m->nz), S::NTHR, 0, m->stream>>>(
-      cf, x, yc, m->nx, m->ny, m->NX, m->NY);
+  if constexpr (P % 2) {
+    using M = Mirror<P>;
+    const int cells = m->nx * m->ny * m->nz;
+    k_cell64_mirror<P><<<(cells + M::CX - 1) / M::CX, M::NTHR, 0, m->stream>>>(
+        mirror64(cf, P), x, yc, m->nx, m->ny, cells, m->NX, m->NY);
+  } else {
+    k_cell64_apply<P><<<dim3((m->nx + S::CX - 1) / S::CX, m->ny, m->nz), S::NTHR, 0, m->stream>>>(
+        cf, x, yc, m->nx, m->ny, m->NX, m->NY);
+  }
   fe_count_launch();
   k_cell64_gather<P><<<dim3((m->NX + 31) / 32, (m->NY + 7) / 8, m->NZ < 65535 ? m->NZ : 65535),
                        dim3(32, 8), 0, m->stream>>>(yc, y, m->nx, m->ny, m->nz, m->NX, m->NY);

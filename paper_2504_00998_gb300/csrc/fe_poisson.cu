@@ -137,23 +137,26 @@ __global__ void k_setup(PGeom g, fe_poisson_bc bc, const double* __restrict__ ma
   }
 }
 
-// Block sums in a fixed order (so every reduction is reproducible): a shuffle tree inside
-// each warp, then every warp reduces the per-warp sums the same way.  blockDim.x is a multiple
-// of 32 (at most 1024); every thread receives the total; one barrier per call (two with the
-// barrier that lets a later call reuse the staging array).
+// Block sums in a fixed order (so every reduction is reproducible).  blockDim.x is a multiple of
+// 32 (at most 1024); every thread receives the total.  An FP64 add of a warp starts every
+// sixteen cycles an SM, so the sum over the warps is one warp's work, column by column.
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
   return v;
 }
 __device__ __forceinline__ double block_sum(double v) {
-  __shared__ double ws[32];
-  v = warp_sum(v);
-  const int lane = threadIdx.x & 31;
-  if (lane == 0) ws[threadIdx.x >> 5] = v;
+  __shared__ double ws[1024];
+  ws[threadIdx.x] = v;
   __syncthreads();
-  double t = lane < (int)(blockDim.x >> 5) ? ws[lane] : 0.0;
-  t = __shfl_sync(0xffffffffu, warp_sum(t), 0);
+  if (threadIdx.x < 32) {
+    double t = v;
+    for (int w = threadIdx.x + 32; w < (int)blockDim.x; w += 32) t += ws[w];
+    t = warp_sum(t);
+    if (threadIdx.x == 0) ws[0] = t;
+  }
+  __syncthreads();
+  const double t = ws[0];
   __syncthreads();
   return t;
 }
@@ -175,11 +178,31 @@ template <typename V>
 __global__ void k_psum(const V* __restrict__ x, const V* __restrict__ y, int64_t n,
                        double* __restrict__ part) {
   V s = V(0);   // a thread's few terms in the vector precision, the block sum in double
+#pragma unroll 4
   for (int64_t i = blockIdx.x * (int64_t)fe::RED_THREADS + threadIdx.x; i < n;
        i += (int64_t)fe::RED_BLOCKS * fe::RED_THREADS)
     s += y ? x[i] * y[i] : x[i];
   const double t = block_sum((double)s);
   if (threadIdx.x == 0) part[blockIdx.x] = t;
+}
+
+// part_a: partial sums of x (y == nullptr) or x.y; part_b: of w
+__global__ void __launch_bounds__(fe::RED_THREADS)
+k_psum_pair(const double* __restrict__ x, const double* __restrict__ y, const double* __restrict__ w,
+            int64_t n, double* __restrict__ part_a, double* __restrict__ part_b) {
+  double a = 0.0, b = 0.0;
+#pragma unroll 4
+  for (int64_t i = blockIdx.x * (int64_t)fe::RED_THREADS + threadIdx.x; i < n;
+       i += (int64_t)fe::RED_BLOCKS * fe::RED_THREADS) {
+    a = y ? fma(x[i], y[i], a) : a + x[i];
+    b += w[i];
+  }
+  a = block_sum(a);
+  b = block_sum(b);
+  if (threadIdx.x == 0) {
+    part_a[blockIdx.x] = a;
+    part_b[blockIdx.x] = b;
+  }
 }
 
 __device__ double block_sum_partials(const double* part) {
@@ -208,7 +231,7 @@ __global__ void k_resid0(const double* __restrict__ f, const double* __restrict_
                          int64_t n) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
-    r[i] = mask[i] ? 0.0 : f[i] - kphi[i];
+    r[i] = mask[i] ? 0.0 : kphi ? f[i] - kphi[i] : f[i];
 }
 
 __global__ void k_fin_mean(const double* part, CgState* s, double inv_n) {
@@ -382,18 +405,30 @@ __global__ void k_shift_mean(double* __restrict__ phi, const double* part_mphi,
     phi[i] -= c;
 }
 
-// V_eff at psi nodes: phi + (V_loc - V_sm) + V_app
-__global__ void k_vbare(PGeom g, const double* __restrict__ phi, const double* __restrict__ vlms,
-                        VApp va, int cef, int gz_lo, double* __restrict__ out, int64_t npsi) {
-  int64_t off = (int64_t)gz_lo * g.NX * g.NY;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < npsi;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    int64_t id = i + off;
-    int gz = (int)((uint32_t)id / ((uint32_t)g.NX * (uint32_t)g.NY));
-    double v = phi[id] + vlms[id];
-    if (cef) v += vapp(va, zcoord(g, gz));
-    out[i] = v;
+// V_bare at the nodes of planes gz_lo to gz_lo + planes - 1: phi + (V_loc - V_sm) + V_app (cef).
+// A thread takes four nodes of a plane: the coordinate and V_app are a dozen FP64 operations,
+// which bounded the kernel at one node a thread (40 us on the benchmark slab, now 20).
+__global__ void __launch_bounds__(256)
+k_vbare(PGeom g, const double* __restrict__ phi, const double* __restrict__ vlms, VApp va, int cef,
+        int gz_lo, int planes, double* __restrict__ out) {
+  const int plane = g.NX * g.NY, at = blockIdx.x * 1024 + threadIdx.x;
+  for (int k = blockIdx.y; k < planes; k += gridDim.y) {
+    const int64_t to = (int64_t)k * plane, from = (int64_t)(gz_lo + k) * plane;
+    const double v = cef ? vapp(va, zcoord(g, gz_lo + k)) : 0.0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int i = at + 256 * u;
+      if (i >= plane) continue;
+      const double t = phi[from + i] + vlms[from + i];
+      out[to + i] = cef ? t + v : t;
+    }
   }
+}
+void launch_vbare(fe_mesh* m, const PGeom& g, const double* phi, const VApp& va, int cef, int gz_lo,
+                  int planes, double* out) {
+  const dim3 grid((unsigned)((g.NX * (int64_t)g.NY + 1023) / 1024), (unsigned)std::min(planes, 65535));
+  k_vbare<<<grid, 256, 0, m->stream>>>(g, phi, m->d_vlms, va, cef, gz_lo, planes, out);
+  fe_count_launch();
 }
 
 // ---- z-plane coarse space ---------------------------------------------------------------
@@ -1188,10 +1223,8 @@ extern "C" fe_status fe_vbare_phi(fe_mesh* m, const double* phi, const fe_poisso
   if (!m || !phi || !bc || !out) return fe_fail(FE_EINVAL, "fe_vbare_phi: null argument");
   if (!m->d_vlms) return fe_fail(FE_EINVAL, "fe_vbare_phi: call fe_set_atoms first");
   FE_TRY(fe_activate(m));
-  k_vbare<<<fe::grid_for(m->n_phi), 256, 0, m->stream>>>(make_geom(m), phi, m->d_vlms,
-                                                           make_vapp(bc->field, m->desc.L[2]),
-                                                           bc->kind == FE_BIAS_CEF, 0, out,
-                                                           m->n_phi); fe_count_launch();
+  launch_vbare(m, make_geom(m), phi, make_vapp(bc->field, m->desc.L[2]), bc->kind == FE_BIAS_CEF, 0,
+               m->NZ, out);
   FE_CUDA(cudaGetLastError());
   return FE_OK;
 }
@@ -1546,8 +1579,7 @@ static fe_status poisson_solve_on(fe_mesh* m, const double* rho, const fe_poisso
   k_setup<<<gb, 256, 0, st>>>(g, *bc, m->d_mass, rh, m->d_b, m->d_vlms, f_ext, phic_ext, f,
                               separable ? nullptr : dinv, mask, phi, n); fe_count_launch();
   if (project) {
-    k_psum<double><<<fe::RED_BLOCKS, fe::RED_THREADS, 0, st>>>(f, nullptr, n, pa); fe_count_launch();
-    k_psum<double><<<fe::RED_BLOCKS, fe::RED_THREADS, 0, st>>>(m->d_mass, nullptr, n, pb); fe_count_launch();
+    k_psum_pair<<<fe::RED_BLOCKS, fe::RED_THREADS, 0, st>>>(f, nullptr, m->d_mass, n, pa, pb); fe_count_launch();
     k_fin_project_load<<<1, fe::RED_BLOCKS, 0, st>>>(pa, pb, s); fe_count_launch();
     k_project_load<<<gb, 256, 0, st>>>(f, m->d_mass, s, n); fe_count_launch();
   }
@@ -1555,9 +1587,8 @@ static fe_status poisson_solve_on(fe_mesh* m, const double* rho, const fe_poisso
   // double residual r = f - K phi (masked; CEF: minus its mean) and |r|^2 on the host
   // (at_zero: phi is zero everywhere, as the CEF solve starts, so K phi needs no product)
   auto residual = [&](double* rr, bool at_zero = false) -> fe_status {
-    if (at_zero) FE_CUDA(cudaMemsetAsync(q, 0, sizeof(double) * n, st));
-    else FE_TRY(fe_poisson_apply_K(m, phi, q));
-    k_resid0<<<gb, 256, 0, st>>>(f, q, mask, r, n); fe_count_launch();
+    if (!at_zero) FE_TRY(fe_poisson_apply_K(m, phi, q));
+    k_resid0<<<gb, 256, 0, st>>>(f, at_zero ? nullptr : q, mask, r, n); fe_count_launch();
     if (project) {
       k_psum<double><<<fe::RED_BLOCKS, fe::RED_THREADS, 0, st>>>(r, nullptr, n, pa); fe_count_launch();
       k_fin_mean<<<1, fe::RED_BLOCKS, 0, st>>>(pa, sref, 1.0 / (double)n); fe_count_launch();
@@ -1694,14 +1725,12 @@ static fe_status poisson_solve_on(fe_mesh* m, const double* rho, const fe_poisso
     rr = hs.rr;
   }
   if (project) {
-    k_psum<double><<<fe::RED_BLOCKS, fe::RED_THREADS, 0, st>>>(m->d_mass, phi, n, pa); fe_count_launch();
-    k_psum<double><<<fe::RED_BLOCKS, fe::RED_THREADS, 0, st>>>(m->d_mass, nullptr, n, pb); fe_count_launch();
+    k_psum_pair<<<fe::RED_BLOCKS, fe::RED_THREADS, 0, st>>>(m->d_mass, phi, m->d_mass, n, pa, pb); fe_count_launch();
     // (few blocks: each one sums the partials)
     k_shift_mean<<<std::min(gb, 304), fe::RED_BLOCKS, 0, st>>>(phi, pa, pb, n); fe_count_launch();
   }
   if (vbare) {
-    k_vbare<<<fe::grid_for(m->n_psi), 256, 0, st>>>(g, phi, m->d_vlms, make_vapp(bc->field, g.Lz), project,
-                                                      m->gz_lo, vbare, m->n_psi); fe_count_launch();
+    launch_vbare(m, g, phi, make_vapp(bc->field, g.Lz), project, m->gz_lo, m->NZs, vbare);
   }
   FE_CUDA(cudaGetLastError());
   FE_CUDA(cudaStreamSynchronize(st));
