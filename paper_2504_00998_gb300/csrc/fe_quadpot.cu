@@ -49,11 +49,7 @@ struct QuadShape {
   static constexpr int G = VC / VW;                // lane groups per node
   static constexpr int LINES = N1 * N1 * G;
   static constexpr int NT = (LINES + 31) / 32 * 32;
-};
-
-template <typename T>
-struct QuadB {
-  T B[FE_MAXN1][FE_MAXN1];   // B[q][i] = l_i(gauss point q), reference interval
+  static constexpr int RES = 896 / NT < 16 ? 896 / NT : 16;   // 28 warps an SM: 72 registers
 };
 
 struct QuadPass {
@@ -67,25 +63,68 @@ __device__ __forceinline__ int class_cell(int t, int cls, int n) {
   return cls == 2 ? n - 1 : 2 * t + cls;
 }
 
-template <typename V>
-__device__ __forceinline__ V vzero();
+// lanes of one 16-byte access; float lanes in pairs, so that an FMA instruction takes two
+__device__ __forceinline__ unsigned long long pack(float a, float b) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 unpack(unsigned long long r) {
+  float2 f;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(r));
+  return f;
+}
+template <typename T>
+struct Lanes;
 template <>
-__device__ __forceinline__ float4 vzero<float4>() { return make_float4(0.f, 0.f, 0.f, 0.f); }
+struct Lanes<float> {
+  unsigned long long a, b;
+  static __device__ __forceinline__ Lanes of(const float4& f) { return {pack(f.x, f.y), pack(f.z, f.w)}; }
+  __device__ __forceinline__ float4 v16() const {
+    const float2 x = unpack(a), y = unpack(b);
+    return make_float4(x.x, x.y, y.x, y.y);
+  }
+};
 template <>
-__device__ __forceinline__ double2 vzero<double2>() { return make_double2(0.0, 0.0); }
-
-__device__ __forceinline__ float4 vfma(float a, const float4& x, const float4& y) {
-  return make_float4(fmaf(a, x.x, y.x), fmaf(a, x.y, y.y), fmaf(a, x.z, y.z), fmaf(a, x.w, y.w));
+struct Lanes<double> {
+  double a, b;
+  static __device__ __forceinline__ Lanes of(const double2& f) { return {f.x, f.y}; }
+  __device__ __forceinline__ double2 v16() const { return make_double2(a, b); }
+};
+using LF = Lanes<float>;
+using LD = Lanes<double>;
+__device__ __forceinline__ unsigned long long fma2(unsigned long long x, unsigned long long y,
+                                                   unsigned long long z) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(x), "l"(y), "l"(z));
+  return r;
 }
-__device__ __forceinline__ double2 vfma(double a, const double2& x, const double2& y) {
-  return make_double2(fma(a, x.x, y.x), fma(a, x.y, y.y));
+__device__ __forceinline__ unsigned long long mul2(unsigned long long x, unsigned long long y) {
+  unsigned long long r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
+  return r;
 }
-__device__ __forceinline__ float4 vscale(float a, const float4& x) {
-  return make_float4(a * x.x, a * x.y, a * x.z, a * x.w);
+__device__ __forceinline__ unsigned long long add2(unsigned long long x, unsigned long long y) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
+  return r;
 }
-__device__ __forceinline__ double2 vscale(double a, const double2& x) {
-  return make_double2(a * x.x, a * x.y);
+__device__ __forceinline__ LF lfma(float c, const LF& x, const LF& y) {
+  const unsigned long long s = pack(c, c);
+  return {fma2(s, x.a, y.a), fma2(s, x.b, y.b)};
 }
+__device__ __forceinline__ LF lmul(float c, const LF& x) {
+  const unsigned long long s = pack(c, c);
+  return {mul2(s, x.a), mul2(s, x.b)};
+}
+__device__ __forceinline__ LF ladd(const LF& x, const LF& y) { return {add2(x.a, y.a), add2(x.b, y.b)}; }
+__device__ __forceinline__ LF lsub(const LF& x, const LF& y) { return lfma(-1.f, y, x); }
+__device__ __forceinline__ LD lfma(double c, const LD& x, const LD& y) { return {fma(c, x.a, y.a), fma(c, x.b, y.b)}; }
+__device__ __forceinline__ LD lmul(double c, const LD& x) { return {c * x.a, c * x.b}; }
+__device__ __forceinline__ LD ladd(const LD& x, const LD& y) { return {x.a + y.a, x.b + y.b}; }
+__device__ __forceinline__ LD lsub(const LD& x, const LD& y) { return {x.a - y.a, x.b - y.b}; }
+__device__ __forceinline__ float4 vzero(float) { return make_float4(0.f, 0.f, 0.f, 0.f); }
+__device__ __forceinline__ double2 vzero(double) { return make_double2(0.0, 0.0); }
 // keep the first k lanes (k < lanes of the access), zero the rest
 __device__ __forceinline__ float4 vkeep(float4 x, int k) {
   if (k < 4) x.w = 0.f;
@@ -104,59 +143,147 @@ __device__ __forceinline__ void vstore_first(float* p, const float4& x, int k) {
 }
 __device__ __forceinline__ void vstore_first(double* p, const double2& x, int) { p[0] = x.x; }
 
-// one line contraction along direction D of the cell block in shared memory ([node][lane],
-// 16-byte groups): forward dst(q) = sum_e B[q][e] src(e) (times the quadrature weight of
-// point q when WEIGH), transposed dst(e) = sum_q B[q][e] src(q).  Line (a, b, group) of the
-// calling thread: a, b the two other local indices.
-template <typename T, int P, int D, bool TR, bool WEIGH>
-__device__ __forceinline__ void contract(const QuadB<T>& cb, const T* __restrict__ src,
-                                         T* __restrict__ dst, const T* __restrict__ Ws, int a,
-                                         int b, int grp) {
-  using S = QuadShape<T, P>;
-  using V = typename QuadLanes<T>::V16;
-  constexpr int N1 = S::N1, G = S::G;
-  constexpr int STRIDE = D == 0 ? 1 : D == 1 ? N1 : N1 * N1;
-  const int base = D == 0 ? (b * N1 + a) * N1 : D == 1 ? b * N1 * N1 + a : b * N1 + a;
-  const V* s = reinterpret_cast<const V*>(src);
-  V* d = reinterpret_cast<V*>(dst);
-  V in[N1];
+// Lines.  The interpolation table commutes with the mirror image of the cell, B[p-q][p-e] = B[q][e],
+// so a line contraction is split into the even parts u_k + u_{p-k} and the odd ones u_k - u_{p-k}:
+// (p + 1)^2 / 2 FMAs and 2 (p + 1) sums for (p + 1)^2 FMAs, and half the constants.
+// Coefficient (j, k) of the even (odd = 0) or odd part; TR: of the transposed table.
+template <int P, bool TR>
+__device__ __forceinline__ constexpr double quad_c(int odd, int j, int k) {
+  const double a = TR ? fe::gauss_b<P>(k, j) : fe::gauss_b<P>(j, k);
+  if (k == P - k) return a;
+  const double b = TR ? fe::gauss_b<P>(P - k, j) : fe::gauss_b<P>(j, P - k);
+  return odd ? 0.5 * (a - b) : 0.5 * (a + b);
+}
+template <typename T, int P>
+struct Parts {
+  static constexpr int E = (P + 2) / 2, O = (P + 1) / 2;
+  Lanes<T> e[E], o[O];
+  __device__ __forceinline__ void split(const Lanes<T> (&u)[P + 1]) {
 #pragma unroll
-  for (int e = 0; e < N1; ++e) in[e] = s[(base + e * STRIDE) * G + grp];
-#pragma unroll
-  for (int q = 0; q < N1; ++q) {
-    V acc = vzero<V>();
-#pragma unroll
-    for (int e = 0; e < N1; ++e) {
-      // float: the interpolation table as compile-time constants (immediate operands)
-      T c;
-      if constexpr (std::is_same<T, float>::value)
-        c = TR ? fe::gauss_b<P>(e, q) : fe::gauss_b<P>(q, e);
-      else
-        c = TR ? cb.B[e][q] : cb.B[q][e];
-      acc = vfma(c, in[e], acc);
+    for (int k = 0; k < O; ++k) {
+      e[k] = ladd(u[k], u[P - k]);
+      o[k] = lsub(u[k], u[P - k]);
     }
-    if constexpr (WEIGH) acc = vscale(Ws[base + q * STRIDE], acc);
-    d[(base + q * STRIDE) * G + grp] = acc;
+    if constexpr (E > O) e[O] = u[O];
+  }
+  // parts of output q
+  template <bool TR>
+  __device__ __forceinline__ Lanes<T> even(int q) const {
+    Lanes<T> s = lmul((T)quad_c<P, TR>(0, q, 0), e[0]);
+#pragma unroll
+    for (int k = 1; k < E; ++k) s = lfma((T)quad_c<P, TR>(0, q, k), e[k], s);
+    return s;
+  }
+  template <bool TR>
+  __device__ __forceinline__ Lanes<T> odd(int q) const {
+    Lanes<T> s = lmul((T)quad_c<P, TR>(1, q, 0), o[0]);
+#pragma unroll
+    for (int k = 1; k < O; ++k) s = lfma((T)quad_c<P, TR>(1, q, k), o[k], s);
+    return s;
+  }
+};
+
+// u <- B u (TR: B^T u)
+template <typename T, int P, bool TR>
+__device__ __forceinline__ void line(Lanes<T> (&u)[P + 1]) {
+  Parts<T, P> s;
+  s.split(u);
+#pragma unroll
+  for (int q = 0; q < Parts<T, P>::E; ++q) {
+    const Lanes<T> ev = s.template even<TR>(q);
+    if (q < Parts<T, P>::O) {
+      const Lanes<T> od = s.template odd<TR>(q);
+      u[q] = ladd(ev, od);
+      u[P - q] = lsub(ev, od);
+    } else {
+      u[q] = ev;
+    }
   }
 }
-
+// u <- B^T diag(w) B u, w[q * stride] the weight of point q
 template <typename T, int P>
-__global__ void __launch_bounds__(QuadShape<T, P>::NT)
-k_quad_apply(const QuadB<T> cb, const QuadPass g, const T* __restrict__ X, T* __restrict__ Y,
-             int64_t ld, int64_t nvec, const T* __restrict__ W, const T* __restrict__ rsq,
-             T alpha) {
+__device__ __forceinline__ void line_weighted(Lanes<T> (&u)[P + 1], const T* __restrict__ w, int stride) {
+  using S = Parts<T, P>;
+  S s;
+  s.split(u);
+  Lanes<T> e[S::E], o[S::O];
+#pragma unroll
+  for (int q = 0; q < S::E; ++q) {
+    Lanes<T> g = s.template even<false>(q), d;
+    if (q < S::O) {
+      const Lanes<T> od = s.template odd<false>(q);
+      const Lanes<T> lo = lmul(w[q * stride], ladd(g, od)), hi = lmul(w[(P - q) * stride], lsub(g, od));
+      g = ladd(lo, hi);
+      d = lsub(lo, hi);
+    } else {
+      g = lmul(w[q * stride], g);
+    }
+#pragma unroll
+    for (int k = 0; k < S::E; ++k) {
+      const T c = (T)quad_c<P, true>(0, k, q);
+      e[k] = q ? lfma(c, g, e[k]) : lmul(c, g);
+    }
+    if (q < S::O) {
+#pragma unroll
+      for (int k = 0; k < S::O; ++k) {
+        const T c = (T)quad_c<P, true>(1, k, q);
+        o[k] = q ? lfma(c, d, o[k]) : lmul(c, d);
+      }
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < S::O; ++k) {
+    u[k] = ladd(e[k], o[k]);
+    u[P - k] = lsub(e[k], o[k]);
+  }
+  if constexpr (S::E > S::O) u[S::O] = e[S::O];
+}
+
+// the calling thread's line of the cell block in shared memory ([node][lane], 16-byte groups)
+template <typename T, int P, int D>
+struct LineAt {
   using S = QuadShape<T, P>;
   using V = typename QuadLanes<T>::V16;
+  static constexpr int STRIDE = D == 0 ? 1 : D == 1 ? S::N1 : S::N1 * S::N1;
+  V* at;
+  int base;
+  // (a, b): the two other local indices
+  __device__ __forceinline__ LineAt(T* buf, int a, int b, int grp)
+      : at(reinterpret_cast<V*>(buf)),
+        base(D == 0 ? (b * S::N1 + a) * S::N1 : D == 1 ? b * S::N1 * S::N1 + a : b * S::N1 + a) {
+    at += base * S::G + grp;
+  }
+  __device__ __forceinline__ void load(Lanes<T> (&u)[P + 1]) const {
+#pragma unroll
+    for (int e = 0; e <= P; ++e) u[e] = Lanes<T>::of(at[e * STRIDE * S::G]);
+  }
+  __device__ __forceinline__ void store(const Lanes<T> (&u)[P + 1]) const {
+#pragma unroll
+    for (int e = 0; e <= P; ++e) at[e * STRIDE * S::G] = u[e].v16();
+  }
+};
+
+// Y += alpha M^-1/2 V M^-1/2 X on the cells of one colour; a CTA takes one cell and VC lanes.
+// What bounds it: memory latency, two trips a CTA (X at the start, Y at the end) with 27 warps an
+// SM to cover them, at 4.6 TB/s of its algorithmic bytes on 16 x 16 x 16 cells p = 5, 256 float
+// vectors: 74 us a colour pass, where dense lines, unpaired float FMAs, a shared round trip
+// between the two z contractions and a node table that the X loads waited for took 83.  The
+// z contraction, the weights and the transposed contraction are one step in registers, and
+// every thread rewrites its own lines only: one buffer, four barriers.  A filter of degree 8 on
+// that slab, kinetic part included: 9.75 -> 9.14 ms.
+template <typename T, int P, bool PREFETCH>
+__global__ void __launch_bounds__(QuadShape<T, P>::NT, QuadShape<T, P>::RES)
+k_quad_apply(const QuadPass g, const T* __restrict__ X, T* __restrict__ Y, int64_t ld, int64_t nvec,
+             const T* __restrict__ W, const T* __restrict__ rsq, T alpha) {
+  using S = QuadShape<T, P>;
+  using V = typename QuadLanes<T>::V16;
+  using L = Lanes<T>;
   constexpr int N1 = S::N1, NN = S::NN, VC = S::VC, VW = S::VW, G = S::G, NT = S::NT;
   constexpr int SLOTS = NN * G;                      // 16-byte slots of the cell block
   constexpr int IT = (SLOTS + NT - 1) / NT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* bufA = reinterpret_cast<T*>(smem_raw);
-  T* bufB = bufA + NN * VC;
-  constexpr int NNE = (NN + 1) & ~1;                 // even: keeps node[] 8-byte aligned
-  T* Ws = bufB + NN * VC;                            // w |J| V at the Gauss points
-  T* rs = Ws + NNE;                                  // M^-1/2 at the cell's nodes
-  int64_t* node = reinterpret_cast<int64_t*>(rs + NNE);
+  T* buf = reinterpret_cast<T*>(smem_raw);
+  T* Ws = buf + NN * VC;                             // w |J| V at the Gauss points
 
   int t = blockIdx.x;
   const int tx = t % g.cntx;
@@ -169,100 +296,97 @@ k_quad_apply(const QuadB<T> cb, const QuadPass g, const T* __restrict__ X, T* __
   const int64_t plane = (int64_t)g.NX * g.NY;
   const int tid = threadIdx.x;
 
-  for (int e = tid; e < NN; e += NT) {
-    const int i = e % N1, j = (e / N1) % N1, k = e / (N1 * N1);
-    int gx = cx * P + i, gy = cy * P + j;
-    gx -= gx >= g.NX ? g.NX : 0;
-    gy -= gy >= g.NY ? g.NY : 0;
-    const int gz = cz * P + k;
-    const bool in = gz >= g.gz_lo && gz <= g.gz_hi;
-    const int64_t n = in ? (gz - g.gz_lo) * plane + (int64_t)gy * g.NX + gx : -1;
-    node[e] = n;
-    rs[e] = in ? rsq[n] : T(0);
-    Ws[e] = W[cell * NN + e];
-  }
-  __syncthreads();
-  const bool act = tid < S::LINES;
+  for (int e = tid; e < NN; e += NT) Ws[e] = W[cell * NN + e];
   const int grp = tid % G, ab = tid / G;
   const int la = ab % N1, lb = ab / N1;     // (j, k) of the thread's x line
-  const int xbase = (lb * N1 + la) * N1;
   const int64_t vv = v0 + (int64_t)grp * VW;
   const int64_t left = nvec - vv;           // lanes of the group that are vectors
+  const bool act = tid < S::LINES;
+  // first node of the row of nodes j, k (-1 outside the stored planes), and the x index of node i
+  auto row_of = [&](int j, int k) {
+    const int gz = cz * P + k;
+    int gy = cy * P + j;
+    gy -= gy >= g.NY ? g.NY : 0;
+    return gz >= g.gz_lo && gz <= g.gz_hi ? (gz - g.gz_lo) * plane + (int64_t)gy * g.NX : (int64_t)-1;
+  };
+  auto x_of = [&](int i) {
+    const int gx = cx * P + i;
+    return i == P && gx >= g.NX ? gx - g.NX : gx;
+  };
+  const int64_t row = act ? row_of(la, lb) : -1;
+  const bool on = row >= 0 && left > 0;
   // x lines straight from global memory: u = M^-1/2 X on the line's nodes (every load of
   // the thread in flight before the first use; zero on Dirichlet faces and past the last
   // vector; a row holds ld >= the group's end, so the whole group is in bounds), then the
-  // forward x contraction
+  // forward x contraction.  A thread reads and writes its own lines only, so one buffer does.
+  // The Y lines, needed at the end, are asked for now where they are not in L2 anyway.
+  L u[N1];
   if (act) {
     V in[N1];
+    T r[N1];
 #pragma unroll
     for (int e = 0; e < N1; ++e) {
-      const int64_t n = node[xbase + e];
-      in[e] = vzero<V>();
-      if (n >= 0 && left > 0) in[e] = *reinterpret_cast<const V*>(X + n * ld + vv);
-    }
-    V* d = reinterpret_cast<V*>(bufB);
-#pragma unroll
-    for (int e = 0; e < N1; ++e) {
-      in[e] = vscale(rs[xbase + e], in[e]);
-      if (left < VW) in[e] = vkeep(in[e], left > 0 ? (int)left : 0);
-    }
-#pragma unroll
-    for (int q = 0; q < N1; ++q) {
-      V acc = vzero<V>();
-#pragma unroll
-      for (int e = 0; e < N1; ++e) {
-        T c;
-        if constexpr (std::is_same<T, float>::value) c = fe::gauss_b<P>(q, e);
-        else c = cb.B[q][e];
-        acc = vfma(c, in[e], acc);
+      in[e] = vzero(T(0));
+      r[e] = T(0);
+      if (on) {
+        const int64_t n = row + x_of(e);
+        in[e] = *reinterpret_cast<const V*>(X + n * ld + vv);
+        r[e] = rsq[n];
+        if (PREFETCH && grp == 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(Y + n * ld + vv));
       }
-      d[(xbase + q) * G + grp] = acc;
     }
+#pragma unroll
+    for (int e = 0; e < N1; ++e) {
+      if (left < VW) in[e] = vkeep(in[e], left > 0 ? (int)left : 0);
+      u[e] = lmul(r[e], L::of(in[e]));
+    }
+    line<T, P, false>(u);
+    LineAt<T, P, 0>(buf, la, lb, grp).store(u);
   }
   __syncthreads();
-  if (act) contract<T, P, 1, false, false>(cb, bufB, bufA, Ws, la, lb, grp);
+  if (act) {
+    const LineAt<T, P, 1> at(buf, la, lb, grp);
+    at.load(u);
+    line<T, P, false>(u);
+    at.store(u);
+  }
   __syncthreads();
-  if (act) contract<T, P, 2, false, true>(cb, bufA, bufB, Ws, la, lb, grp);
+  if (act) {
+    const LineAt<T, P, 2> at(buf, la, lb, grp);
+    at.load(u);
+    line_weighted<T, P>(u, Ws + at.base, N1 * N1);
+    at.store(u);
+  }
   __syncthreads();
-  if (act) contract<T, P, 2, true, false>(cb, bufB, bufA, Ws, la, lb, grp);
-  __syncthreads();
-  if (act) contract<T, P, 1, true, false>(cb, bufA, bufB, Ws, la, lb, grp);
+  if (act) {
+    const LineAt<T, P, 1> at(buf, la, lb, grp);
+    at.load(u);
+    line<T, P, true>(u);
+    at.store(u);
+  }
   __syncthreads();
   if (!g.foldy) {
     // transposed x contraction in registers and Y += alpha M^-1/2 (.) along the line; a
     // single cell along x (foldx) adds its two copies of node 0 before writing it once
     if (act) {
-      const V* sv = reinterpret_cast<const V*>(bufB);
-      V in[N1], out[N1];
-#pragma unroll
-      for (int q = 0; q < N1; ++q) in[q] = sv[(xbase + q) * G + grp];
-#pragma unroll
-      for (int e = 0; e < N1; ++e) {
-        V acc = vzero<V>();
-#pragma unroll
-        for (int q = 0; q < N1; ++q) {
-          T c;
-          if constexpr (std::is_same<T, float>::value) c = fe::gauss_b<P>(q, e);
-          else c = cb.B[q][e];
-          acc = vfma(c, in[q], acc);
-        }
-        out[e] = acc;
-      }
-      if (g.foldx) out[0] = vfma(T(1), out[P], out[0]);
+      LineAt<T, P, 0>(buf, la, lb, grp).load(u);
+      line<T, P, true>(u);
+      if (g.foldx) u[0] = ladd(u[P], u[0]);
+      if (!on) return;
       V yv[N1];
+      T r[N1];
 #pragma unroll
       for (int e = 0; e < N1; ++e) {
-        const int64_t n = node[xbase + e];
-        yv[e] = vzero<V>();
-        if (n >= 0 && left > 0 && !(g.foldx && e == P))
-          yv[e] = *reinterpret_cast<const V*>(Y + n * ld + vv);
+        const int64_t n = row + x_of(e);
+        yv[e] = vzero(T(0));
+        r[e] = rsq[n];
+        if (!(g.foldx && e == P)) yv[e] = *reinterpret_cast<const V*>(Y + n * ld + vv);
       }
 #pragma unroll
       for (int e = 0; e < N1; ++e) {
-        const int64_t n = node[xbase + e];
-        if (n < 0 || left <= 0 || (g.foldx && e == P)) continue;
-        const V o = vfma(alpha * rs[xbase + e], out[e], yv[e]);
-        T* yp = Y + n * ld + vv;
+        if (g.foldx && e == P) continue;
+        const V o = lfma(alpha * r[e], u[e], L::of(yv[e])).v16();
+        T* yp = Y + (row + x_of(e)) * ld + vv;
         if (left >= VW)
           *reinterpret_cast<V*>(yp) = o;
         else
@@ -273,24 +397,27 @@ k_quad_apply(const QuadB<T> cb, const QuadPass g, const T* __restrict__ X, T* __
   }
   // a single cell along y: the two copies of each j = 0 node are in different x lines, so
   // the block goes back to the nodes in shared memory and is folded there
-  if (act) contract<T, P, 0, true, false>(cb, bufB, bufA, Ws, la, lb, grp);
+  if (act) {
+    const LineAt<T, P, 0> at(buf, la, lb, grp);
+    at.load(u);
+    line<T, P, true>(u);
+    at.store(u);
+  }
   __syncthreads();
-  V* A = reinterpret_cast<V*>(bufA);
+  V* A = reinterpret_cast<V*>(buf);
   if (g.foldx) {
     for (int idx = tid; idx < N1 * N1 * G; idx += NT) {
       const int gg = idx % G, r = idx / G;   // r = (k, j)
-      V x = A[(r * N1) * G + gg];
-      const V y = A[(r * N1 + P) * G + gg];
-      A[(r * N1) * G + gg] = vfma(T(1), y, x);
+      const L x = L::of(A[(r * N1) * G + gg]), y = L::of(A[(r * N1 + P) * G + gg]);
+      A[(r * N1) * G + gg] = ladd(x, y).v16();
     }
     __syncthreads();
   }
   for (int idx = tid; idx < N1 * N1 * G; idx += NT) {
     const int gg = idx % G, r = idx / G;
     const int i = r % N1, k = r / N1;
-    V x = A[(k * N1 * N1 + i) * G + gg];
-    const V y = A[(k * N1 * N1 + P * N1 + i) * G + gg];
-    A[(k * N1 * N1 + i) * G + gg] = vfma(T(1), y, x);
+    const L x = L::of(A[(k * N1 * N1 + i) * G + gg]), y = L::of(A[(k * N1 * N1 + P * N1 + i) * G + gg]);
+    A[(k * N1 * N1 + i) * G + gg] = ladd(x, y).v16();
   }
   __syncthreads();
   // Y += alpha M^-1/2 (V u): all loads of Y first, then the updates
@@ -299,11 +426,12 @@ k_quad_apply(const QuadB<T> cb, const QuadPass g, const T* __restrict__ X, T* __
 #pragma unroll
     for (int it = 0; it < IT; ++it) {
       const int sl = tid + it * NT;
-      yv[it] = vzero<V>();
+      yv[it] = vzero(T(0));
       if (sl < SLOTS) {
         const int e = sl / G, ww = (sl % G) * VW;
-        const int64_t n = node[e];
-        if (n >= 0 && v0 + ww < nvec) yv[it] = *reinterpret_cast<const V*>(Y + n * ld + v0 + ww);
+        const int64_t nr = row_of((e / N1) % N1, e / (N1 * N1));
+        if (nr >= 0 && v0 + ww < nvec)
+          yv[it] = *reinterpret_cast<const V*>(Y + (nr + x_of(e % N1)) * ld + v0 + ww);
       }
     }
 #pragma unroll
@@ -313,9 +441,9 @@ k_quad_apply(const QuadB<T> cb, const QuadPass g, const T* __restrict__ X, T* __
       const int e = sl / G, ww = (sl % G) * VW;
       const int i = e % N1, j = (e / N1) % N1;
       if ((g.foldx && i == P) || j == P) continue;
-      const int64_t n = node[e];
-      if (n < 0 || v0 + ww >= nvec) continue;
-      const V o = vfma(alpha * rs[e], A[sl], yv[it]);
+      const int64_t nr = row_of(j, e / (N1 * N1)), n = nr + x_of(i);
+      if (nr < 0 || v0 + ww >= nvec) continue;
+      const V o = lfma(alpha * rsq[n], L::of(A[sl]), L::of(yv[it])).v16();
       T* yp = Y + n * ld + v0 + ww;
       const int64_t rem = nvec - (v0 + ww);
       if (rem >= VW)
@@ -329,20 +457,24 @@ k_quad_apply(const QuadB<T> cb, const QuadPass g, const T* __restrict__ X, T* __
 template <typename T, int P>
 size_t quad_smem() {
   using S = QuadShape<T, P>;
-  return sizeof(T) * (2 * (size_t)S::NN * S::VC + 2 * (size_t)((S::NN + 1) & ~1)) +
-         sizeof(int64_t) * S::NN;
+  return sizeof(T) * ((size_t)S::NN * S::VC + S::NN);
 }
 
 template <typename T, int P>
-fe_status quad_apply_p(fe_mesh* m, const QuadB<T>& cb, const T* X, T* Y, int64_t ld,
-                       int64_t nvec, const T* W, const T* rsq, T alpha) {
+fe_status quad_apply_p(fe_mesh* m, const T* X, T* Y, int64_t ld, int64_t nvec, const T* W,
+                       const T* rsq, T alpha) {
   using S = QuadShape<T, P>;
   constexpr int VC = S::VC;
   const size_t smem = quad_smem<T, P>();
-  cudaError_t e = cudaFuncSetAttribute(k_quad_apply<T, P>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // Y's lines are asked for at the start where the block exceeds L2 (524 MB: 1164 -> 1114 us an
+  // H X); smaller blocks only pay for the instructions (94 MB: 247 -> 256 us, 71 MB: 207 -> 211).
+  int l2 = 0;
+  if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, m->device) != cudaSuccess) cudaGetLastError();
+  const bool beyond = (double)m->n_psi * (double)ld * sizeof(T) > (double)l2;
+  auto kern = beyond ? k_quad_apply<T, P, true> : k_quad_apply<T, P, false>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_quad_apply<T, P>, cudaFuncAttributePreferredSharedMemoryCarveout,
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
                              (int)cudaSharedmemCarveoutMaxShared);
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -386,8 +518,8 @@ fe_status quad_apply_p(fe_mesh* m, const QuadB<T>& cb, const T* X, T* Y, int64_t
         if (cells > 0x7fffffffLL) return fe_fail(FE_EINVAL, "quadrature potential: mesh too large");
         g.ox = clx[c]; g.oy = cly[b]; g.oz = clz[a];
         g.cntx = cnx[c]; g.cnty = cny[b]; g.cntz = cnz[a];
-        k_quad_apply<T, P><<<dim3((unsigned)cells, (unsigned)nchunk), S::NT, smem, m->stream>>>(
-            cb, g, X, Y, ld, nvec, W, rsq, alpha);
+        kern<<<dim3((unsigned)cells, (unsigned)nchunk), S::NT, smem, m->stream>>>(
+            g, X, Y, ld, nvec, W, rsq, alpha);
         fe_count_launch();
       }
   FE_CUDA(cudaGetLastError());
@@ -397,16 +529,13 @@ fe_status quad_apply_p(fe_mesh* m, const QuadB<T>& cb, const T* X, T* Y, int64_t
 template <typename T>
 fe_status quad_apply_t(fe_mesh* m, const T* X, T* Y, int64_t ld, int64_t nvec, const T* W,
                        const T* rsq, T alpha) {
-  QuadB<T> cb;
-  for (int q = 0; q < FE_MAXN1; ++q)
-    for (int i = 0; i < FE_MAXN1; ++i) cb.B[q][i] = (T)m->Bq[q][i];
   switch (m->p) {
-    case 1: return quad_apply_p<T, 1>(m, cb, X, Y, ld, nvec, W, rsq, alpha);
-    case 2: return quad_apply_p<T, 2>(m, cb, X, Y, ld, nvec, W, rsq, alpha);
-    case 3: return quad_apply_p<T, 3>(m, cb, X, Y, ld, nvec, W, rsq, alpha);
-    case 4: return quad_apply_p<T, 4>(m, cb, X, Y, ld, nvec, W, rsq, alpha);
-    case 5: return quad_apply_p<T, 5>(m, cb, X, Y, ld, nvec, W, rsq, alpha);
-    case 6: return quad_apply_p<T, 6>(m, cb, X, Y, ld, nvec, W, rsq, alpha);
+    case 1: return quad_apply_p<T, 1>(m, X, Y, ld, nvec, W, rsq, alpha);
+    case 2: return quad_apply_p<T, 2>(m, X, Y, ld, nvec, W, rsq, alpha);
+    case 3: return quad_apply_p<T, 3>(m, X, Y, ld, nvec, W, rsq, alpha);
+    case 4: return quad_apply_p<T, 4>(m, X, Y, ld, nvec, W, rsq, alpha);
+    case 5: return quad_apply_p<T, 5>(m, X, Y, ld, nvec, W, rsq, alpha);
+    case 6: return quad_apply_p<T, 6>(m, X, Y, ld, nvec, W, rsq, alpha);
     default: return fe_fail(FE_EUNSUPPORTED, "p = %d", m->p);
   }
 }

@@ -1,5 +1,5 @@
 """Writes fe_gll_tables.h: the shape-only 1D tables of the Hamiltonian sweep kernel and of the
-float Gauss-quadrature potential kernel.
+Gauss-quadrature potential kernel.
 
 They depend on the degree p only; the mesh enters through scalars at run time.  K1, M1 are the
 exactly integrated 1D stiffness and mass matrices of the Lagrange basis on the p + 1
@@ -103,16 +103,6 @@ def gauss_interp(p):
     return [[lagrange(xi, i, gq[q])[0] for i in range(p + 1)] for q in range(p + 1)]
 
 
-def f32(v):
-    import struct
-    return struct.unpack("f", struct.pack("f", v))[0]
-
-
-def emit(name, A):
-    rows = ",\n    ".join("{" + ", ".join(repr(f32(v)) + "f" for v in r) + "}" for r in A)
-    return f"__device__ constexpr float {name}[{len(A)}][{len(A)}] = {{\n    {rows}}};\n"
-
-
 def emit_double(name, A):
     rows = ",\n    ".join("{" + ", ".join(repr(v) for v in r) + "}" for r in A)
     return f"__device__ constexpr double {name}[{len(A)}][{len(A[0])}] = {{\n    {rows}}};\n"
@@ -124,7 +114,7 @@ def main():
            "// definition).",
            "#pragma once", "", "namespace fe {", ""]
     for p in range(1, 7):
-        out.append(emit(f"kGaussB{p}", gauss_interp(p)))
+        out.append(emit_double(f"kGaussB{p}", gauss_interp(p)))
         KH, GH, TH, NH = hat_tables(p)
         out.append(emit_double(f"kHatK{p}", KH))
         out.append(emit_double(f"kHatG{p}", GH))
@@ -132,7 +122,7 @@ def main():
         out.append(emit_double(f"kHatN{p}", [NH]))
     out.append("""// GB[q][i] of degree P
 template <int P>
-__device__ __forceinline__ constexpr float gauss_b(int q, int i) {
+__device__ __forceinline__ constexpr double gauss_b(int q, int i) {
   if constexpr (P == 1) return kGaussB1[q][i];
   else if constexpr (P == 2) return kGaussB2[q][i];
   else if constexpr (P == 3) return kGaussB3[q][i];

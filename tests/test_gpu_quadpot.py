@@ -82,6 +82,22 @@ def test_apply_Hq_matches_oracle(fe, L, ncell, p, dirichlet, prec, nvec, ld):
     assert torch.all(yb[:, nvec:] == 3.0)      # padding lanes untouched
 
 
+@pytest.mark.parametrize("p", [1, 2, 3, 4, 5, 6])
+@pytest.mark.parametrize("nvec", [3, 31, 32, 33])
+def test_apply_Hq_lane_chunks(fe, p, nvec):
+    """Full and partial lane chunks (32 float, 16 double lanes) for every degree, on odd and even
+    cell rows; tolerances of the collocated operator, the padding of the rows untouched."""
+    om, H, m, rng, Vq = _setup(fe, (3.0, 5.0, 5.0), (3, 4, 2), p, (True, False), seed=p)
+    ld = -(-nvec // 4) * 4
+    for prec, dt, tol in ((fe.FE_F64, torch.float64, 1e-10), (fe.FE_F32, torch.float32, 2e-5)):
+        X = _block(rng.standard_normal((om.n_psi, nvec)), dt, ld)
+        Y = torch.full_like(X, 7.0)
+        fe._lib.call("fe_apply_H", m.handle, fe._ptr(X), fe._ptr(Y), nvec, ld, int(prec))
+        ref = H @ X[:, :nvec].double().cpu().numpy()
+        assert np.linalg.norm(Y[:, :nvec].double().cpu().numpy() - ref) <= tol * np.linalg.norm(ref)
+        assert torch.all(Y[:, nvec:] == 7.0)
+
+
 def test_apply_Hq_is_bitwise_repeatable(fe):
     om, H, m, rng, Vq = _setup(fe, *CASES[3])
     X = torch.tensor(rng.standard_normal((om.n_psi, 64)), dtype=torch.float32, device="cuda")
