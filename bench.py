@@ -319,14 +319,13 @@ def fp64_gemm_peak(dev, n=8192, reps=5):
 
 
 def sumfact_flops_per_hx(slab, nvec):
-    """Arithmetic of the sum-factorised operator: per node-vector seven assembled 1D
-    contractions (y: M1 and K1; x: M1 on both, K1 on one; z: M1 and K1), each with the
-    average tap count of an assembled GLL line (p + 1 taps at p - 1 interior nodes of a
-    cell segment, 2p + 1 at the shared node: (p (p + 1) + p) / p per node), plus the
-    potential and the two-term Chebyshev update: 2 flops per FMA."""
+    """Arithmetic of the sum-factorised operator, per cell line of p nodes: three stiffness
+    contractions (x, y, z) of (p + 1)^2 FMAs, and four mass ones (y; x on both; z), each a dot
+    product and an update of p + 1 FMAs; per node-vector the two in-plane scales, the
+    potential and the Chebyshev update: 2 flops per FMA."""
     p = slab.p
-    taps = (p * (p + 1) + p) / p
-    return 2.0 * (7.0 * taps + 3.0) * slab.n_psi * nvec
+    fmas = (3.0 * (p + 1) ** 2 + 8.0 * (p + 1)) / p + 4.0
+    return 2.0 * fmas * slab.n_psi * nvec
 
 
 # ------------------------------------------------------------------------------------------
@@ -558,7 +557,7 @@ def sweep_measure(steps, warmup):
         "filter_tflops": flops_hx * degree / (f_ms * 1e-3) / 1e12,
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": None, "peak_source": peak_src,
-                     "kernel": "kron_batch_f32_p4",
+                     "kernel": "sweep_batch_f32_p4",
                      "algorithmic_bytes_per_launch": bytes_filter / degree,
                      "launch_ms": f_ms / degree},
         "gpu_launches": launches, "clocks": clk.summary()}
@@ -691,7 +690,7 @@ def run_gpu(args):
     launch_ms = phase[2] / degree
     achieved = bytes_per_launch / (launch_ms * 1e-3) / 1e9
     peak, peak_src = measured_peaks()
-    kernel_key = {fe.FE_F32: "kron_f32_p5", fe.FE_F64: "kron_f64_p5",
+    kernel_key = {fe.FE_F32: "sweep_f32_p5", fe.FE_F64: "sweep_f64_p5",
                   fe.FE_F32_F32ACC: "ktc_f32_p5"}.get(prec, "tc_p5")
     # (the nonlocal term adds its own kernels to the filter time: no single-kernel traffic)
     traffic = traffic_record(kernel_key, n * nvec) if not nl_desc else None
@@ -868,7 +867,8 @@ def run_gpu(args):
             extra["fp64_roofline"] = {
                 "bound": "fp64", "achieved": hw, "peak": pk64, "unit": "TFLOP/s",
                 "frac": hw / pk64, "peak_source": "measured in this run: cuBLAS DGEMM 8192^3",
-                "flops": "sum-factorised operator arithmetic: 2 (7 (p + 2) + 3) per node-vector"}
+                "flops": "sum-factorised operator arithmetic: 2 ((3 (p + 1)^2 + 8 (p + 1)) / p + 4) "
+                         "per node-vector"}
         torch.cuda.empty_cache()
 
     conformant = None
@@ -1108,7 +1108,7 @@ def large_measure(steps, warmup):
         "ritz_range_ha": [float(theta[0]), float(theta[-1])],
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": None, "peak_source": peak_src,
-                     "kernel": "kron_f32_p5 (256-vector block, leading dimension 1024)",
+                     "kernel": "sweep_f32_p5 (256-vector block, leading dimension 1024)",
                      "algorithmic_bytes_per_launch": bytes_launch, "launch_ms": launch_ms},
         "gpu_launches": launches, "clocks": clk.summary()}
     m.close()

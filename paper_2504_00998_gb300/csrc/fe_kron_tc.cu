@@ -5,7 +5,7 @@
 // exactly integrated stiffness of the uniform tensor-product mesh
 //   K = ax K1 (x) M1 (x) M1 + ay M1 (x) K1 (x) M1 + az M1 (x) M1 (x) K1.
 // The kernel evaluates the fused Chebyshev step Y = alpha (Ht - shift) X + beta Z with the
-// same sum factorisation and z sweep as the CUDA-core operator (fe_kron.cuh): a CTA owns
+// same sum factorisation and z sweep as the one-vector operator (fe_kron.cuh): a CTA owns
 // the nodes of an xy block of B x B cells and 8 vectors, stages each z plane with its
 // p-node periodic halo, and accumulates the z contraction of the plane's in-plane results
 // into the p + 1 output planes of the current cell layer, in registers.  What changes is

@@ -29,9 +29,9 @@
 // What bounds it.  On the 16 x 16 x 48-cell p = 5 slab with 512 float vectors a filter step takes
 // 2.83 ms (9.3 GB algorithmic, 0.49 of the measured copy bandwidth), where the sweep with dense
 // mass contractions, scalar in-plane phases and three barriers a plane took 3.86 ms; on the
-// 16 x 16 x 16-cell slab with 256 vectors 484 against 681 us, from 261 M against 615 M warp
-// instructions.  DRAM moves 1.77 GB there (algorithmic 1.56), 54 % of the copy rate; issue slots
-// are 45 % busy, the FMA pipe 37 %, the shared-memory pipe 62 %: with 160 registers a thread
+// 16 x 16 x 16-cell slab with 256 vectors 484 against 681 us, from 266 M against 615 M warp
+// instructions.  DRAM moves 1.78 GB there (algorithmic 1.56), 54 % of the copy rate; issue slots
+// are 46 % busy, the FMA pipe 37 %, the shared-memory data pipe 56 %: with 160 registers a thread
 // only ten warps are resident, too few to cover the FMA and shared-memory latencies.  The
 // accumulators set the registers, so more warps mean spills, and those were slower (three CTAs
 // an SM at p = 5: 734 us); so were planes staged without the one-barrier double buffer of a, b
