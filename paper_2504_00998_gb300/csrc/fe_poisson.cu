@@ -1243,8 +1243,8 @@ extern "C" fe_status fe_poisson_solve_load(fe_mesh* m, const double* f, const fe
 }
 
 // Meshes of at least this many phi nodes take the separable preconditioner unless the caller has
-// chosen another.  It is the faster one at every size measured (rtol 1e-12, CEF): 4,950 nodes
-// 0.44 ms against 6.6 ms, 50,176 nodes 0.57 against 7.0, 1.54 M nodes 2.6 against 28.6; the line
+// chosen another.  It is the faster one at every size measured (rtol 1e-12, CEF): 3,600 nodes
+// 0.31 ms against 3.6 ms, 50,176 nodes 0.34 against 6.5, 1.54 M nodes 1.2 against 28.6; the line
 // only keeps the coarse-space CG, with its iteration count and cap, on the few-hundred-node
 // meshes whose callers count iterations.
 constexpr int64_t SEP_MIN_NODES = 2048;
