@@ -13,7 +13,7 @@
 
 #define FE_MAXP 6
 #define FE_MAXN1 (FE_MAXP + 1)
-#define FE_NWS 20   // workspace slots of a mesh
+#define FE_NWS 21   // workspace slots of a mesh
 
 // ---- error state ------------------------------------------------------------------------
 fe_status fe_fail(fe_status st, const char* fmt, ...);
@@ -306,7 +306,7 @@ struct fe_mesh {
 enum { WS_CHEB = 0, WS_RR_X = 1, WS_RR_HX = 2, WS_RR_SMALL = 3, WS_CG = 4, WS_RED = 5,
        WS_LANCZOS = 6, WS_TC = 7, WS_TC_IMG = 8, WS_YCELL = 9, WS_RR_TC32 = 10,
        WS_PCOARSE = 11, WS_NL = 12, WS_KCELL = 13, WS_XC = 14, WS_KPT = 15, WS_KTC = 16,
-       WS_CGF = 17, WS_PMODES = 18, WS_SEP = 19 };
+       WS_CGF = 17, WS_PMODES = 18, WS_SEP = 19, WS_KCELL64 = 20 };
 
 fe_status fe_ws(fe_mesh* m, int slot, size_t bytes, void** out);
 // Rayleigh-Ritz of a complex (Bloch) block: nvec, ld count complex entries (fe_kpoint.cu)
@@ -316,8 +316,12 @@ fe_status fe_rr_complex(fe_mesh* m, void* X, int64_t nvec, int64_t ld, double* e
 // scratch (WS_KCELL) is fe_kcell_scratch_bytes
 size_t fe_kcell_scratch_bytes(const fe_mesh* m);
 fe_status fe_kcell_apply_f32(fe_mesh* m, const float* x, float* y);
-// the same in double (fe_kcell64.cu), where its scratch can be had (*done)
+// the same in double (fe_kcell64.cu), where its scratch can be had (*done).  Its scratch is a slot
+// of its own (WS_KCELL64) with one size for the mesh's life, so neither product ever frees an
+// address that a captured graph of the other, or of its own, still uses; reserve takes it now
+// (*ws null: no memory, or the stream is being captured).
 fe_status fe_kcell_apply_f64(fe_mesh* m, const double* x, double* y, bool* done);
+fe_status fe_kcell64_reserve(fe_mesh* m, double** ws);
 fe_status fe_activate(const fe_mesh* m);
 KronGeom fe_geom(const fe_mesh* m, bool psi);
 // Y = alpha (Ht - shift) X + beta Z (plus alpha Ht_nloc X and the quadrature potential when

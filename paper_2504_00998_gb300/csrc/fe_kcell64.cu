@@ -385,23 +385,30 @@ fe_status run(fe_mesh* m, const double* x, double* y, double* yc) {
 
 }  // namespace
 
-// y = K x; *done is false (nothing enqueued) when the scratch of (p + 1)^3 doubles a cell is
-// neither there nor to be had now (a capturing stream, no memory) or the grid would be too
-// large: the caller then takes the sweep kernel, which needs no scratch
-fe_status fe_kcell_apply_f64(fe_mesh* m, const double* x, double* y, bool* done) {
-  *done = false;
-  if (m->ny > 65535 || m->nz > 65535) return FE_OK;
-  const size_t bytes = 2 * fe_kcell_scratch_bytes(m);
-  if (m->ws_bytes[WS_KCELL] < bytes) {
+fe_status fe_kcell64_reserve(fe_mesh* m, double** ws) {
+  *ws = nullptr;
+  const size_t bytes = 2 * fe_kcell_scratch_bytes(m);   // (p + 1)^3 doubles a cell
+  if (m->ws_bytes[WS_KCELL64] < bytes) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     FE_CUDA(cudaStreamIsCapturing(m->stream, &cs));
     if (cs != cudaStreamCaptureStatusNone) return FE_OK;
   }
   void* w = nullptr;
-  const fe_status st = fe_ws(m, WS_KCELL, bytes, &w);
+  const fe_status st = fe_ws(m, WS_KCELL64, bytes, &w);
   if (st == FE_ENOMEM) return FE_OK;
   FE_TRY(st);
-  double* yc = static_cast<double*>(w);
+  *ws = static_cast<double*>(w);
+  return FE_OK;
+}
+
+// y = K x; *done is false (nothing enqueued) when the scratch is neither there nor to be had now
+// or the grid would be too large: the caller then takes the sweep kernel, which needs no scratch
+fe_status fe_kcell_apply_f64(fe_mesh* m, const double* x, double* y, bool* done) {
+  *done = false;
+  if (m->ny > 65535 || m->nz > 65535) return FE_OK;
+  double* yc = nullptr;
+  FE_TRY(fe_kcell64_reserve(m, &yc));
+  if (!yc) return FE_OK;
   *done = true;
   switch (m->p) {
     case 1: return run<1>(m, x, y, yc);

@@ -1293,10 +1293,13 @@ template <typename V, typename Hook>
 fe_status cg_run(fe_mesh* m, const CgBuf<V>& b, int project, double rtol, double tol2_abs,
                  int maxit, bool use_graph, cudaGraphExec_t* exec, int64_t* graph_kernels,
                  CgState* out, const fe_cg::FusedStop* stop, Hook&& hook) {
+  // the operator's scratch exists before any graph capture
   if constexpr (std::is_same<V, float>::value) {
-    // the float operator's scratch exists before any graph capture
     void* w = nullptr;
     FE_TRY(fe_ws(m, WS_KCELL, fe_kcell_scratch_bytes(m), &w));
+  } else {
+    double* w = nullptr;
+    FE_TRY(fe_kcell64_reserve(m, &w));
   }
   const int64_t n = m->n_phi;
   const int64_t plane = (int64_t)m->NX * m->NY;

@@ -400,3 +400,54 @@ def test_apply_K_cell_strips(fe, ncell, p):
     y, ref = y.cpu().numpy(), K @ x
     assert np.linalg.norm(y - ref) / np.linalg.norm(ref) <= 1e-12
     assert np.all(np.abs(y - ref) <= 1e-13 * (abs(K) @ np.abs(x)))
+
+
+def test_captured_product_survives_the_other(fe):
+    """A graph around the float product replays correctly after double products and a solve whose
+    float iteration refines against them (CEF, Jacobi only: no double product before the
+    capture of its iterations)."""
+    base = W.small_slab(ncell=(4, 4, 8), p=5, L=(8.0, 8.0, 18.0), natoms=3, seed=7)
+    slab = W.Slab(base.name, base.L, base.ncell, base.p, base.R, base.Z, W.Bias("cef", field=0.01))
+    om, K, M, X = _oracle(slab)
+    s = torch.cuda.Stream()
+    m = fe.Mesh(slab.L, slab.ncell, slab.p, stream=s)
+    m.set_atoms(slab.R, slab.Z)
+    m.set_poisson_precond(False)
+    x = torch.tensor(np.random.default_rng(2).standard_normal(om.n_phi).astype(np.float32), device="cuda")
+    ref = K @ x.double().cpu().numpy()
+    y = torch.zeros_like(x)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s):
+        m.poisson_apply_K(x, y)
+        g = torch.cuda.CUDAGraph()
+        s.synchronize()
+        with torch.cuda.graph(g, stream=s):
+            m.poisson_apply_K(x, y)
+        phi, _, info = m.poisson_solve(slab.bias, rtol=1e-12)
+        m.poisson_apply_K(x.double())
+        y.zero_()
+        g.replay()
+    s.synchronize()
+    assert info.status == 0
+    assert np.linalg.norm(y.double().cpu().numpy() - ref) / np.linalg.norm(ref) <= 1e-5
+    f = 4 * math.pi * M * sum(potentials.densities(X, M, slab.R, slab.Z, slab.L))
+    phi_ref = poisson.solve_cef_direct(K, f, M)
+    assert np.max(np.abs(phi.cpu().numpy() - phi_ref)) <= 1e-9 * np.max(np.abs(phi_ref))
+
+
+def test_double_cg_captures_the_cell_product(fe):
+    """FE_POISSON_F64 runs the same products in its captured iterations whether or not one was
+    made before (its scratch is taken before the capture): bitwise equal potentials."""
+    base = W.small_slab(ncell=(3, 3, 8), p=4, L=(6.0, 6.0, 18.0), natoms=3, seed=7)
+    bias = W.Bias("cef", field=0.01)
+    out = []
+    for warm in (False, True):
+        m = fe.Mesh.from_slab(base)
+        m.set_poisson_precond(False)
+        m.set_poisson_mixed(False)
+        if warm:
+            m.poisson_apply_K(torch.ones(m.n_phi, dtype=torch.float64, device="cuda"))
+        phi, _, info = m.poisson_solve(bias, rtol=1e-12)
+        assert info.status == 0
+        out.append(phi)
+    assert torch.equal(out[0], out[1])

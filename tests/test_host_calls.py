@@ -1,0 +1,81 @@
+"""What libfe asks of the CUDA runtime, call by call, checked without a GPU.
+
+A child process preloads fake_cuda.c in place of the CUDA runtime, cuBLAS and cuSOLVER and drives
+the C ABI; the log of allocations, copies and launches is then compared with what the library
+promises.  Faults that could reach the GPU (an address used after it was freed, a launch outside
+the limits, a misaligned access) are shown here and nowhere else.
+"""
+import os
+import re
+import subprocess
+import sys
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+PKG = os.path.join(os.path.dirname(HERE), "paper_2504_00998_gb300")
+
+PRELUDE = """
+import ctypes as C, importlib.util, time
+spec = importlib.util.spec_from_file_location("fe_lib", {lib!r})
+L = importlib.util.module_from_spec(spec)
+spec.loader.exec_module(L)
+lib = L.load()
+fake = C.CDLL({fake!r})
+fake.fake_log.restype = C.c_char_p
+fake.fake_fail_malloc.argtypes = [C.c_size_t]
+
+def mesh(ncell, p, L3=(4.0, 4.0, 4.0)):
+    d = L.FeMeshDesc()
+    for k in range(3):
+        d.L[k], d.ncell[k] = L3[k], ncell[k]
+    d.p = p
+    h = C.c_void_p()
+    L.call("fe_mesh_create", C.byref(d), C.byref(h))
+    return h
+
+def host(n):                    # n doubles, 16-byte aligned
+    b = C.create_string_buffer(8 * n + 16)
+    host.keep.append(b)
+    return (C.addressof(b) + 15) // 16 * 16
+host.keep = []
+
+def log():
+    return fake.fake_log().decode()
+"""
+
+
+@pytest.fixture(scope="module")
+def child(tmp_path_factory):
+    """Runs a script against the fake runtime and returns what it printed."""
+    from paper_2504_00998_gb300 import build
+    build.build()
+    so = str(tmp_path_factory.mktemp("fake") / "fake_cuda.so")
+    subprocess.run(["gcc", "-shared", "-fPIC", "-O1", "-o", so, os.path.join(HERE, "fake_cuda.c")],
+                   check=True)
+    prelude = PRELUDE.format(lib=os.path.join(PKG, "_lib.py"), fake=so)
+
+    def run(script):
+        r = subprocess.run([sys.executable, "-c", prelude + script], capture_output=True, text=True,
+                           timeout=120, env=dict(os.environ, LD_PRELOAD=so))
+        assert r.returncode == 0, r.stderr
+        return r.stdout
+
+    return run
+
+
+@pytest.mark.parametrize("p", [4, 5])
+@pytest.mark.parametrize("first", ["fe_poisson_apply_K_f32", "fe_poisson_apply_K"])
+def test_stiffness_scratch_is_never_freed(child, p, first):
+    """A graph captured around one stiffness product stays valid after the other: both keep the
+    address of their scratch for the mesh's life, in either order."""
+    out = child(f"""
+h = mesh((3, 3, 3), {p})
+x, y = host(4000), host(4000)
+fake.fake_reset()
+for name in ({first!r}, "fe_poisson_apply_K", "fe_poisson_apply_K_f32"):
+    L.call(name, h, x, y)
+print(log())
+""")
+    assert "k_cell_apply" in out and "k_cell64" in out
+    assert not re.search("^free ", out, re.M), out
