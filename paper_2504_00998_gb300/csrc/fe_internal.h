@@ -233,6 +233,9 @@ struct fe_mesh {
 
   KronCoef coefH;          // Hamiltonian (mass-scaled, 1/2 factor)
   KronCoef coefK;          // plain stiffness
+  // the caller's stream whose double stiffness products no call has waited for (fe_kcell64.cu)
+  bool kcell64_pending = false;
+  cudaStream_t kcell64_user = nullptr;
   double kx = 0.0, ky = 0.0;   // Bloch wave vector
   bool has_k = false;
 

@@ -401,11 +401,38 @@ fe_status fe_kcell64_reserve(fe_mesh* m, double** ws) {
   return FE_OK;
 }
 
-// y = K x; *done is false (nothing enqueued) when the scratch is neither there nor to be had now
-// or the grid would be too large: the caller then takes the sweep kernel, which needs no scratch
+namespace {
+
+// Whether a product enqueued now has the scratch to itself.  Products on one stream follow one
+// another, and the library's own stream follows the caller's; but after fe_mesh_set_stream the
+// former stream's products may still be running, and a graph that the caller captures may be
+// replayed on any stream.
+fe_status scratch_ours(fe_mesh* m, bool* ours) {
+  const cudaStream_t user = (cudaStream_t)m->desc.stream;
+  *ours = !m->kcell64_pending || m->kcell64_user == user;
+  if (*ours && m->stream != m->aux_stream) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    FE_CUDA(cudaStreamIsCapturing(m->stream, &cs));
+    *ours = cs == cudaStreamCaptureStatusNone;
+  }
+  if (*ours) {
+    m->kcell64_pending = true;
+    m->kcell64_user = user;
+  }
+  return FE_OK;
+}
+
+}  // namespace
+
+// y = K x; *done is false (nothing enqueued) when the scratch is neither there nor to be had now,
+// when another stream or a captured graph may use it at the same time, or when the grid would be
+// too large: the caller then takes the sweep kernel, which needs no scratch
 fe_status fe_kcell_apply_f64(fe_mesh* m, const double* x, double* y, bool* done) {
   *done = false;
   if (m->ny > 65535 || m->nz > 65535) return FE_OK;
+  bool ours = false;
+  FE_TRY(scratch_ours(m, &ours));
+  if (!ours) return FE_OK;
   double* yc = nullptr;
   FE_TRY(fe_kcell64_reserve(m, &yc));
   if (!yc) return FE_OK;

@@ -1737,6 +1737,8 @@ static fe_status poisson_solve_on(fe_mesh* m, const double* rho, const fe_poisso
   }
   FE_CUDA(cudaGetLastError());
   FE_CUDA(cudaStreamSynchronize(st));
+  // (st follows the caller's stream, so its products have run too)
+  if (m->kcell64_user == (cudaStream_t)m->desc.stream) m->kcell64_pending = false;
   double rel = bnorm2 > 0 ? std::sqrt(rr / bnorm2) : 0.0;
   bool conv = bnorm2 == 0.0 || rr <= tol2;
   if (info) {

@@ -79,3 +79,39 @@ print(log())
 """)
     assert "k_cell_apply" in out and "k_cell64" in out
     assert not re.search("^free ", out, re.M), out
+
+
+def test_stiffness_scratch_has_one_stream(child):
+    """The double product's scratch serves one stream at a time: a product on another stream, and
+    one inside the caller's capture, take the scratch-free kernel until a solve has waited for
+    the first stream's products."""
+    out = child("""
+h = mesh((2, 2, 2), 4)
+x, y = host(2000), host(2000)
+A, B = C.c_void_p(0x1000), C.c_void_p(0x2000)
+def product(stream, capture=False):
+    L.call("fe_mesh_set_stream", h, stream)
+    fake.fake_reset()
+    if capture:
+        fake.cudaStreamBeginCapture(stream, 0)
+    L.call("fe_poisson_apply_K", h, x, y)
+    if capture:
+        fake.cudaStreamEndCapture(stream, C.byref(C.c_void_p()))
+    print("cell" if "k_cell64" in log() else "sweep" if "kron_kernel" in log() else log())
+def solve(stream):
+    L.call("fe_mesh_set_stream", h, stream)
+    bc, info = L.FePoissonBC(), L.FeSolveInfo()
+    bc.kind, bc.rtol, bc.max_iter = L.FE_BIAS_CEF, 1e-10, 10
+    L.call("fe_poisson_solve_load", h, x, C.byref(bc), None, y, C.byref(info))
+product(A, capture=True)
+product(A)
+product(A, capture=True)
+product(B)
+solve(B)
+product(B)
+product(A)
+solve(A)
+product(B)
+product(A)
+""")
+    assert out.split() == ["sweep", "cell", "sweep", "sweep", "sweep", "cell", "cell", "sweep"]
