@@ -115,3 +115,21 @@ product(B)
 product(A)
 """)
     assert out.split() == ["sweep", "cell", "sweep", "sweep", "sweep", "cell", "cell", "sweep"]
+
+
+# 192 tiles of 64 columns, 257 and 341 of 48, the most columns taken (256 of 64)
+@pytest.mark.parametrize("n,tiles", [(12288, 192), (12289, 257), (16321, 341), (16384, 256)])
+def test_rayleigh_ritz_of_many_columns_launches(child, n, tiles):
+    """Every launch of a double Rayleigh-Ritz stays within the grid limits up to the widest
+    block that is accepted, and the Gram grid has every pair of column tiles."""
+    out = child(f"""
+h = mesh((16, 16, 9), 4)        # 143,360 nodes; no kernel runs, so the blocks are only addresses
+L.call("fe_set_potential", h, 0x1000)
+fake.fake_reset()
+st = lib.fe_rayleigh_ritz(h, 0x10000, {n}, {n + n % 2}, 0x1000, L.FE_F64)
+print(st, lib.fe_last_error().decode() if st else "ok")
+print(log())
+""")
+    assert out.startswith("0 ok"), out.splitlines()[0]
+    grids = [int(g) for g in re.findall(r"^launch \S*k_gram_partial\S* (\d+) 1 1 ", out, re.M)]
+    assert grids and all(g == tiles * tiles for g in grids)
