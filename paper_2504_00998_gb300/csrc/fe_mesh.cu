@@ -395,9 +395,8 @@ extern "C" fe_status fe_lumped_mass(const fe_mesh* m, double* out) {
   return FE_OK;
 }
 
-// both copies of the potential in one launch
-__global__ void k_set_potential(const double* __restrict__ v, double* __restrict__ d,
-                                float* __restrict__ f, int64_t n) {
+// both copies of the potential in one launch (v may be d itself)
+__global__ void k_set_potential(const double* v, double* d, float* __restrict__ f, int64_t n) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i < n) {
     const double x = v[i];
@@ -415,6 +414,18 @@ extern "C" fe_status fe_set_potential(fe_mesh* m, const double* veff) {
       cudaGetLastError();
       return fe_fail(FE_ENOMEM, "potential allocation failed");
     }
+  }
+  // The kernel reads veff itself where that is aligned memory of this device; an array of
+  // another device, of the host, or off its alignment is copied first.
+  cudaPointerAttributes at;
+  const bool direct = (uintptr_t)veff % sizeof(double) == 0 &&
+                      cudaPointerGetAttributes(&at, veff) == cudaSuccess &&
+                      at.type == cudaMemoryTypeDevice && at.device == m->device;
+  if (!direct) {
+    cudaGetLastError();
+    FE_CUDA(cudaMemcpyAsync(m->d_veff, veff, m->n_psi * sizeof(double), cudaMemcpyDeviceToDevice,
+                            m->stream));
+    veff = m->d_veff;
   }
   int nb = (int)((m->n_psi + 255) / 256);
   k_set_potential<<<nb, 256, 0, m->stream>>>(veff, m->d_veff, m->d_veff_f, m->n_psi); fe_count_launch();

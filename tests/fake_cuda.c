@@ -59,6 +59,16 @@ int cudaFree(void* p) {
     }
   return fail(E_VALUE);
 }
+/* addresses below 1 << 20 belong to no memory, those below 1 << 24 to device 1, others to device 0 */
+typedef struct { int type, device; void *dev, *host; long reserved[8]; } PointerAttributes;
+int cudaPointerGetAttributes(PointerAttributes* a, const void* p) {
+  memset(a, 0, sizeof *a);
+  if ((uintptr_t)p < 1u << 20) return OK;
+  a->type = 2;
+  a->device = (uintptr_t)p < 1u << 24;
+  a->dev = (void*)p;
+  return OK;
+}
 int cudaHostAlloc(void** p, size_t n, unsigned f) { (void)f; *p = calloc(1, n); return *p ? OK : fail(E_NOMEM); }
 int cudaFreeHost(void* p) { free(p); return OK; }
 int cudaMemcpyAsync(void* d, const void* s, size_t n, int kind, void* st) {

@@ -310,3 +310,17 @@ def test_rayleigh_ritz_gram_sizes(fe, n):
     assert np.max(np.abs(Q.T @ Q - np.eye(n))) <= 1e-10
     assert np.max(np.abs(Q.T @ (H @ Q) - np.diag(lam))) <= 1e-9
     assert torch.all(buf[:, n:] == 0.0)
+
+
+def test_set_potential_from_unaligned_array(fe):
+    """A potential that starts off its 8-byte alignment is copied bytewise: the same Ht X."""
+    om, H, m, rng = _setup(fe, (4.0, 4.0, 9.0), (2, 2, 4), 3, (True, True))
+    V = torch.tensor(rng.uniform(-1.0, 1.0, om.n_psi), device="cuda")
+    X = torch.tensor(rng.standard_normal((om.n_psi, 4)), device="cuda")
+    m.set_potential(V)
+    ref = m.apply_H(X)
+    raw = torch.zeros(8 * om.n_psi + 8, dtype=torch.uint8, device="cuda")
+    raw[4:4 + 8 * om.n_psi] = V.view(torch.uint8)
+    m.set_potential(torch.zeros_like(V))
+    fe.call("fe_set_potential", m.handle, raw.data_ptr() + 4)
+    assert torch.equal(m.apply_H(X), ref)

@@ -133,3 +133,18 @@ print(log())
     assert out.startswith("0 ok"), out.splitlines()[0]
     grids = [int(g) for g in re.findall(r"^launch \S*k_gram_partial\S* (\d+) 1 1 ", out, re.M)]
     assert grids and all(g == tiles * tiles for g in grids)
+
+
+# memory of this device, off its alignment, of another device, unknown to CUDA (fake_cuda.c)
+@pytest.mark.parametrize("veff,copied", [(1 << 25, False), ((1 << 25) + 4, True), (1 << 22, True),
+                                         (1 << 16, True)])
+def test_set_potential_copies_what_a_kernel_must_not_read(child, veff, copied):
+    out = child(f"""
+h = mesh((2, 2, 2), 3)
+fake.fake_reset()
+L.call("fe_set_potential", h, {veff})
+print(log())
+""")
+    copies = re.findall(r"^copy 3 \S+ (\S+) ", out, re.M)
+    assert copies == ([hex(veff)] if copied else []), out
+    assert "k_set_potential" in out
