@@ -148,3 +148,24 @@ print(log())
     copies = re.findall(r"^copy 3 \S+ (\S+) ", out, re.M)
     assert copies == ([hex(veff)] if copied else []), out
     assert "k_set_potential" in out
+
+
+# 65,535 and 65,536 tiles of eight 16-byte groups, and the 65,535 tiles of 128 vectors that the
+# term once took
+@pytest.mark.parametrize("prec,nvec", [("FE_F64", 16 * 65535), ("FE_F64", 16 * 65535 + 1),
+                                       ("FE_F32", 32 * 65535 + 1), ("FE_F32", 128 * 65535)])
+def test_nonlocal_term_of_many_vectors_launches(child, prec, nvec):
+    out = child(f"""
+h = mesh((1, 1, 2), 1)
+L.call("fe_set_potential", h, 1 << 25)
+one = (C.c_double * 6)(*[2.0] * 6)
+L.call("fe_set_nonlocal", h, 2, one, one, (C.c_double * 8)(*[1.0] * 8), 3.0)
+ld = ({nvec} + 3) // 4 * 4
+fake.fake_reset()
+st = lib.fe_apply_H(h, 1 << 32, 1 << 40, {nvec}, ld, L.{prec})
+print(st, lib.fe_last_error().decode() if st else "ok")
+print(log())
+""")
+    assert out.startswith("0 ok"), out.splitlines()[0]
+    tiles = -(-nvec // (16 if prec == "FE_F64" else 32))
+    assert re.search(rf"k_nl_project\S* {2 * tiles} 1 1 256 ", out)
