@@ -554,7 +554,8 @@ k_sep_direction(double* __restrict__ p, const double* __restrict__ z, int64_t n,
     p[i] = fma(beta, p[i], z[i]);
 }
 
-// p.q; the last block takes alpha = r.z / p.q
+// p.q; the last block takes alpha = r.z / p.q, or zero when that is no step: a residual outside
+// the floats' range makes z zero or not finite, and nothing of it must reach phi
 __global__ void __launch_bounds__(256)
 k_sep_dot(const double* __restrict__ p, const double* __restrict__ q, int64_t n,
           double* __restrict__ part, Scalars* s) {
@@ -566,11 +567,14 @@ k_sep_dot(const double* __restrict__ p, const double* __restrict__ q, int64_t n,
   if (threadIdx.x == 0) part[blockIdx.x] = v;
   if (last_block(&s->ticket[1], gridDim.x)) {
     const double pq = sum_partials(part, gridDim.x);
-    if (threadIdx.x == 0) s->alpha = pq != 0.0 ? s->rz / pq : 0.0;
+    if (threadIdx.x == 0) {
+      const double a = s->rz / pq;
+      s->alpha = isfinite(a) && isfinite(pq) ? a : 0.0;
+    }
   }
 }
 
-// phi += alpha p, r -= alpha q on free nodes (p is zero elsewhere); |r|^2
+// phi += alpha p, r -= alpha q on free nodes (p is zero elsewhere), nothing for alpha = 0; |r|^2
 __global__ void __launch_bounds__(256)
 k_sep_update(double* __restrict__ phi, double* __restrict__ r, const double* __restrict__ p,
              const double* __restrict__ q, const unsigned char* __restrict__ mask, int64_t n,
@@ -579,9 +583,12 @@ k_sep_update(double* __restrict__ phi, double* __restrict__ r, const double* __r
   double v = 0.0;
 #pragma unroll 4
   for (int64_t i = blockIdx.x * (int64_t)256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
-    phi[i] = fma(alpha, p[i], phi[i]);
-    const double x = mask[i] ? 0.0 : fma(-alpha, q[i], r[i]);
-    r[i] = x;
+    double x = mask[i] ? 0.0 : r[i];
+    if (alpha != 0.0) {
+      phi[i] = fma(alpha, p[i], phi[i]);
+      if (!mask[i]) x = fma(-alpha, q[i], x);
+      r[i] = x;
+    }
     v = fma(x, x, v);
   }
   v = block_total(v);
@@ -722,12 +729,14 @@ fe_status solve(fe_mesh* m, const Buf& b, double tol2, int maxit, double* rr, in
     k_sep_update<<<VEC_BLOCKS, 256, 0, st>>>(b.phi, b.r, b.p, b.q, b.mask, n, part, s);
     fe_count_launch();
     FE_CUDA(cudaGetLastError());
-    FE_CUDA(cudaMemcpyAsync(rr, &s->rr, sizeof(double), cudaMemcpyDeviceToHost, st));
+    Scalars h;
+    FE_CUDA(cudaMemcpyAsync(&h, s, sizeof h, cudaMemcpyDeviceToHost, st));
     FE_CUDA(cudaStreamSynchronize(st));
+    *rr = h.rr;
     *iters = it + 1;
-    // no progress over thirty iterations, or a breakdown: hand the solve back
+    // no progress over thirty iterations, or no step at all: hand the solve back
     if (*rr < 0.25 * best) { best = *rr; since = 0; } else { ++since; }
-    if (!std::isfinite(*rr) || since >= 30) { *lost = true; break; }
+    if (h.alpha == 0.0 || since >= 30) { *lost = true; break; }
   }
   return FE_OK;
 }

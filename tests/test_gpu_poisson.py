@@ -451,3 +451,29 @@ def test_double_cg_captures_the_cell_product(fe):
         assert info.status == 0
         out.append(phi)
     assert torch.equal(out[0], out[1])
+
+
+# loads inside the floats' range, above it, and below it
+@pytest.mark.parametrize("scale", [1e25, 1e42, 1e-30, 1e-46])
+@pytest.mark.parametrize("kind", ["cef", "cpd"])
+def test_default_solve_of_scaled_loads(fe, kind, scale):
+    """The problem is linear: a load outside the range of the float preconditioner is handed to
+    the other iterations and solved, with the bound of test_separable_preconditioner."""
+    L = (9.0, 9.0, 14.0)
+    om = OMesh(L, (4, 4, 4), 4)
+    K, M = assembly.assemble_stiffness(om), assembly.lumped_mass(om)
+    f = np.random.default_rng(3).standard_normal(om.n_phi) * M
+    assert om.n_phi >= 4096
+    m = fe.Mesh(L, (4, 4, 4), 4)
+    m.set_atoms(np.zeros((0, 3)), np.zeros(0))
+    if kind == "cef":
+        bias = W.Bias("cef", field=0.01)
+        ref = poisson.solve_cef_direct(K, f, M)
+    else:
+        bias = W.Bias("cpd", dV=0.0, zA=0.0, zB=L[2])
+        mask = m.poisson_constraints(bias)[0].cpu().numpy()
+        ref = poisson.solve_cpd_direct(K, f, mask, np.zeros(om.n_phi))
+    phic = None if kind == "cef" else torch.zeros(om.n_phi, dtype=torch.float64, device="cuda")
+    phi, info = m.poisson_solve_load(torch.tensor(scale * f, device="cuda"), bias, phic=phic, rtol=1e-12)
+    assert info.status == 0 and info.rel_residual <= 1e-12
+    assert np.max(np.abs(phi.cpu().numpy() / scale - ref)) <= 1e-9 * np.max(np.abs(ref))
