@@ -1636,9 +1636,18 @@ static fe_status poisson_solve_on(fe_mesh* m, const double* rho, const fe_poisso
       // the float work area (6 n floats) holds the two transform arrays and the partials
       double* part = (double*)(((uintptr_t)(fl + 2 * n) + 15) & ~(uintptr_t)15);
       const fe_sep::Buf sb{phi, r, z, p, q, mask, fl, fl + n, part};
+      // The iteration stops on its recurrence r -= alpha q, which rounding takes away from
+      // f - K phi: the stopping test is on the latter.  Where it has not been met the iteration
+      // starts again from it, as long as that halves it; the iterations below take over then.
       bool lost = false;
-      FE_TRY(fe_sep::solve(m, sb, tol2, bc->max_iter, &rr, &used, &lost));
-      if (lost) FE_TRY(residual(&rr));
+      double before = 0.0;
+      do {
+        before = rr;
+        int its = 0;
+        FE_TRY(fe_sep::solve(m, sb, tol2, bc->max_iter - used, &rr, &its, &lost));
+        used += its;
+        FE_TRY(residual(&rr));
+      } while (!lost && rr > tol2 && rr <= 0.25 * before && used < bc->max_iter);
     }
   }
   // coarse space of z-planes for the iterations below (z and q serve as scratch before they

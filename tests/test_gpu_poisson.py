@@ -477,3 +477,25 @@ def test_default_solve_of_scaled_loads(fe, kind, scale):
     phi, info = m.poisson_solve_load(torch.tensor(scale * f, device="cuda"), bias, phic=phic, rtol=1e-12)
     assert info.status == 0 and info.rel_residual <= 1e-12
     assert np.max(np.abs(phi.cpu().numpy() / scale - ref)) <= 1e-9 * np.max(np.abs(ref))
+
+
+# smooth load on a long chain: rounding of K phi stays far above the recurrence's last residual
+@pytest.mark.parametrize("p,ncell,rtol", [(4, (4, 4, 40), 1e-10), (5, (3, 3, 30), 1e-11), (6, (3, 3, 24), 1e-10)])
+def test_default_solve_reports_the_residual_of_phi(fe, p, ncell, rtol):
+    """rel_residual of the default solve is that of the returned potential, |f - K phi| over the
+    free nodes relative to its value at the start, to a tenth."""
+    L = (2.0 * ncell[0], 2.0 * ncell[1], 2.0 * ncell[2])
+    m = fe.Mesh(L, ncell, p)
+    m.set_atoms(np.zeros((0, 3)), np.zeros(0))
+    X = m.node_coords()
+    f = m.lumped_mass() * torch.sin(math.pi * X[:, 2] / L[2])
+    bias = W.Bias("cpd", dV=0.5, zA=0.0, zB=L[2])
+    mask, vals = m.poisson_constraints(bias)
+    phi, info = m.poisson_solve_load(f, bias, phic=vals, rtol=rtol)
+    assert info.status == 0 and info.rel_residual <= rtol
+
+    def residual(x):
+        return torch.linalg.vector_norm((f - m.poisson_apply_K(x))[~mask]).item()
+
+    true = residual(phi) / residual(torch.where(mask, vals, torch.zeros_like(vals)))
+    assert abs(info.rel_residual - true) <= 0.1 * true, (info.rel_residual, true)
