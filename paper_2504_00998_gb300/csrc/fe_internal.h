@@ -291,7 +291,6 @@ struct fe_mesh {
   int sep_state = 0;
   fe_poisson_bc sep_key = {};
   int sep_lo = 0, sep_hi = 0;
-  float sep_null = 0.f;
 
   // tensor-core path: p of the uploaded cell-matrix image, pinned wait-expiry flag
   int tc_img_p = -1;

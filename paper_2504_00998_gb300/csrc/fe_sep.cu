@@ -290,10 +290,9 @@ struct Gemm {
   int M, N, K;
   int64_t in_batch, out_batch;
   // spectral scaling (left products of the z direction): rows are z modes, a column is
-  // b NX + a
+  // b NX + a; the part of eigenvalue zero, the constant's, is dropped
   const float *lx, *ly, *lz;
   int NX;
-  float null_below;      // eigenvalues at or below this are the null space: their part is dropped
   // double ends of the x products
   const double* in_d;
   double* out_d;
@@ -482,7 +481,7 @@ __global__ void __launch_bounds__(GT) k_sep_gemm_z(const Gemm g) {
       if constexpr (MODE == LEFT_SCALE) {
         const int bb = nn / g.NX, aa = nn - bb * g.NX;
         const float l = g.lz[mm] + (g.ly[bb] + g.lx[aa]);
-        v = l > g.null_below ? v / l : 0.f;
+        v = l > 0.f ? v / l : 0.f;
       }
       g.out[(int64_t)mm * g.N + nn] = v;
     }
@@ -631,7 +630,6 @@ fe_status plan(fe_mesh* m, const double* cnt, bool constant_null) {
   const double scale[3] = {m->h[1] * m->h[2] / (2.0 * m->h[0]), m->h[0] * m->h[2] / (2.0 * m->h[1]),
                            m->h[0] * m->h[1] / (2.0 * m->h[2])};
   std::vector<float> host;
-  double top = 0.0;
   std::vector<float> lam_f[3];
   for (int d = 0; d < 3; ++d) {
     std::vector<double> lam;
@@ -646,12 +644,12 @@ fe_status plan(fe_mesh* m, const double* cnt, bool constant_null) {
         host[at + (size_t)i * n[d] + a] = (float)V[(size_t)a * n[d] + i];   // V [node][mode]
         host[at + nn + (size_t)a * n[d] + i] = (float)V[(size_t)a * n[d] + i];
       }
-    double mx = 0.0;
-    for (double l : lam) {
-      mx = std::max(mx, scale[d] * l);
-      lam_f[d].push_back((float)(scale[d] * l));
-    }
-    top += mx;
+    // The constant is an eigenvector of every chain without a constrained end, and its
+    // eigenvalue zero comes out at rounding level: set to zero, the sum over the directions is zero
+    // for the constant alone, however different the cell lengths (a threshold on the sum
+    // dropped the slow modes along cells 80 times longer than wide).
+    if (d < 2 || constant_null) *std::min_element(lam.begin(), lam.end()) = 0.0;
+    for (double l : lam) lam_f[d].push_back((float)(scale[d] * l));
   }
   for (int d = 0; d < 3; ++d) host.insert(host.end(), lam_f[d].begin(), lam_f[d].end());
   void* w = nullptr;
@@ -661,9 +659,6 @@ fe_status plan(fe_mesh* m, const double* cnt, bool constant_null) {
   FE_CUDA(cudaStreamSynchronize(m->stream));
   m->sep_lo = lo;
   m->sep_hi = hi;
-  // the zero eigenvalue of the constant comes out at rounding level; the next one is at least
-  // (pi / Lz)^2 against (p^2 / h)^2, above 1e-9 of the largest for every chain taken here
-  m->sep_null = constant_null ? (float)(1e-10 * top) : 0.f;
   m->sep_state = 1;
   return FE_OK;
 }
@@ -707,7 +702,7 @@ fe_status solve(fe_mesh* m, const Buf& b, double tol2, int maxit, double* rr, in
     FE_TRY(gemm<LEFT>(g, nz, st));
     g = {};
     g.W = t.Vz; g.in = b.tb; g.out = b.ta; g.M = nz; g.N = (int)plane; g.K = nz;
-    g.lx = t.lx; g.ly = t.ly; g.lz = t.lz; g.NX = NX; g.null_below = m->sep_null;
+    g.lx = t.lx; g.ly = t.ly; g.lz = t.lz; g.NX = NX;
     FE_TRY(gemm_z<LEFT_SCALE>(g, st));
     g = {};
     g.W = t.VzT; g.in = b.ta; g.out = b.tb; g.M = nz; g.N = (int)plane; g.K = nz;
