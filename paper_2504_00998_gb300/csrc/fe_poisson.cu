@@ -1628,8 +1628,11 @@ static fe_status poisson_solve_on(fe_mesh* m, const double* rho, const fe_poisso
       k_plane_sum<double><<<nzp, fe::RED_THREADS, 0, st>>>(nullptr, mask, plane_n, z); fe_count_launch();
       FE_CUDA(cudaMemcpyAsync(hcnt.data(), z, sizeof(double) * nzp, cudaMemcpyDeviceToHost, st));
       FE_CUDA(cudaStreamSynchronize(st));
-      m->sep_state = 0;
-      FE_TRY(fe_sep::plan(m, hcnt.data(), project));
+      // (a plan that fails leaves none; without memory for its tables the iterations below, which
+      // do not need them, solve)
+      const fe_status planned = fe_sep::plan(m, hcnt.data(), project);
+      if (planned != FE_OK) m->sep_state = 0;
+      if (planned != FE_OK && planned != FE_ENOMEM) return planned;
       m->sep_key = *bc;
     }
     if (m->sep_state == 1) {

@@ -1,6 +1,6 @@
 /* Host stand-in for the CUDA runtime, cuBLAS and cuSOLVER entry points that libfe imports,
  * preloaded by test_host_calls.py: no kernel runs and no GPU is needed.  Every call is written
- * to a log; allocations are zero-filled host memory, copies to and from the host are made, and a
+ * to a log; allocations are host memory of one byte value, copies to and from the host are made, and a
  * launch outside CUDA's documented grid and block limits is refused as the runtime refuses it. */
 #define _GNU_SOURCE
 #include <stdarg.h>
@@ -17,6 +17,7 @@ static char* log_buf;
 static size_t log_len, log_cap;
 static int last_error;
 static size_t fail_bytes;        /* allocations of this size fail */
+static int fill;                 /* byte that new allocations hold */
 static void* capturing;          /* the stream under capture */
 
 static void note(const char* fmt, ...) {
@@ -33,6 +34,7 @@ static int fail(int e) { return last_error = e; }
 const char* fake_log(void) { return log_buf ? log_buf : ""; }
 void fake_reset(void) { log_len = 0; if (log_buf) log_buf[0] = 0; }
 void fake_fail_malloc(size_t bytes) { fail_bytes = bytes; }
+void fake_fill(int byte) { fill = byte; }
 
 /* ---- memory ---- */
 static struct { void* p; size_t n; } blocks[4096];
@@ -42,6 +44,7 @@ int cudaMalloc(void** p, size_t n) {
   if (fail_bytes && n == fail_bytes) { note("nomem %zu", n); return fail(E_NOMEM); }
   void* q = mmap(NULL, n ? n : 1, PROT_READ | PROT_WRITE, MAP_PRIVATE | MAP_ANONYMOUS | MAP_NORESERVE, -1, 0);
   if (q == MAP_FAILED || nblocks == 4096) return fail(E_NOMEM);
+  if (fill) memset(q, fill, n);
   blocks[nblocks].p = q;
   blocks[nblocks++].n = n ? n : 1;
   note("malloc %p %zu", q, n);

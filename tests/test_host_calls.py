@@ -169,3 +169,29 @@ print(log())
     assert out.startswith("0 ok"), out.splitlines()[0]
     tiles = -(-nvec // (16 if prec == "FE_F64" else 32))
     assert re.search(rf"k_nl_project\S* {2 * tiles} 1 1 256 ", out)
+
+
+def test_solve_without_memory_for_the_eigenbases(child):
+    """The default solve needs the tables of the separable preconditioner for speed only: when
+    they cannot be allocated the other iterations solve, and the next solve tries again.  (The
+    bytes 0x40 read as 32.5 everywhere, so the residual is above the tolerance and planes count
+    as free; 4 x 4 x 4 cells of p = 4 are chains of 16, 16 and 17 nodes.)"""
+    out = child("""
+fake.fake_fill(0x40)
+h = mesh((4, 4, 4), 4)
+x, y = host(4352), host(4352)
+tables = 4 * (2 * (16 * 16 + 16 * 16 + 17 * 17) + 16 + 16 + 17)
+def solve():
+    fake.fake_reset()
+    bc, info = L.FePoissonBC(), L.FeSolveInfo()
+    bc.kind, bc.rtol, bc.max_iter = L.FE_BIAS_CEF, 1e-3, 32
+    st = lib.fe_poisson_solve_load(h, x, C.byref(bc), None, y, C.byref(info))
+    print(st, f" {tables}\\n" in log(), "k_sep_gemm" in log(), "graph" in log())
+fake.fake_fail_malloc(tables)
+solve()
+solve()
+fake.fake_fail_malloc(0)
+solve()
+""")
+    assert out.splitlines()[:2] == ["0 True False True"] * 2, out
+    assert out.splitlines()[2].split()[1:3] == ["True", "True"], out
