@@ -105,14 +105,14 @@ enum { FE_RR_PRODUCTS_F64 = 0, FE_RR_PRODUCTS_TC32 = 1 };
  *     factorised once per solve.  It removes the slow modes that are constant over x and y,
  *     which dominate on long slabs.  The converged solution is the same; only the
  *     iteration count changes. */
-/*     Until this option is set, solves in FE_POISSON_MIXED arithmetic on meshes of at least
- *     2048 phi nodes use a separable preconditioner instead: K on the planes that hold free
- *     nodes is diagonal in the eigenbasis of the one-dimensional element matrices, so its
- *     inverse is six small products along the axes (in float), inside a CG in double.  It
- *     takes two or three iterations (about twenty with an L-CPD patch); the eigenbases are
- *     built once per mesh and constraint set.  Setting any value selects the iterations
- *     described here. */
-/*     FE_PRECOND_JACOBI_PLANES_MODES (default where that does not apply): the plane coarse space enriched, on every
+/*     FE_PRECOND_SEPARABLE (default): K on the planes that hold free nodes is diagonal in the
+ *     eigenbasis of the one-dimensional element matrices, so its inverse is six small products
+ *     along the axes (in float), inside a CG in double.  It takes two or three iterations (about
+ *     twenty with an L-CPD patch); the eigenbases are built once per mesh and constraint set.
+ *     Used by solves in FE_POISSON_MIXED arithmetic with FE_POISSON_ITER_PERSISTENT on meshes
+ *     of at least 2048 phi nodes and at most 512 a direction; elsewhere, and where that CG
+ *     makes no more progress, FE_PRECOND_JACOBI_PLANES_MODES. */
+/*     FE_PRECOND_JACOBI_PLANES_MODES: the plane coarse space enriched, on every
  *     plane, with the in-plane Fourier modes of wavenumber one (cos and sin of 2 pi x / Lx
  *     and of 2 pi y / Ly on the plane's nodes); on a mesh without constrained phi nodes (the
  *     CEF setup) they are decoupled from one another by the cell-translation invariance of
@@ -121,7 +121,8 @@ enum { FE_RR_PRODUCTS_F64 = 0, FE_RR_PRODUCTS_TC32 = 1 };
  *     both x and y (on narrower slabs these modes are not slow ones) and the planes hold a
  *     multiple of four nodes along x; elsewhere it acts as FE_PRECOND_JACOBI_PLANES.  Built
  *     once per mesh and constraint set (4 x (2p + 1) more double operator applications). */
-enum { FE_PRECOND_JACOBI = 0, FE_PRECOND_JACOBI_PLANES = 1, FE_PRECOND_JACOBI_PLANES_MODES = 2 };
+enum { FE_PRECOND_JACOBI = 0, FE_PRECOND_JACOBI_PLANES = 1, FE_PRECOND_JACOBI_PLANES_MODES = 2,
+       FE_PRECOND_SEPARABLE = 3 };
 /*   FE_OPT_POISSON_ARITH: arithmetic of the Poisson solve.  FE_POISSON_F64: CG in double.
  *     FE_POISSON_MIXED (default): a float CG (operator, vectors and preconditioner in float,
  *     dot products accumulated in double) with reliable updates -- whenever its residual has

@@ -263,10 +263,8 @@ struct fe_mesh {
   int rr_eigen = 0;                 // FE_RR_EIGEN_SYEVD / FE_RR_EIGEN_SYEVJ
   syevjInfo_t syevj_params = nullptr;
   // Poisson CG preconditioner: 0 Jacobi, 1 Jacobi plus the exact z-plane coarse solve, 2 with
-  // the in-plane modes; precond_set once the caller has chosen one (else the solve takes the
-  // separable preconditioner where it pays)
-  int poisson_precond = 2;          // FE_PRECOND_JACOBI_PLANES_MODES
-  bool precond_set = false;
+  // the in-plane modes, 3 separable (2 where that does not apply)
+  int poisson_precond = 3;          // FE_PRECOND_SEPARABLE
   // Poisson arithmetic: 0 double CG, 1 float corrections with double residuals
   int poisson_arith = 1;
   int poisson_iter = 0;             // FE_POISSON_ITER_PERSISTENT / FE_POISSON_ITER_LAUNCHES

@@ -343,10 +343,9 @@ extern "C" fe_status fe_set_option(fe_mesh* m, int option, int64_t value) {
       return FE_OK;
     case FE_OPT_POISSON_PRECOND:
       if (value != FE_PRECOND_JACOBI && value != FE_PRECOND_JACOBI_PLANES &&
-          value != FE_PRECOND_JACOBI_PLANES_MODES)
+          value != FE_PRECOND_JACOBI_PLANES_MODES && value != FE_PRECOND_SEPARABLE)
         return fe_fail(FE_EINVAL, "fe_set_option: bad Poisson preconditioner");
       m->poisson_precond = (int)value;
-      m->precond_set = true;
       return FE_OK;
     case FE_OPT_POISSON_ARITH:
       if (value != FE_POISSON_F64 && value != FE_POISSON_MIXED)

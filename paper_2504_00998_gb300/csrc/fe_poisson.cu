@@ -12,10 +12,10 @@
 //   and dV - (V_loc - V_sm) on Omega_1 = {z >= zB} (intersected with the patch for L-CPD);
 //   CG runs on the free nodes with the constrained rows and columns masked; V_app = 0.
 //
-// By default (no preconditioner chosen by the caller) the solve is a CG in double with the
-// separable preconditioner of fe_sep.cu, two or three iterations long; the iterations below
-// take over where it does not apply (a constraint set without a separable form, tiny meshes,
-// the double-arithmetic and launch-per-step options) or stops making progress.
+// By default the solve is a CG in double with the separable preconditioner of fe_sep.cu, two or
+// three iterations long; the iterations below take over where the caller chose another
+// preconditioner, where it does not apply (a constraint set without a separable form, tiny
+// meshes, the double-arithmetic and launch-per-step options) or stops making progress.
 //
 // Every CG iteration below is a fixed sequence of stream-ordered launches with all scalars on the
 // device; a block of iterations is captured once into a CUDA graph and replayed, and the
@@ -1093,13 +1093,11 @@ static fe_status coarse_setup(fe_mesh* m, const fe_poisson_bc* bc, const unsigne
   *Amodes = nullptr;
   *mtab = nullptr;
   const int nz = m->NZ;
-  if ((m->poisson_precond != FE_PRECOND_JACOBI_PLANES &&
-       m->poisson_precond != FE_PRECOND_JACOBI_PLANES_MODES) || nz > 2048)
-    return FE_OK;
+  if (m->poisson_precond == FE_PRECOND_JACOBI || nz > 2048) return FE_OK;
   // (the wavenumber-one modes are slow modes of the Jacobi-preconditioned operator only when
   // the slab spans many cells in x and y; on narrow slabs they would only add to the top of
   // the preconditioned spectrum)
-  const bool want_modes = m->poisson_precond == FE_PRECOND_JACOBI_PLANES_MODES &&
+  const bool want_modes = m->poisson_precond != FE_PRECOND_JACOBI_PLANES &&
                           m->nx >= MODES_MIN_CELLS && m->ny >= MODES_MIN_CELLS;
   const int64_t plane = (int64_t)m->NX * m->NY, n = m->n_phi;
   void* wsp;
@@ -1576,7 +1574,8 @@ static fe_status poisson_solve_on(fe_mesh* m, const double* rho, const fe_poisso
   PGeom g = make_geom(m);
 
   // (the separable preconditioner does not use the Jacobi inverse: forty FP64 operations a node)
-  const bool separable = mixed && use_graph && n >= SEP_MIN_NODES && !m->precond_set &&
+  const bool separable = mixed && use_graph && n >= SEP_MIN_NODES &&
+                         m->poisson_precond == FE_PRECOND_SEPARABLE &&
                          m->poisson_iter == FE_POISSON_ITER_PERSISTENT && m->cg_stall < 0 &&
                          fe_sep::supported(m);
   k_setup<<<gb, 256, 0, st>>>(g, *bc, m->d_mass, rh, m->d_b, m->d_vlms, f_ext, phic_ext, f,

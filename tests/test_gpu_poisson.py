@@ -515,3 +515,20 @@ def test_separable_unequal_cells(fe, p, ncell, h):
     f = m.lumped_mass() * torch.tensor(np.random.default_rng(9).standard_normal(m.n_phi), device="cuda")
     phi, info = m.poisson_solve_load(f, W.Bias("cef", field=0.0), rtol=1e-4)
     assert info.status == 0 and info.iters <= 6, info.iters
+
+
+def test_default_preconditioner_can_be_set_again(fe):
+    """After another preconditioner the default one comes back: the same iterations and bits as
+    on a fresh mesh; values without a meaning stay refused."""
+    base = W.small_slab(ncell=(4, 4, 8), p=3, L=(8.0, 8.0, 18.0), natoms=3, seed=7)
+    bias = W.Bias("cef", field=0.01)
+    m = fe.Mesh.from_slab(base)
+    phi, _, info = m.poisson_solve(bias, rtol=1e-12)
+    m.set_poisson_precond(True, modes=True)
+    other = m.poisson_solve(bias, rtol=1e-12)[2].iters
+    m.reset_poisson_precond()
+    again, _, info2 = m.poisson_solve(bias, rtol=1e-12)
+    assert info2.iters == info.iters < other and torch.equal(phi, again)
+    for value in (-1, 4):
+        with pytest.raises(fe.FeError):
+            fe.call("fe_set_option", m.handle, fe._lib.FE_OPT_POISSON_PRECOND, value)
