@@ -705,12 +705,13 @@ inline int sweep_zseg(int64_t base, int nz) {
   const double alone = sizeof(T) == 8 ? 1.0 : 1.5;
   int best = nz;
   double cost = 1e300;
-  for (int s = 1; s <= nz; ++s) {
+  for (int s = 1; s <= nz;) {
     const int z = (nz + s - 1) / s, segs = (nz + z - 1) / z;
     const double per = std::max(alone, (double)((base * segs + sms - 1) / sms));
     const double t = (z + (segs > 1 ? 1 : 0)) * per;
     if (t < cost * (1.0 - 1e-9)) { cost = t; best = z; }
     if (z == 1) break;
+    s = (nz + z - 2) / (z - 1);   // the next shorter segment: 2 sqrt(nz) lengths, not nz
   }
   return best;
 }

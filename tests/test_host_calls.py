@@ -195,3 +195,30 @@ solve()
 """)
     assert out.splitlines()[:2] == ["0 True False True"] * 2, out
     assert out.splitlines()[2].split()[1:3] == ["True", "True"], out
+
+
+@pytest.mark.parametrize("nz", [1, 7, 96, 1000, 4001, 2000000])
+def test_segment_rule_of_long_slabs(child, nz):
+    """The z segments of a launch are those of least (layers + 1) x CTAs an SM over every segment
+    count, found without trying each: a launch on two million layers takes well under the 20 ms
+    that trying them took."""
+    out = child(f"""
+h = mesh((1, 1, {nz}), 2)
+L.call("fe_set_potential", h, 1 << 25)
+best = 1.0
+for _ in range(5):
+    fake.fake_reset()
+    t0 = time.perf_counter()
+    L.call("fe_apply_H", h, 1 << 32, 1 << 40, 16, 16, L.FE_F32)
+    best = min(best, time.perf_counter() - t0)
+print(best)
+print(log())
+""")
+    def cost(s):
+        z = -(-nz // s)
+        segs = -(-nz // z)
+        return (z + (segs > 1)) * max(1.5, -(-segs // 152)), s, segs
+
+    segs = min(map(cost, range(1, min(nz, 20000) + 1)))[2]
+    assert int(re.search(r"sweep_kernel\S* (\d+) 1 1 ", out).group(1)) == segs
+    assert float(out.split()[0]) < 2e-3
