@@ -1241,10 +1241,9 @@ extern "C" fe_status fe_poisson_solve_load(fe_mesh* m, const double* f, const fe
 }
 
 // Meshes of at least this many phi nodes take the separable preconditioner unless the caller has
-// chosen another.  It is the faster one at every size measured (rtol 1e-12, CEF): 3,600 nodes
-// 0.31 ms against 3.6 ms, 50,176 nodes 0.34 against 6.5, 1.54 M nodes 1.2 against 28.6; the line
-// only keeps the coarse-space CG, with its iteration count and cap, on the few-hundred-node
-// meshes whose callers count iterations.
+// chosen another.  It is the faster one at every size measured (rtol 1e-12, CEF): SEPFIG; the
+// line is no measured crossing, it only keeps the coarse-space CG, with its iteration count and
+// cap, on the smallest meshes, whose callers may count iterations.
 constexpr int64_t SEP_MIN_NODES = 2048;
 
 // ---- preconditioned CG in a given vector precision -------------------------------------------
@@ -1577,7 +1576,9 @@ static fe_status poisson_solve_on(fe_mesh* m, const double* rho, const fe_poisso
   const bool separable = mixed && use_graph && n >= SEP_MIN_NODES &&
                          m->poisson_precond == FE_PRECOND_SEPARABLE &&
                          m->poisson_iter == FE_POISSON_ITER_PERSISTENT && m->cg_stall < 0 &&
-                         fe_sep::supported(m);
+                         fe_sep::supported(m) &&
+                         // (the partials share the float work area with two transform arrays)
+                         sizeof(double) * fe_sep::part_doubles(m) + 16 <= 4 * sizeof(float) * (size_t)n;
   k_setup<<<gb, 256, 0, st>>>(g, *bc, m->d_mass, rh, m->d_b, m->d_vlms, f_ext, phic_ext, f,
                               separable ? nullptr : dinv, mask, phi, n); fe_count_launch();
   if (project) {

@@ -611,7 +611,9 @@ bool supported(const fe_mesh* m) {
 }
 
 size_t part_doubles(const fe_mesh* m) {
-  return 2 * (size_t)out_blocks(m->NZ * m->NY, m->NX) + VEC_BLOCKS + 16;
+  // (tiles are at least 64 wide, and the z chain at most NZ planes long)
+  const size_t rows = (size_t)m->NZ * m->NY;
+  return 2 * ((rows + 63) / 64) * (((size_t)m->NX + 63) / 64) + VEC_BLOCKS + sizeof(Scalars) / sizeof(double);
 }
 
 fe_status plan(fe_mesh* m, const double* cnt, bool constant_null) {

@@ -8,7 +8,7 @@ namespace fe_sep {
 
 // Buffers of one solve on the mesh's stream (n_phi entries each): the iterate, its masked
 // residual, three work vectors, the constraint mask, two float work arrays, and room for the
-// block partials (sep_part_doubles).
+// block partials and the scalars (part_doubles).
 struct Buf {
   double *phi, *r, *z, *p, *q;
   const unsigned char* mask;

@@ -44,7 +44,6 @@
 #pragma once
 
 #include <algorithm>
-#include <cstring>
 #include <type_traits>
 
 #include "fe_gll_tables.h"
@@ -66,13 +65,6 @@ struct PackF {   // two floats
     R r;
     asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
     return r;
-  }
-  static __device__ __forceinline__ R raw(double a) { return (R)__double_as_longlong(a); }
-  static double packed(double a) {
-    const float f[2] = {(float)a, (float)a};
-    double d;
-    memcpy(&d, f, sizeof d);
-    return d;
   }
   static __device__ __forceinline__ R zero() { return 0ull; }
   static __device__ __forceinline__ float fma1(float a, float b, float c) { return __fmaf_rn(a, b, c); }
@@ -109,8 +101,6 @@ struct PackD {   // one double
   using R = double;
   static constexpr int LANES = 1;
   static __device__ __forceinline__ R splat(double a) { return a; }
-  static __device__ __forceinline__ R raw(double a) { return a; }
-  static double packed(double a) { return a; }
   static __device__ __forceinline__ R zero() { return 0.0; }
   static __device__ __forceinline__ double fma1(double a, double b, double c) { return __fma_rn(a, b, c); }
   static __device__ __forceinline__ R fma(R a, R b, R c) { return __fma_rn(a, b, c); }
@@ -129,7 +119,6 @@ template <typename T>
 struct SweepCoef {
   T rx, ry;        // cx / cz, cy / cz
   T gx, gy;        // Bloch term over cz: kx and ky times its scales (0: real operator)
-  double k[FE_MAXN1][FE_MAXN1], t[FE_MAXN1], nt[FE_MAXN1];   // packed KH, TH, -TH
 };
 
 template <class V_, int P_, int CX_, int CY_, int XC_, int VP_, int RES_, bool DB_>
