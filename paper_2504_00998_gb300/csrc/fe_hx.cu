@@ -152,8 +152,7 @@ extern "C" fe_status fe_poisson_apply_K(fe_mesh* m, const double* x, double* y) 
   bool done = false;
   FE_TRY(fe_kcell_apply_f64(m, x, y, &done));
   if (done) return FE_OK;
-  KronIO<double> io{x, 1, y, 1, nullptr, 1, nullptr, 1, 1.0, 0.0, 0.0};
-  return fe::kron_k1(m->coefK, fe_geom(m, false), io, m->stream);
+  return fe::kron_k1(m->coefK, fe_geom(m, false), x, y, m->stream);
 }
 
 extern "C" fe_status fe_poisson_apply_K_f32(fe_mesh* m, const float* x, float* y) {

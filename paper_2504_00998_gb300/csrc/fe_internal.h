@@ -136,16 +136,6 @@ struct KronGeom {
   int nbx, nby;           // blocks in x, y
 };
 
-template <typename T>
-struct KronIO {
-  const T* X; int64_t ldx;
-  T* Y; int64_t ldy;
-  const T* Z; int64_t ldz;   // previous Chebyshev iterate (nullptr: beta ignored)
-  const T* V;                // potential per stored node (nullptr: none)
-  int64_t nvec;
-  T alpha, beta, shift;      // Y = alpha (H - shift) X + beta Z
-};
-
 // Arguments of a sweep launch: Y = alpha (Ht - shift) X + beta Z with the scalars in the form
 // the kernel uses (fe::sweep_scalars), one leading dimension for the three blocks.
 template <typename T>
@@ -183,8 +173,7 @@ void sweep_scalars_f64(const KronCoef& cf, int p, double alpha, double beta, dou
                        SweepIO<double>* io);
 void sweep_scalars_f32(const KronCoef& cf, int p, double alpha, double beta, double shift,
                        SweepIO<float>* io);
-fe_status kron_k1(const KronCoef& cf, const KronGeom& g, const KronIO<double>& io,
-                  cudaStream_t st);
+fe_status kron_k1(const KronCoef& cf, const KronGeom& g, const double* x, double* y, cudaStream_t st);
 // Batched launches: plan fills the tile fields, z segmentation, nvt and cta0 of n host
 // instances (g from fe_geom, io.nvec set) and returns the total CTA count; launch runs one
 // operator application over the device copy of those instances (widest: their largest nvec).

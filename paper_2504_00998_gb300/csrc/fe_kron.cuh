@@ -1,29 +1,21 @@
 // Matrix-free application of the finite-element stiffness of Section 2.3 on the uniform
-// tensor-product slab mesh, without scratch memory (the double product of one vector where the
-// cell-by-cell form's scratch cannot be had; blocks of vectors run in fe_sweep.cuh).
+// tensor-product slab mesh to one double vector, without scratch memory (where the cell-by-cell
+// form's scratch cannot be had; blocks of vectors run in fe_sweep.cuh), and the coefficient
+// tables and helpers that it shares with the tensor-core operator (fe_kron_tc.cu).
 //
 // For a uniform hexahedral mesh the assembled stiffness K_IJ = int grad N_I . grad N_J is a
 // sum of Kronecker products of the exactly integrated 1D element matrices,
 //   K = ax K1 (x) M1 (x) M1 + ay M1 (x) K1 (x) M1 + az M1 (x) M1 (x) K1,
-// (ax = hy hz / (2 hx), ...) and the GLL-lumped overlap is M = J mx (x) my (x) mz.  The
-// kernel evaluates, output-stationary,
-//   Y = alpha * ( oscale * K (S X) + (V - shift) X ) + beta * Z
-// with S = 1 and oscale = 1 for the Poisson operator (no potential), or the mass-scaled form.
+// (ax = hy hz / (2 hx), ...).
 //
-// Work decomposition: one CTA owns the nodes of an xy block of BX x BY cells (half-open),
-// a tile of NCH vector chunks, and a range of z layers.  It sweeps the z planes in order.
-// Each plane (with a p-node periodic halo in x and y), the potential and the previous
-// Chebyshev iterate of the owned nodes are staged into shared memory with cp.async one
-// plane ahead; the plane is contracted in y then in x (cell by cell, the shared boundary
-// node taking the previous cell's last row), and the two in-plane results are accumulated
-// into the p+1 output planes of the current z layer held in registers.  A layer's first p
-// planes are final once its top plane is processed; the top plane's sum carries into the
-// next layer.  No scatter, no atomics: every output node is written once by the thread that
-// owns it, so results are bitwise reproducible.
-//
-// All tile dimensions are compile-time constants; each thread's staging addresses are
-// computed once per launch.  CTAs are small (a few hundred threads, ~50 KB of shared
-// memory) so that several share an SM and one CTA's barriers overlap another's work.
+// Work decomposition: one CTA owns the nodes of an xy block of B x B cells (half-open) and a
+// range of z layers.  It sweeps the z planes in order.  Each plane (with a p-node periodic halo
+// in x and y) is staged into shared memory with cp.async one plane ahead; the plane is
+// contracted in y then in x (cell by cell, the shared boundary node taking the previous cell's
+// last row), and the two in-plane results are accumulated into the p+1 output planes of the
+// current z layer held in registers.  A layer's first p planes are final once its top plane
+// is processed; the top plane's sum carries into the next layer.  No scatter, no atomics: every
+// output node is written once by the thread that owns it, so results are bitwise reproducible.
 #pragma once
 
 #include <algorithm>
@@ -93,28 +85,6 @@ inline KronCoefT<T> convert_coef(const KronCoef& c) {
   return o;
 }
 
-// A chunk is CH consecutive vector entries of one node: 16 bytes (float4 / double2) or,
-// for single-vector operators, one element.  Aligned to its size so that every shared- and
-// global-memory access of a chunk is one vector instruction (the block layouts guarantee
-// it: 16-byte aligned blocks whose rows are a multiple of 16 bytes).
-template <typename T, int CH>
-struct alignas(sizeof(T) * CH) Chunk {
-  T v[CH];
-  __device__ __forceinline__ void zero() {
-#pragma unroll
-    for (int e = 0; e < CH; ++e) v[e] = T(0);
-  }
-  __device__ __forceinline__ void fma(T a, const Chunk& x) {
-#pragma unroll
-    for (int e = 0; e < CH; ++e) v[e] = fma_t(a, x.v[e], v[e]);
-  }
-  __device__ __forceinline__ static T fma_t(T a, T b, T c) { return a * b + c; }
-};
-
-template <>
-__device__ __forceinline__ double Chunk<double, 1>::fma_t(double a, double b, double c) {
-  return __fma_rn(a, b, c);
-}
 template <int BYTES>
 __device__ __forceinline__ void cp_async(void* smem, const void* gmem, int nbytes_valid) {
   unsigned s = (unsigned)__cvta_generic_to_shared(smem);
@@ -140,299 +110,113 @@ __device__ __forceinline__ int pmod(int a, int n) {
   return r < 0 ? r + n : r;
 }
 
-// compile-time tile shape
-template <int P_, int BX_, int BY_, int NCH_, int NTHR_>
-struct KronTileT {
-  static constexpr int P = P_, BX = BX_, BY = BY_, NCH = NCH_, NTHR = NTHR_;
-  static constexpr int BXn = BX * P, BYn = BY * P;
-  static constexpr int BXH = BXn + P + 1, BYH = BYn + P + 1;
-  static constexpr int NZI = BXn * BYn * NCH;            // output items (node, chunk)
-  static constexpr int IPT = (NZI + NTHR - 1) / NTHR;    // output items per thread
-  static constexpr int NST = BYH * BXH * NCH;            // staged chunks per plane
-  static constexpr int SPT = (NST + NTHR - 1) / NTHR;    // staged chunks per thread
-  static constexpr int NYI = BXH * NCH * BY;             // y-phase items (cell segments)
-  static constexpr int NXI = BYn * NCH * BX;             // x-phase items (cell segments)
-  static constexpr int ZR = P + 2;                       // ring of staged Chebyshev planes
-  // stage (and V) slots: plane gz + 2 is staged while other threads may still read plane gz
-  // after the plane's last barrier, so three slots keep those reads race-free
-  static constexpr int NSB = 3;
-  // row strides (in nodes) of the in-plane intermediates, odd so that the x phase's
-  // column-wise accesses (consecutive threads on consecutive rows) fall in distinct banks
-  static constexpr int ARS = BXH | 1;
-  static constexpr int WRS = BXn | 1;
+// cells per block side for each p: about ten nodes per side
+template <int P>
+struct KronBlock {
+  static constexpr int B = P == 1 ? 8 : P == 2 ? 5 : P == 3 ? 3 : 2;
 };
 
-// One CTA's work: xy block bxy (x fastest), vector tile vti, z segment zsi.
-// FULL: every xy block is complete and every vector tile full, so no ownership, edge or
-// ragged-vector test is needed anywhere in the sweep.
-template <typename T, int CH, class TL, bool FULL>
-__device__ __forceinline__ void kron_body(const KronCoefT<T>& cf, const KronGeom& g,
-                                          const KronIO<T>& io, int bxy, int vti, int zsi) {
-  using C = Chunk<T, CH>;
-  constexpr int P = TL::P, NCH = TL::NCH, BXn = TL::BXn, BYn = TL::BYn;
-  constexpr int BXH = TL::BXH, NTHR = TL::NTHR, IPT = TL::IPT;
-  constexpr int ARS = TL::ARS, WRS = TL::WRS;
-  constexpr int NZI = TL::NZI, NST = TL::NST, SPT = TL::SPT;
-  constexpr int CHB = CH * (int)sizeof(T);
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* stage0 = reinterpret_cast<C*>(smem_raw);                  // [NSB][BYH][BXH][NCH]
-  C* A = stage0 + TL::NSB * NST;                               // [BYn][ARS][NCH]
-  C* B = A + BYn * ARS * NCH;
-  C* W1 = B + BYn * ARS * NCH;                                 // [BYn][WRS][NCH]
-  C* W2 = W1 + BYn * WRS * NCH;
-  C* Zr = W2 + BYn * WRS * NCH;                                // [ZR][BYn][BXn][NCH]
-  const bool mass_scale = cf.mass_scale;
-  const bool use_z = io.Z != nullptr;                          // (beta != 0 by launch)
-  const bool use_v = io.V != nullptr;
-  T* Vs = reinterpret_cast<T*>(Zr + (use_z ? TL::ZR * NZI : 0));   // [NSB][BYn][BXn]
+// compile-time tile shape; threads: enough for one output node and one y-phase item each
+template <int P_>
+struct KronTile {
+  static constexpr int P = P_, B = KronBlock<P>::B, BN = B * P, BH = BN + P + 1;
+  static constexpr int NZI = BN * BN;                    // output nodes
+  static constexpr int NST = BH * BH;                    // staged nodes per plane
+  static constexpr int NYI = BH * B, NXI = BN * B;       // y- and x-phase items (cell segments)
+  static constexpr int NTHR = ((NZI > NYI ? NZI : NYI) + 31) / 32 * 32;
+  static constexpr int SPT = (NST + NTHR - 1) / NTHR;    // staged nodes per thread
+  // stage slots: plane gz + 2 is staged while other threads may still read plane gz after the
+  // plane's last barrier, so three slots keep those reads race-free
+  static constexpr int NSB = 3;
+  // row strides of the in-plane intermediates, odd so that the x phase's column-wise accesses
+  // (consecutive threads on consecutive rows) fall in distinct banks
+  static constexpr int ARS = BH | 1, WRS = BN | 1;
+  static constexpr size_t SMEM = sizeof(double) * (NSB * (size_t)NST + 2 * (size_t)BN * ARS + 2 * (size_t)BN * WRS);
+  static_assert(NTHR <= 512 && NXI <= NTHR, "one item a thread in every phase");
+};
 
-  const int tid = threadIdx.x;
-  const int bxi = bxy % g.nbx, byi = bxy / g.nbx;
-  const int x0 = bxi * BXn, y0 = byi * BYn;
-  const int64_t vt0 = (int64_t)vti * NCH * CH;
-  const int c0 = zsi * g.zseg;
-  const int c1 = min(c0 + g.zseg, g.nz);
+// y = K x on the phi nodes; block b: xy block b % (nbx nby) (x fastest), z segment b / (nbx nby)
+template <class TL>
+__global__ void __launch_bounds__(TL::NTHR)
+kron_kernel(const KronCoefT<double> cf, const KronGeom g, const double* __restrict__ x,
+            double* __restrict__ y) {
+  constexpr int P = TL::P, BN = TL::BN, BH = TL::BH, NTHR = TL::NTHR, NST = TL::NST, SPT = TL::SPT;
+  constexpr int ARS = TL::ARS, WRS = TL::WRS;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double* stage0 = reinterpret_cast<double*>(smem_raw);   // [NSB][BH][BH]
+  double* A = stage0 + TL::NSB * NST;                     // [BN][ARS]
+  double* Bs = A + BN * ARS;
+  double* W1 = Bs + BN * ARS;                             // [BN][WRS]
+  double* W2 = W1 + BN * WRS;
+
+  const int tid = threadIdx.x, nxy = g.nbx * g.nby, zsi = blockIdx.x / nxy, bxy = blockIdx.x - zsi * nxy;
+  const int x0 = (bxy % g.nbx) * BN, y0 = (bxy / g.nbx) * BN;
+  const int c0 = zsi * g.zseg, c1 = min(c0 + g.zseg, g.nz);
   const int cb = c0 > 0 ? c0 - 1 : 0;
   const int gbeg = cb * P, gend = c1 * P;
   const int64_t plane_nodes = (int64_t)g.NX * g.NY;
 
-  // ---- staging addresses (per thread, once) ---------------------------------------------
-  int64_t s_goff[SPT];
-  int s_bytes[SPT];
+  // staging offsets within a plane (per thread, once)
+  int64_t s_off[SPT];
 #pragma unroll
   for (int i = 0; i < SPT; ++i) {
-    const int e = tid + i * NTHR;
-    const int ec = e < NST ? e : 0;
-    const int ch = ec % NCH, node = ec / NCH;
-    const int xh = node % BXH, yh = node / BXH;
-    const int gx = pmod(x0 - P + xh, g.NX), gy = pmod(y0 - P + yh, g.NY);
-    const int64_t v0 = vt0 + (int64_t)ch * CH;
-    const int64_t rem = io.nvec - v0;
-    s_bytes[i] = e >= NST ? -1
-                          : (FULL ? CHB : (rem <= 0 ? 0 : (rem >= CH ? CHB : (int)(rem * sizeof(T)))));
-    s_goff[i] = (gx + (int64_t)g.NX * gy) * io.ldx + v0;
-  }
-
-  // ---- the thread's output items ---------------------------------------------------------
-  int it_x[IPT], it_y[IPT], it_ch[IPT];
-  bool it_own[IPT];
-  int64_t it_node[IPT];     // in-plane node index of the output
-  int64_t it_yo[IPT];       // offset of the item's entries in a plane of Y
-  T it_sxy[IPT], it_isxy[IPT];
-  int it_w[IPT], it_v[IPT], it_s[IPT];   // the item's offsets in W1 / W2, a V plane, a stage
-  C acc[IPT][P + 1];
-#pragma unroll
-  for (int i = 0; i < IPT; ++i) {
-    const int item = tid + i * NTHR;
-    const bool valid = item < NZI;
-    const int itc = valid ? item : 0;
-    it_ch[i] = itc % NCH;
-    const int node = itc / NCH;
-    it_x[i] = node % BXn;
-    it_y[i] = node / BXn;
-    const int64_t v0 = vt0 + (int64_t)it_ch[i] * CH;
-    it_own[i] = valid && (FULL || ((x0 + it_x[i] < g.NX) && (y0 + it_y[i] < g.NY) && (v0 < io.nvec)));
-    it_node[i] = (x0 + it_x[i]) + (int64_t)g.NX * (y0 + it_y[i]);
-    it_yo[i] = it_node[i] * io.ldy + v0;
-    it_sxy[i] = mass_scale ? cf.sig[it_x[i] % P] * cf.sig[it_y[i] % P] : T(1);
-    it_isxy[i] = T(1) / it_sxy[i];
-    it_w[i] = (it_y[i] * TL::WRS + it_x[i]) * NCH + it_ch[i];
-    it_v[i] = it_y[i] * BXn + it_x[i];
-    it_s[i] = ((it_y[i] + P) * BXH + (it_x[i] + P)) * NCH + it_ch[i];
-#pragma unroll
-    for (int j = 0; j <= P; ++j) acc[i][j].zero();
-  }
-
-  auto stored = [&](int gz) { return gz - g.gz_lo >= 0 && gz - g.gz_lo < g.NZs; };
-  auto owned_plane = [&](int gz) {   // planes this segment writes
-    return stored(gz) && ((gz >= c0 * P && gz < c1 * P) || (gz == g.nz * P && c1 == g.nz));
-  };
-
-  // stage plane gz: the halo block of X into the stage buffer, V and the Chebyshev operand
-  // of the owned nodes into their rings
-  // (called for gz = gbeg, gbeg + 1, ... in order: offsets and ring slots advance by one plane)
-  int64_t st_xoff = (int64_t)(gbeg - g.gz_lo) * plane_nodes * io.ldx;
-  const int64_t st_xstride = plane_nodes * io.ldx;
-  int st_slot = 0;                   // (gz - gbeg) % NSB of the plane to stage
-  int st_zslot = gbeg % TL::ZR;      // gz % ZR of the plane to stage
-  // the thread's V node and Z chunk offsets within a plane, and their plane offsets
-  int64_t st_voff = (int64_t)(gbeg - g.gz_lo) * plane_nodes;
-  int64_t st_zoff = st_voff * io.ldz;
-  const int64_t st_zstride = plane_nodes * io.ldz;
-  int64_t v_in = 0;
-  bool v_ok = false;
-  if (tid < BXn * BYn) {
-    const int x = tid % BXn, y = tid / BXn;
-    v_ok = FULL || (x0 + x < g.NX && y0 + y < g.NY);
-    v_in = (x0 + x) + (int64_t)g.NX * (y0 + y);
-  }
-  int64_t z_in[IPT];
-  int z_nb[IPT];
-#pragma unroll
-  for (int i = 0; i < IPT; ++i) {
-    const int64_t v0 = vt0 + (int64_t)it_ch[i] * CH;
-    const int64_t rem = io.nvec - v0;
-    z_nb[i] = !it_own[i] ? 0 : (FULL ? CHB : (rem <= 0 ? 0 : (rem >= CH ? CHB : (int)(rem * sizeof(T)))));
-    z_in[i] = it_node[i] * io.ldz + v0;
+    const int e = tid + i * NTHR, ec = e < NST ? e : 0;
+    s_off[i] = pmod(x0 - P + ec % BH, g.NX) + (int64_t)g.NX * pmod(y0 - P + ec / BH, g.NY);
   }
   auto stage_plane = [&](int gz) {
-    const int64_t pbase = st_xoff, vbase = st_voff, zbase = st_zoff;
-    const int sslot = st_slot, zslot = st_zslot;
-    st_xoff += st_xstride;
-    st_voff += plane_nodes;
-    st_zoff += st_zstride;
-    st_slot = st_slot + 1 == TL::NSB ? 0 : st_slot + 1;
-    st_zslot = st_zslot + 1 == TL::ZR ? 0 : st_zslot + 1;
-    if (!stored(gz)) return;
-    C* dst = stage0 + sslot * NST;
+    double* dst = stage0 + (gz - gbeg) % TL::NSB * NST;
+    const double* src = x + gz * plane_nodes;
 #pragma unroll
     for (int i = 0; i < SPT; ++i) {
       const int e = tid + i * NTHR;
-      if constexpr (FULL && NST % NTHR == 0) {
-        // full tile, every thread stages SPT whole chunks
-        cp_async<CHB>(dst + e, io.X + pbase + s_goff[i], CHB);
-      } else {
-        if (s_bytes[i] > 0) cp_async<CHB>(dst + e, io.X + pbase + s_goff[i], s_bytes[i]);
-        else if (s_bytes[i] == 0) cp_async<CHB>(dst + e, io.X, 0);
-      }
-    }
-    if (use_v && tid < BXn * BYn) {
-      T* vd = Vs + sslot * (BXn * BYn) + tid;
-      if constexpr (FULL)
-        cp_async<(int)sizeof(T)>(vd, io.V + vbase + v_in, (int)sizeof(T));
-      else
-        cp_async<(int)sizeof(T)>(vd, v_ok ? io.V + vbase + v_in : io.V, v_ok ? (int)sizeof(T) : 0);
-    }
-    if (use_z && owned_plane(gz)) {
-      C* zd = Zr + zslot * NZI;
-#pragma unroll
-      for (int i = 0; i < IPT; ++i) {
-        const int item = tid + i * NTHR;
-        if (item >= NZI) continue;
-        if constexpr (FULL) {
-          cp_async<CHB>(zd + item, io.Z + zbase + z_in[i], CHB);
-        } else {
-          const int nb = z_nb[i];
-          const T* src = nb ? io.Z + zbase + z_in[i] : io.Z;
-          cp_async<CHB>(zd + item, src, nb);
-        }
-      }
+      if (e < NST) cp_async<8>(dst + e, src + s_off[i], 8);
     }
   };
 
-  // write the final value of output plane gzo held in acc[i][j]
-  // layer c's bottom plane c P: its Z ring slot (c P) % ZR
-  int wr_zbase = (cb * P) % TL::ZR;
-  auto write_plane = [&](int gzo, int j) {
-    if (!owned_plane(gzo)) return;
-    const int zs = gzo - g.gz_lo;
-    T rs = T(1);   // 1 / sqrt(mz) of the plane (local index j; 1 for the plain stiffness)
-    if (mass_scale)
-      rs = j != 0 ? cf.rsq[j] : ((gzo == 0 || gzo == g.nz * P) ? cf.rsq_face : cf.rsq[0]);
-    const T ps = cf.zout * rs;
-    int zsl = wr_zbase + j;
-    zsl -= zsl >= TL::ZR ? TL::ZR : 0;
-    const C* zsrc = Zr + zsl * NZI;
-    T* yplane = io.Y + (int64_t)zs * plane_nodes * io.ldy;
+  // the thread's output node
+  const int ox = tid % BN, oy = tid / BN;
+  const bool own = tid < TL::NZI && x0 + ox < g.NX && y0 + oy < g.NY;
+  const int ow = tid < TL::NZI ? oy * WRS + ox : 0;
+  double* out = y + (x0 + ox) + (int64_t)g.NX * (y0 + oy);
+  double acc[P + 1];
 #pragma unroll
-    for (int i = 0; i < IPT; ++i) {
-      if (!it_own[i]) continue;
-      const int64_t v0 = vt0 + (int64_t)it_ch[i] * CH;
-      const T sc = io.alpha * ps * it_sxy[i];
-      C out;
-#pragma unroll
-      for (int e = 0; e < CH; ++e) out.v[e] = sc * acc[i][j].v[e];
-      if (use_z) {
-        const C zc = zsrc[tid + i * NTHR];
-#pragma unroll
-        for (int e = 0; e < CH; ++e) out.v[e] = C::fma_t(io.beta, zc.v[e], out.v[e]);
-      }
-      T* yp = yplane + it_yo[i];
-      if (FULL || v0 + CH <= io.nvec) {
-        *reinterpret_cast<C*>(yp) = out;
-      } else {
-        for (int e = 0; e < CH; ++e)
-          if (v0 + e < io.nvec) yp[e] = out.v[e];
-      }
-    }
+  for (int j = 0; j <= P; ++j) acc[j] = 0.0;
+  // planes this segment writes
+  auto write_plane = [&](int gz, int j) {
+    if (own && ((gz >= c0 * P && gz < c1 * P) || (gz == g.nz * P && c1 == g.nz))) out[gz * plane_nodes] = acc[j];
   };
-
-  // Plane with local index K (compile time, so every coefficient is an immediate operand):
-  // the potential term of the plane's own nodes (when pot) and the z contraction of its
-  // in-plane results into the layer accumulators.
-  auto plane_z = [&](auto kc, bool pot, bool face, T inv_ps, const T* vv, const C* st,
-                     const C* w1, const C* w2) {
+  // z contraction of the in-plane results of the plane with local index K (compile time, so
+  // every coefficient is an immediate operand) into the layer accumulators
+  auto plane_z = [&](auto kc, double a, double b) {
     constexpr int K = decltype(kc)::value;
     if constexpr (K <= P) {
 #pragma unroll
-      for (int i = 0; i < IPT; ++i) {
-        if (pot && it_own[i]) {
-          const T pv = (vv[it_v[i]] - io.shift) * inv_ps * it_isxy[i];
-          const C xs = st[it_s[i]];
-          acc[i][K].fma(pv, xs);
-        }
-        C a = w1[i], b = w2[i];
-#pragma unroll
-        if (face) {
-#pragma unroll
-          for (int e = 0; e < CH; ++e) { a.v[e] *= cf.face_fix; b.v[e] *= cf.face_fix; }
-        }
-#pragma unroll
-        for (int j = 0; j <= P; ++j) {
-          acc[i][j].fma(cf.AzKs[j][K], a);
-          acc[i][j].fma(cf.AzMs[j][K], b);
-        }
+      for (int j = 0; j <= P; ++j) {
+        acc[j] = __fma_rn(cf.AzKs[j][K], a, acc[j]);
+        acc[j] = __fma_rn(cf.AzMs[j][K], b, acc[j]);
       }
     }
   };
-  auto dispatch_z = [&](int k, bool pot, bool face, T inv_ps, const T* vv, const C* st,
-                        const C* w1, const C* w2) {
+  auto dispatch_z = [&](int k, double a, double b) {
     switch (k) {
-      case 0: plane_z(std::integral_constant<int, 0>{}, pot, face, inv_ps, vv, st, w1, w2); break;
-      case 1: plane_z(std::integral_constant<int, 1>{}, pot, face, inv_ps, vv, st, w1, w2); break;
-      case 2: plane_z(std::integral_constant<int, 2>{}, pot, face, inv_ps, vv, st, w1, w2); break;
-      case 3: plane_z(std::integral_constant<int, 3>{}, pot, face, inv_ps, vv, st, w1, w2); break;
-      case 4: plane_z(std::integral_constant<int, 4>{}, pot, face, inv_ps, vv, st, w1, w2); break;
-      case 5: plane_z(std::integral_constant<int, 5>{}, pot, face, inv_ps, vv, st, w1, w2); break;
-      case 6: plane_z(std::integral_constant<int, 6>{}, pot, face, inv_ps, vv, st, w1, w2); break;
+      case 0: plane_z(std::integral_constant<int, 0>{}, a, b); break;
+      case 1: plane_z(std::integral_constant<int, 1>{}, a, b); break;
+      case 2: plane_z(std::integral_constant<int, 2>{}, a, b); break;
+      case 3: plane_z(std::integral_constant<int, 3>{}, a, b); break;
+      case 4: plane_z(std::integral_constant<int, 4>{}, a, b); break;
+      case 5: plane_z(std::integral_constant<int, 5>{}, a, b); break;
+      case 6: plane_z(std::integral_constant<int, 6>{}, a, b); break;
       default: break;
     }
   };
 
-  auto shift_layer = [&]() {
-#pragma unroll
-    for (int i = 0; i < IPT; ++i) {
-      acc[i][0] = acc[i][P];
-#pragma unroll
-      for (int j = 1; j <= P; ++j) acc[i][j].zero();
-    }
-  };
+  const int yh = tid % BH, yc = tid / BH * P;   // y-phase item: halo column, first row of the cell
+  const int xr = tid % BN, xc = tid / BN * P;   // x-phase item: row, first node of the cell
 
-  // in-plane 1D coefficients
-  auto cYM = [&](int j, int k) -> T { return cf.AyM[j][k]; };
-  auto cYK = [&](int j, int k) -> T { return cf.AyK[j][k]; };
-  auto cXM = [&](int j, int k) -> T { return cf.AxM[j][k]; };
-  auto cXK = [&](int j, int k) -> T { return cf.AxK[j][k]; };
-
-  // scalar-lane items of the in-plane phases (used when each thread has at most one)
-  constexpr int NL = NCH * CH;
-  int y_ibase = 0, y_obase = 0, x_ibase = 0, x_obase = 0;
-  {
-    const int l = tid % NL, r = tid / NL;
-    const int xh = r % BXH, yb = (r / BXH) * P;
-    y_ibase = (yb * BXH + xh) * NL + l;
-    y_obase = (yb * ARS + xh) * NL + l;
-    const int y = r % BYn, xb = (r / BYn) * P;
-    x_ibase = y * ARS * NL + xb * NL + l;
-    x_obase = (y * WRS + xb) * NL + l;
-  }
-
-  // ---- sweep -----------------------------------------------------------------------------
   stage_plane(gbeg);
   cp_commit();
   int c = cb;
-  int cur_slot = 0;   // (gz - gbeg) % NSB
-  for (int gz = gbeg; gz <= gend; ++gz, cur_slot = cur_slot + 1 == TL::NSB ? 0 : cur_slot + 1) {
+  for (int gz = gbeg; gz <= gend; ++gz) {
     const int k = gz - c * P;
     if (gz < gend) {
       stage_plane(gz + 1);
@@ -442,162 +226,87 @@ __device__ __forceinline__ void kron_body(const KronCoefT<T>& cf, const KronGeom
       cp_wait<0>();
     }
     __syncthreads();
-    const C* st = stage0 + cur_slot * NST;
-
-    if (stored(gz)) {
-      // The two in-plane phases run on scalar lanes: an item is one cell segment of one
-      // vector entry, so that every thread has work (a chunk-wide item would leave most of
-      // the CTA idle at the following barrier).  NL scalars per node, lane-fastest indexing
-      // keeps consecutive threads on consecutive words.
-      using S1 = Chunk<T, 1>;
-      const S1* sts = reinterpret_cast<const S1*>(st);
-      S1* As = reinterpret_cast<S1*>(A);
-      S1* Bs = reinterpret_cast<S1*>(B);
-      // phase Y: a = AyM U, b = AyK U along y for every halo x
-      auto phase_y = [&](int ibase, int obase) {
-        S1 own[P + 1], prv[P];
+    const double* st = stage0 + (gz - gbeg) % TL::NSB * NST;
+    // phase Y: a = AyM u, b = AyK u along y for every halo x
+    if (tid < TL::NYI) {
+      double u[P + 1], prv[P];
 #pragma unroll
-        for (int kk = 0; kk <= P; ++kk) own[kk] = sts[ibase + (P + kk) * BXH * NL];
+      for (int kk = 0; kk <= P; ++kk) u[kk] = st[(yc + P + kk) * BH + yh];
 #pragma unroll
-        for (int kk = 0; kk < P; ++kk) prv[kk] = sts[ibase + kk * BXH * NL];
+      for (int kk = 0; kk < P; ++kk) prv[kk] = st[(yc + kk) * BH + yh];
 #pragma unroll
-        for (int j = 0; j < P; ++j) {
-          S1 a, b;
-          a.zero();
-          b.zero();
+      for (int j = 0; j < P; ++j) {
+        double a = 0.0, b = 0.0;
 #pragma unroll
-          for (int kk = 0; kk <= P; ++kk) {
-            a.fma(cYM(j, kk), own[kk]);
-            b.fma(cYK(j, kk), own[kk]);
-          }
-          if (j == 0) {
-#pragma unroll
-            for (int kk = 0; kk < P; ++kk) {
-              a.fma(cYM(P, kk), prv[kk]);
-              b.fma(cYK(P, kk), prv[kk]);
-            }
-            a.fma(cYM(P, P), own[0]);
-            b.fma(cYK(P, P), own[0]);
-          }
-          As[obase + j * ARS * NL] = a;
-          Bs[obase + j * ARS * NL] = b;
+        for (int kk = 0; kk <= P; ++kk) {
+          a = __fma_rn(cf.AyM[j][kk], u[kk], a);
+          b = __fma_rn(cf.AyK[j][kk], u[kk], b);
         }
-      };
-      if constexpr (TL::NYI * CH == NTHR) {
-        phase_y(y_ibase, y_obase);
-      } else if constexpr (TL::NYI * CH <= NTHR) {
-        if (tid < TL::NYI * CH) phase_y(y_ibase, y_obase);
-      } else {
-#pragma unroll 1
-        for (int e = tid; e < TL::NYI * CH; e += NTHR) {
-          const int l = e % NL, r = e / NL, xh = r % BXH, yb = (r / BXH) * P;
-          phase_y((yb * BXH + xh) * NL + l, (yb * ARS + xh) * NL + l);
+        if (j == 0) {
+#pragma unroll
+          for (int kk = 0; kk < P; ++kk) {
+            a = __fma_rn(cf.AyM[P][kk], prv[kk], a);
+            b = __fma_rn(cf.AyK[P][kk], prv[kk], b);
+          }
+          a = __fma_rn(cf.AyM[P][P], u[0], a);
+          b = __fma_rn(cf.AyK[P][P], u[0], b);
         }
+        A[(yc + j) * ARS + yh] = a;
+        Bs[(yc + j) * ARS + yh] = b;
       }
-      __syncthreads();
-      // phase X: W1 = AxM a, W2 = AxK a + AxM b along x for every owned y
-      {
-        S1* W1s = reinterpret_cast<S1*>(W1);
-        S1* W2s = reinterpret_cast<S1*>(W2);
-        auto phase_x = [&](int ibase, int obase) {
-          const S1* arow = As + ibase;
-          const S1* brow = Bs + ibase;
-          S1 ao[P + 1], bo[P + 1];
+    }
+    __syncthreads();
+    // phase X: W1 = AxM a, W2 = AxK a + AxM b along x for every owned y
+    if (tid < TL::NXI) {
+      const double* ar = A + xr * ARS + xc;
+      const double* br = Bs + xr * ARS + xc;
+      double ao[P + 1], bo[P + 1];
 #pragma unroll
-          for (int kk = 0; kk <= P; ++kk) {
-            ao[kk] = arow[(P + kk) * NL];
-            bo[kk] = brow[(P + kk) * NL];
-          }
+      for (int kk = 0; kk <= P; ++kk) {
+        ao[kk] = ar[P + kk];
+        bo[kk] = br[P + kk];
+      }
 #pragma unroll
-          for (int j = 0; j < P; ++j) {
-            S1 u, v;
-            u.zero();
-            v.zero();
+      for (int j = 0; j < P; ++j) {
+        double u = 0.0, v = 0.0;
 #pragma unroll
-            for (int kk = 0; kk <= P; ++kk) {
-              u.fma(cXM(j, kk), ao[kk]);
-              v.fma(cXK(j, kk), ao[kk]);
-              v.fma(cXM(j, kk), bo[kk]);
-            }
-            if (j == 0) {
-#pragma unroll
-              for (int kk = 0; kk < P; ++kk) {
-                const S1 ap = arow[kk * NL];
-                const S1 bp = brow[kk * NL];
-                u.fma(cXM(P, kk), ap);
-                v.fma(cXK(P, kk), ap);
-                v.fma(cXM(P, kk), bp);
-              }
-              u.fma(cXM(P, P), ao[0]);
-              v.fma(cXK(P, P), ao[0]);
-              v.fma(cXM(P, P), bo[0]);
-            }
-            W1s[obase + j * NL] = u;
-            W2s[obase + j * NL] = v;
-          }
-        };
-        if constexpr (TL::NXI * CH <= NTHR) {
-          if (tid < TL::NXI * CH) phase_x(x_ibase, x_obase);
-        } else {
-#pragma unroll 1
-          for (int e = tid; e < TL::NXI * CH; e += NTHR) {
-            const int l = e % NL, r = e / NL, y = r % BYn, xb = (r / BYn) * P;
-            phase_x(y * ARS * NL + xb * NL + l, (y * WRS + xb) * NL + l);
-          }
+        for (int kk = 0; kk <= P; ++kk) {
+          u = __fma_rn(cf.AxM[j][kk], ao[kk], u);
+          v = __fma_rn(cf.AxK[j][kk], ao[kk], v);
+          v = __fma_rn(cf.AxM[j][kk], bo[kk], v);
         }
-      }
-      __syncthreads();
-      C w1[IPT], w2[IPT];
+        if (j == 0) {
 #pragma unroll
-      for (int i = 0; i < IPT; ++i) {
-        const int item = it_w[i];
-        w1[i] = W1[item];
-        w2[i] = W2[item];
+          for (int kk = 0; kk < P; ++kk) {
+            u = __fma_rn(cf.AxM[P][kk], ar[kk], u);
+            v = __fma_rn(cf.AxK[P][kk], ar[kk], v);
+            v = __fma_rn(cf.AxM[P][kk], br[kk], v);
+          }
+          u = __fma_rn(cf.AxM[P][P], ao[0], u);
+          v = __fma_rn(cf.AxK[P][P], ao[0], v);
+          v = __fma_rn(cf.AxM[P][P], bo[0], v);
+        }
+        W1[xr * WRS + xc + j] = u;
+        W2[xr * WRS + xc + j] = v;
       }
-      const bool face = gz == 0 || gz == g.nz * P;
-      T sqz = T(1);   // sqrt(mz) of the plane (1 for the plain stiffness)
-      if (mass_scale) {
-        const int l = k == P ? 0 : k;   // gz % P
-        sqz = l != 0 ? cf.sq[l] : (face ? cf.sq_face : cf.sq[0]);
-      }
-      const T inv_ps = sqz * cf.izout;
-      const T* vv = Vs + cur_slot * (BXn * BYn);
-      dispatch_z(k, use_v, face, inv_ps, vv, st, w1, w2);
-      if (k == P) {
-        // the layer is complete: its first P planes are final; the top plane's sum
-        // becomes the bottom accumulator of the next layer
-#pragma unroll
-        for (int j = 0; j < P; ++j) write_plane(c * P + j, j);
-        shift_layer();
-        ++c;
-        wr_zbase += P;
-        wr_zbase -= wr_zbase >= TL::ZR ? TL::ZR : 0;
-        if (c < c1) dispatch_z(0, false, face, inv_ps, vv, st, w1, w2);
-      }
-    } else if (k == P) {
-      // an unstored (homogeneous Dirichlet) plane contributes nothing
+    }
+    __syncthreads();
+    const double w1 = W1[ow], w2 = W2[ow];
+    dispatch_z(k, w1, w2);
+    if (k == P) {
+      // the layer is complete: its first P planes are final; the top plane's sum becomes the
+      // bottom accumulator of the next layer
 #pragma unroll
       for (int j = 0; j < P; ++j) write_plane(c * P + j, j);
-      shift_layer();
+      acc[0] = acc[P];
+#pragma unroll
+      for (int j = 1; j <= P; ++j) acc[j] = 0.0;
       ++c;
-      wr_zbase += P;
-      wr_zbase -= wr_zbase >= TL::ZR ? TL::ZR : 0;
+      if (c < c1) dispatch_z(0, w1, w2);
     }
   }
   // the last processed plane (gend = c1 P) is final only if it is the top face
   write_plane(gend, 0);
-}
-
-// 1D grid, vector tile fastest: the CTAs that read the other halves of a node's DRAM
-// bursts (neighbouring vector tiles of the same xy block) run side by side, so a burst is
-// fetched once; neighbouring xy blocks (halo sharing) follow within the resident window.
-template <typename T, int CH, class TL, bool FULL>
-__global__ void __launch_bounds__(TL::NTHR)
-kron_kernel(const KronCoefT<T> cf, const KronGeom g, const KronIO<T> io, int nvt) {
-  const int b = blockIdx.x;
-  const int nxy = g.nbx * g.nby;
-  const int r = b / nvt;
-  kron_body<T, CH, TL, FULL>(cf, g, io, r % nxy, b % nvt, r / nxy);
 }
 
 // Dynamic shared memory limit, and the largest shared-memory carveout so that the residency
@@ -616,60 +325,6 @@ inline fe_status kron_func_setup(K kern, size_t smem) {
   return FE_OK;
 }
 
-// shared memory of one CTA
-template <typename T, int CH, class TL>
-inline size_t kron_smem(bool use_z, bool use_v) {
-  const size_t cb = sizeof(Chunk<T, CH>);
-  size_t s = cb * (TL::NSB * (size_t)TL::NST + 2 * (size_t)TL::BYn * TL::ARS * TL::NCH +
-                   2 * (size_t)TL::BYn * TL::WRS * TL::NCH);
-  if (use_z) s += cb * TL::ZR * (size_t)TL::NZI;
-  if (use_v) s += sizeof(T) * TL::NSB * (size_t)TL::BXn * TL::BYn;
-  return s;
-}
-
-template <typename T, int CH, class TL>
-fe_status kron_launch_t(const KronCoef& cf, const KronGeom& g, const KronIO<T>& io,
-                        cudaStream_t st) {
-  if (g.bx != TL::BX || g.by != TL::BY) return fe_fail(FE_EINVAL, "tile shape mismatch");
-  KronIO<T> io2 = io;
-  if (io2.Z != nullptr && io2.beta == T(0)) io2.Z = nullptr;
-  const size_t smem = kron_smem<T, CH, TL>(io2.Z != nullptr, io2.V != nullptr);
-  if (smem > 227 * 1024) return fe_fail(FE_EINVAL, "tile needs %zu bytes of shared memory", smem);
-  const int64_t vtile = (int64_t)TL::NCH * CH;
-  const bool full = g.NX % TL::BXn == 0 && g.NY % TL::BYn == 0 && io.nvec % vtile == 0;
-  auto kern = full ? kron_kernel<T, CH, TL, true> : kron_kernel<T, CH, TL, false>;
-  FE_TRY(kron_func_setup(kern, smem));
-  const int64_t nvt = (io.nvec + vtile - 1) / vtile;
-  const int64_t total = (int64_t)g.nbx * g.nby * nvt * ((g.nz + g.zseg - 1) / g.zseg);
-  if (total > 0x7fffffffLL || nvt > 0x7fffffffLL) return fe_fail(FE_EINVAL, "grid too large");
-  KronCoefT<T> cft = convert_coef<T>(cf);
-  kern<<<(unsigned)total, TL::NTHR, smem, st>>>(cft, g, io2, (int)nvt); fe_count_launch();
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return fe_fail(FE_ECUDA, "kron kernel launch: %s", cudaGetErrorString(e));
-  return FE_OK;
-}
-
-// cells per block side for each p: about ten nodes per side
-template <int P>
-struct KronBlock {
-  static constexpr int B = P == 1 ? 8 : P == 2 ? 5 : P == 3 ? 3 : 2;
-};
-
-// threads: enough for one output item (node, chunk) and one y-phase scalar item each
-template <int P, int NCH, int CH>
-struct KronTileFor {
-  static constexpr int B = KronBlock<P>::B;
-  static constexpr int NZ_ITEMS = B * P * B * P * NCH;
-  static constexpr int NY_ITEMS = (B * P + P + 1) * B * NCH * CH;
-  static constexpr int N = NZ_ITEMS > NY_ITEMS ? NZ_ITEMS : NY_ITEMS;
-  static constexpr int NTHR = (N + 31) / 32 * 32 > 512 ? 512 : (N + 31) / 32 * 32;
-  using type = KronTileT<P, B, B, NCH, NTHR>;
-};
-
-}  // namespace fe
-
-namespace fe {
-
 inline int device_sms() {
   static int sms = 0;
   if (sms == 0) {
@@ -681,35 +336,24 @@ inline int device_sms() {
   return sms;
 }
 
-// fill the block grid and the z segmentation for tile TL, then launch
-template <typename T, int CH, class TL>
-fe_status kron_go(const KronCoef& cf, KronGeom g, const KronIO<T>& io, cudaStream_t st) {
-  g.bx = TL::BX;
-  g.by = TL::BY;
+// z segments are halved while the grid has fewer than four CTAs an SM
+template <class TL>
+fe_status kron_launch(const KronCoef& cf, KronGeom g, const double* x, double* y, cudaStream_t st) {
   const int nx = g.NX / g.p, ny = g.NY / g.p;
-  g.nbx = (nx + TL::BX - 1) / TL::BX;
-  g.nby = (ny + TL::BY - 1) / TL::BY;
-  const int64_t vt = (io.nvec + (int64_t)TL::NCH * CH - 1) / ((int64_t)TL::NCH * CH);
-  const int64_t base = (int64_t)g.nbx * g.nby * vt;
-  const int64_t want = 4 * (int64_t)device_sms();
-  int zseg = g.nz;
-  while (zseg > 2 && base * ((g.nz + zseg - 1) / zseg) < want) zseg = (zseg + 1) / 2;
-  g.zseg = zseg;
-  return kron_launch_t<T, CH, TL>(cf, g, io, st);
-}
-
-template <typename T, int CH, int NCH>
-fe_status kron_dispatch(const KronCoef& cf, const KronGeom& g, const KronIO<T>& io,
-                        cudaStream_t st) {
-  switch (g.p) {
-    case 1: return kron_go<T, CH, typename KronTileFor<1, NCH, CH>::type>(cf, g, io, st);
-    case 2: return kron_go<T, CH, typename KronTileFor<2, NCH, CH>::type>(cf, g, io, st);
-    case 3: return kron_go<T, CH, typename KronTileFor<3, NCH, CH>::type>(cf, g, io, st);
-    case 4: return kron_go<T, CH, typename KronTileFor<4, NCH, CH>::type>(cf, g, io, st);
-    case 5: return kron_go<T, CH, typename KronTileFor<5, NCH, CH>::type>(cf, g, io, st);
-    case 6: return kron_go<T, CH, typename KronTileFor<6, NCH, CH>::type>(cf, g, io, st);
-    default: return fe_fail(FE_EUNSUPPORTED, "p = %d", g.p);
-  }
+  g.bx = g.by = TL::B;
+  g.nbx = (nx + TL::B - 1) / TL::B;
+  g.nby = (ny + TL::B - 1) / TL::B;
+  const int64_t base = (int64_t)g.nbx * g.nby, want = 4 * (int64_t)device_sms();
+  g.zseg = g.nz;
+  while (g.zseg > 2 && base * ((g.nz + g.zseg - 1) / g.zseg) < want) g.zseg = (g.zseg + 1) / 2;
+  const int64_t total = base * ((g.nz + g.zseg - 1) / g.zseg);
+  if (total > 0x7fffffffLL) return fe_fail(FE_EINVAL, "grid too large");
+  FE_TRY(kron_func_setup(kron_kernel<TL>, TL::SMEM));
+  kron_kernel<TL><<<(unsigned)total, TL::NTHR, TL::SMEM, st>>>(convert_coef<double>(cf), g, x, y);
+  fe_count_launch();
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return fe_fail(FE_ECUDA, "kron kernel launch: %s", cudaGetErrorString(e));
+  return FE_OK;
 }
 
 }  // namespace fe
