@@ -66,19 +66,19 @@ constexpr int PROJ_THREADS = PROJ_GROUPS * PROJ_SLOTS;
 // flight each, and the slots summed in a fixed order: with one thread walking all entries of
 // a vector the launch took 300 us (64 atoms, 128 float vectors, 190,400 nodes, p = 5), bound by
 // the latency of its loads; now 24 us.  (The coefficients D are applied here, once an atom,
-// instead of at every node.)  Block b: atom b % natoms of tile b / natoms.
+// instead of at every node.)  Grid: atoms in x, tiles in y and, past its 65,535, in z.
 template <typename T>
 __global__ void __launch_bounds__(PROJ_THREADS)
-k_nl_project(const T* __restrict__ X, int64_t ld, int64_t nvec, int natoms,
-             const int* __restrict__ atom_ptr,
+k_nl_project(const T* __restrict__ X, int64_t ld, int64_t nvec, const int* __restrict__ atom_ptr,
              const int* __restrict__ ent_node, const T* __restrict__ ent_val,
              const T* __restrict__ Dv, T* __restrict__ C, int64_t ldc) {
   using G = NlGroup<T>;
   using V = typename G::V;
   __shared__ V red[PROJ_THREADS / 32][PROJ_GROUPS][NCHAN];
-  const int tile = blockIdx.x / natoms, a = blockIdx.x - tile * natoms;
-  const int g = threadIdx.x % PROJ_GROUPS, slot = threadIdx.x / PROJ_GROUPS;
-  const int64_t v = ((int64_t)tile * PROJ_GROUPS + g) * G::W;
+  const int a = blockIdx.x, g = threadIdx.x % PROJ_GROUPS, slot = threadIdx.x / PROJ_GROUPS;
+  const int64_t tile = blockIdx.y + (int64_t)blockIdx.z * gridDim.y;
+  const int64_t v = (tile * PROJ_GROUPS + g) * G::W;
+  if (tile * PROJ_GROUPS * G::W >= nvec) return;
   const bool in = v < nvec;
   const int e1 = atom_ptr[a + 1];
   V c[NCHAN];
@@ -285,12 +285,14 @@ fe_status fe_nonlocal_apply(fe_mesh* m, const void* X, void* Y, int64_t nvec, in
   void* c;
   FE_TRY(fe_ws(m, WS_NL, eb * NCHAN * (size_t)nl.natoms * ldc + 64, &c));
   const int64_t tiles = (ng + PROJ_GROUPS - 1) / PROJ_GROUPS;
-  if (tiles * nl.natoms > 0x7fffffffLL) return fe_fail(FE_EINVAL, "nonlocal term: too many vectors");
+  const int64_t ty = std::min<int64_t>(tiles, 65535), tz = (tiles + ty - 1) / ty;
+  if (tz > 65535) return fe_fail(FE_EINVAL, "nonlocal term: too many vectors");
+  const dim3 pg(nl.natoms, (unsigned)ty, (unsigned)tz);
   const int ab = (int)std::min<int64_t>(((int64_t)nl.ntouched * ng + 255) / 256, 152 * 32);
   auto run = [&](auto zero, const auto* val, const auto* D) {
     using T = decltype(zero);
-    k_nl_project<T><<<(unsigned)(tiles * nl.natoms), PROJ_THREADS, 0, st>>>(
-        (const T*)X, ld, nvec, nl.natoms, nl.atom_ptr, nl.ent_node, val, D, (T*)c, ldc);
+    k_nl_project<T><<<pg, PROJ_THREADS, 0, st>>>((const T*)X, ld, nvec, nl.atom_ptr, nl.ent_node, val,
+                                                 D, (T*)c, ldc);
     fe_count_launch();
     k_nl_apply<T><<<ab, 256, 0, st>>>((T*)Y, ld, nvec, nl.ntouched, nl.tn_node, nl.tn_ptr, nl.tn_ent,
                                       nl.ent_atom, val, (const T*)c, ldc, (T)alpha);

@@ -168,7 +168,8 @@ print(log())
 """)
     assert out.startswith("0 ok"), out.splitlines()[0]
     tiles = -(-nvec // (16 if prec == "FE_F64" else 32))
-    assert re.search(rf"k_nl_project\S* {2 * tiles} 1 1 256 ", out)
+    y, z = map(int, re.search(r"k_nl_project\S* 2 (\d+) (\d+) 256 ", out).groups())
+    assert tiles <= y * z < tiles + y
 
 
 def test_solve_without_memory_for_the_eigenbases(child):
