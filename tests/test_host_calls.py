@@ -131,8 +131,8 @@ print(st, lib.fe_last_error().decode() if st else "ok")
 print(log())
 """)
     assert out.startswith("0 ok"), out.splitlines()[0]
-    grids = [int(g) for g in re.findall(r"^launch \S*k_gram_partial\S* (\d+) 1 1 ", out, re.M)]
-    assert grids and all(g == tiles * tiles for g in grids)
+    grids = re.findall(r"^launch \S*k_gram_partial\S* 1 (\d+) (\d+) ", out, re.M)
+    assert grids and all(0 <= int(y) * int(z) - tiles * tiles < int(y) for y, z in grids)
 
 
 # memory of this device, off its alignment, of another device, unknown to CUDA (fake_cuda.c)
