@@ -124,7 +124,8 @@ enum { FE_RR_PRODUCTS_F64 = 0, FE_RR_PRODUCTS_TC32 = 1 };
 enum { FE_PRECOND_JACOBI = 0, FE_PRECOND_JACOBI_PLANES = 1, FE_PRECOND_JACOBI_PLANES_MODES = 2,
        FE_PRECOND_SEPARABLE = 3 };
 /*   FE_OPT_POISSON_ARITH: arithmetic of the Poisson solve.  FE_POISSON_F64: CG in double.
- *     FE_POISSON_MIXED (default): a float CG (operator, vectors and preconditioner in float,
+ *     FE_POISSON_MIXED (default): with FE_PRECOND_SEPARABLE a double CG around the float
+ *     preconditioner, started again from f - K phi until that meets rtol; otherwise a float CG (operator, vectors and preconditioner in float,
  *     dot products accumulated in double) with reliable updates -- whenever its residual has
  *     dropped by 1e2, phi (double) takes the float iterate and the residual is replaced by
  *     the double residual f - K phi (the search direction restarts when the two residuals

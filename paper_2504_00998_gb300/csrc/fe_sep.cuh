@@ -24,9 +24,9 @@ size_t part_doubles(const fe_mesh* m);
 // separable form.  Synchronises.
 fe_status plan(fe_mesh* m, const double* cnt, bool constant_null);
 // CG in double with the separable preconditioner from phi and r until |r|^2 <= tol2, at most
-// maxit iterations; *rr is the |r|^2 of the recurrence at return.  *lost is set when the iteration stopped
-// making progress or r is outside the floats' range, phi then being finite (the caller solves on
-// from phi by other means).
+// maxit iterations; *rr is the |r|^2 of the recurrence at return (rounding takes it below that of
+// f - K phi).  *lost is set when the iteration stopped making progress or r is outside the
+// floats' range, phi then being finite (the caller solves on from phi by other means).
 fe_status solve(fe_mesh* m, const Buf& b, double tol2, int maxit, double* rr, int* iters,
                 bool* lost);
 
