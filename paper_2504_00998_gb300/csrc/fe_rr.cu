@@ -160,14 +160,13 @@ __device__ __forceinline__ void gram_share(const double* __restrict__ X, int64_t
     }
 }
 
-// Grid: row shares in x, tile pairs in y and, past its 65,535, in z (16,368 columns are 341 tiles).
+// Grid: row shares in x, the tile pair's I in y and J in z.
 template <int MB, bool H>
 __global__ void __launch_bounds__(GRAM_THREADS, 2)
 k_gram_partial(const double* __restrict__ X, int64_t ld, const double* __restrict__ HX, int64_t ldh,
-               int n, int tiles, int64_t N, double* __restrict__ part) {
+               int n, int64_t N, double* __restrict__ part) {
   __shared__ double xs[GRAM_ROWS][16 * MB], ys[GRAM_ROWS][16 * MB], hs[H ? GRAM_ROWS : 1][16 * MB];
-  const int pair = blockIdx.y + blockIdx.z * gridDim.y, I = pair % tiles, J = pair / tiles;
-  if (J >= tiles) return;
+  const int I = blockIdx.y, J = blockIdx.z;
   const int i0 = I * 16 * MB, j0 = J * 16 * MB;
   const int64_t r0 = N * blockIdx.x / gridDim.x, r1 = N * (blockIdx.x + 1) / gridDim.x;
   double* ps = part + (int64_t)blockIdx.x * (H ? 2 : 1) * n * n;
@@ -201,10 +200,9 @@ template <int MB>
 void gram_launch(const double* X, int64_t ld, const double* HX, int64_t ldh, int n, int64_t N,
                  int shares, double* part, cudaStream_t st) {
   const int tiles = (n + 16 * MB - 1) / (16 * MB);
-  const unsigned pairs = (unsigned)tiles * tiles, py = std::min(pairs, 65535u);
-  const dim3 grid(shares, py, (pairs + py - 1) / py);
-  if (HX) k_gram_partial<MB, true><<<grid, GRAM_THREADS, 0, st>>>(X, ld, HX, ldh, n, tiles, N, part);
-  else k_gram_partial<MB, false><<<grid, GRAM_THREADS, 0, st>>>(X, ld, nullptr, 0, n, tiles, N, part);
+  const dim3 grid(shares, tiles, tiles);
+  if (HX) k_gram_partial<MB, true><<<grid, GRAM_THREADS, 0, st>>>(X, ld, HX, ldh, n, N, part);
+  else k_gram_partial<MB, false><<<grid, GRAM_THREADS, 0, st>>>(X, ld, nullptr, 0, n, N, part);
 }
 
 struct RrWs {
