@@ -704,7 +704,7 @@ inline int sweep_zseg(int64_t base, int nz) {
     const double t = (z + (segs > 1 ? 1 : 0)) * per;
     if (t < cost * (1.0 - 1e-9)) { cost = t; best = z; }
     if (z == 1) break;
-    s = (nz + z - 2) / (z - 1);   // the next shorter segment: 2 sqrt(nz) lengths, not nz
+    s = (int)(((int64_t)nz + z - 2) / (z - 1));   // the next shorter segment: 2 sqrt(nz) lengths, not nz
   }
   return best;
 }
